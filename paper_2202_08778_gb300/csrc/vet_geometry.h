@@ -124,8 +124,7 @@ void build_template(const double *d, int ext, int B, double h, unsigned char *ou
   int off = 0;
   for (int e = 0; e < n; ++e) {
     cpos[ev[e].axis * B + ev[e].m] = (int16_t)e;
-    cev[e].len = R((ev[e].t - prev) * scale);
-    cev[e].off = off * (int)(2 * sizeof(R));  // bytes: one (kappa, S) pair per tile cell
+    set_event(cev[e], (ev[e].t - prev) * scale, off * (int)(2 * sizeof(R)));  // bytes: one (kappa, S) pair per tile cell
     off -= sgn[ev[e].axis] * cstride[ev[e].axis];  // crossing the plane moves one cell upwind
     prev = ev[e].t;
   }
@@ -143,8 +142,7 @@ void build_template(const double *d, int ext, int B, double h, unsigned char *ou
   off = 0;
   for (int e = 0; e < n; ++e) {
     npos[ev[e].axis * (B + 1) + ev[e].m] = (int16_t)e;
-    nev[e].len = R((ev[e].t - prev) * scale);
-    nev[e].off = off * (int)(2 * sizeof(R));
+    set_event(nev[e], (ev[e].t - prev) * scale, off * (int)(2 * sizeof(R)));
     off -= sgn[ev[e].axis] * nstride[ev[e].axis];
     prev = ev[e].t;
   }

@@ -12,6 +12,7 @@
 
 #include "vet.h"
 #include "vet_bridge.h"
+#include "vet_exp64.h"
 #include "vet_geometry.h"
 #include "vet_internal.h"
 
@@ -35,6 +36,7 @@ struct vet_ctx {
   FaceItem *d_items = nullptr;
   int *d_cell_order = nullptr;   // cell-pass visiting order of internal directions
   uint16_t *d_node_order = nullptr;  // paired face pass: face nodes by ray length (dims.node_order)
+  double *d_exp64 = nullptr;     // FP64: tables of the segment weight
   void *d_faces = nullptr;       // [N][blocks][3][fstride], upwind frame, padded
   void *d_emax = nullptr;        // 8 bytes: bit pattern of max E (nonnegative)
   void *d_E = nullptr;           // [cells] E when the caller does not want M
@@ -93,6 +95,7 @@ void free_ctx(vet_ctx *c) {
   cudaFree(c->d_items);
   cudaFree(c->d_cell_order);
   cudaFree(c->d_node_order);
+  cudaFree(c->d_exp64);
   cudaFree(c->d_faces);
   cudaFree(c->d_emax);
   cudaFree(c->d_E);
@@ -311,6 +314,14 @@ vet_status build_context(vet_ctx *c) {
   }
   if ((e = cudaMemcpy(c->d_coef, coef.data(), sizeof(R) * coef.size(), cudaMemcpyHostToDevice)))
     return cuda_err(c, e, "upload coefficients");
+  if (c->fp64) {
+    std::vector<double> tab(vet::kExp64TableDoubles);
+    vet::exp64_fill_table(tab.data());
+    if ((e = cudaMalloc((void **)&c->d_exp64, sizeof(double) * tab.size()))) return cuda_err(c, e, "cudaMalloc(exp table)");
+    if ((e = cudaMemcpy(c->d_exp64, tab.data(), sizeof(double) * tab.size(), cudaMemcpyHostToDevice)))
+      return cuda_err(c, e, "upload exp table");
+    c->dims.exp64 = c->d_exp64;
+  }
   if ((e = vet::prepare_kernels())) return cuda_err(c, e, "cudaFuncSetAttribute");
   return enable_tail_split(c);
 }

@@ -72,6 +72,16 @@ struct alignas(2 * sizeof(R)) TplEvent {
   R len;
   int off;
 };
+// FP64 events carry an FP32 copy of the length beside it, from which the
+// segment weight (vet_exp64.h) picks its table step: 1024 len.
+template <>
+struct alignas(16) TplEvent<double> {
+  double len;
+  int off;
+  float lens;
+};
+inline void set_event(TplEvent<float> &e, double len, int off) { e = {(float)len, off}; }
+inline void set_event(TplEvent<double> &e, double len, int off) { e = {len, off, (float)(1024.0 * len)}; }
 
 // The head and the node-ray parts come first, so that the face pass stages
 // only [0, node_bytes) of a template.
@@ -124,6 +134,7 @@ struct GridDims {
   // three faces merged the same way, [N][6][(B+1)^2] (geom::node_order;
   // null: row order)
   const uint16_t *node_order;
+  const double *exp64;  // FP64 passes: tables of the segment weight (vet_exp64.h)
 };
 
 // Shared-memory kappa/S tiles of a block, in entries of 8 bytes (kappa, S) or,

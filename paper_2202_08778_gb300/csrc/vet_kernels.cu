@@ -20,6 +20,7 @@
 #include <cstddef>
 #include <cstdint>
 
+#include "vet_exp64.h"
 #include "vet_internal.h"
 
 namespace vet {
@@ -46,8 +47,8 @@ template <typename R> using vec2_t = typename Vec2<R>::T;
 //     zero-mean) grows by e^-x / (1 - e^-x) <= 3.5 at x >= 1/4.
 // The FMA pipe bounds the FP32 ray march, so the thin range is set to 1/4,
 // where a cubic suffices (a quartic on x < 1/2 costs one more fused
-// multiply-add per segment: 8% of the cell pass).  FP64: expm1 and exp2 of
-// the CUDA math library in the same two forms, thin for x < 1/2.
+// multiply-add per segment: 8% of the cell pass).  FP64: the same two forms
+// with the weight of vet_exp64.h, thin for x < 1/2.
 constexpr float kQ3 = kThinQ3, kQ2 = kThinQ2, kQ1 = kThinQ1, kQ0 = kThinQ0;  // vet_internal.h
 __device__ __forceinline__ float seg_weight(float y, bool &thin) {
   float e;
@@ -60,35 +61,57 @@ __device__ __forceinline__ float seg_weight(float y, bool &thin) {
   return thin ? q * y : e;
 }
 
-__device__ __forceinline__ double seg_weight(double y, bool &thin) {
-  thin = y > -0.7213475204444817;
-  return thin ? expm1(y * 0.6931471805599453094) : exp2(y);
+// FP64 weight where vet_exp64.h's premise does not hold (vacuum-lit NaN or
+// infinite fields, a depth beyond 690, a negative kappa): the library's
+// functions, out of line.
+__device__ __noinline__ double seg_weight_general(double y) {
+  return y > -0.7213475204444817 ? expm1(y * 0.6931471805599453094) : exp2(y);
 }
 
 // tb: byte address of the ray's start cell in the tile; ev.off is the byte
-// offset of the segment's cell from it.
-template <typename R>
-__device__ __forceinline__ void segment(const unsigned char *__restrict__ tb, const TplEvent<R> &ev, R &I) {
-  const vec2_t<R> ks = *reinterpret_cast<const vec2_t<R> *>(tb + ev.off);
+// offset of the segment's cell from it.  tab: FP64's weight tables.
+__device__ __forceinline__ void segment(const unsigned char *__restrict__ tb, const TplEvent<float> &ev,
+                                        const double *, float &I) {
+  const float2 ks = *reinterpret_cast<const float2 *>(tb + ev.off);
   bool thin;
-  const R w = seg_weight(ks.x * ev.len, thin);
+  const float w = seg_weight(ks.x * ev.len, thin);
+  I = fmaf(I - ks.y, w, thin ? I : ks.y);
+}
+// The FP64 pipe bounds this march (two operations per clock per SM): five
+// operations a segment (r, q and w of the weight, I - S and the update) where
+// expm1 and exp2 took about 44.  64^3 cells in 16^3 blocks, 192 directions,
+// moments wanted: closure 74.0 -> 11.4 ms (cell pass 64.4 -> 10.0, faces 9.5
+// -> 1.40), the FP64 pipe 90% busy before and after.
+__device__ __forceinline__ void segment(const unsigned char *__restrict__ tb, const TplEvent<double> &ev,
+                                        const double *__restrict__ tab, double &I) {
+  const double2 ks = *reinterpret_cast<const double2 *>(tb + ev.off);
+  bool thin;
+  double w;
+  if (!exp64_weight(ks.x, ev.len, ev.lens, tab, w, thin)) {
+    const double y = ks.x * ev.len;
+    thin = y > -0.7213475204444817;
+    w = seg_weight_general(y);
+  }
   I = fma(I - ks.y, w, thin ? I : ks.y);
 }
+
+__device__ __forceinline__ void clear_event(TplEvent<float> &e) { e = {0.f, 0}; }
+__device__ __forceinline__ void clear_event(TplEvent<double> &e) { e = {0.0, 0, 0.f}; }
 
 // Intensity at a ray's start point: entering with I at the upwind end of
 // segment `last`, the segments last, last-1, ..., 0 are crossed downwind.
 // last = -1 (a start point on the upwind face) returns I unchanged.
 template <typename R>
 __device__ __forceinline__ R march(const vec2_t<R> *__restrict__ tile, int idx0, int last,
-                                   const TplEvent<R> *__restrict__ ev, R I) {
+                                   const TplEvent<R> *__restrict__ ev, const double *__restrict__ tab, R I) {
   const unsigned char *tb = reinterpret_cast<const unsigned char *>(tile + idx0);
   int e = last;
   for (; e > 0; e -= 2) {  // two segments per trip
     const TplEvent<R> e0 = ev[e], e1 = ev[e - 1];
-    segment<R>(tb, e0, I);
-    segment<R>(tb, e1, I);
+    segment(tb, e0, tab, I);
+    segment(tb, e1, tab, I);
   }
-  if (e == 0) segment<R>(tb, ev[0], I);
+  if (e == 0) segment(tb, ev[0], tab, I);
   return I;
 }
 
@@ -98,17 +121,17 @@ __device__ __forceinline__ R march(const vec2_t<R> *__restrict__ tile, int idx0,
 // index read is below the template's event capacity (3B).
 template <typename R>
 __device__ __forceinline__ R march_aligned(const vec2_t<R> *__restrict__ tile, int idx0, int last, int wl,
-                                           const TplEvent<R> *__restrict__ ev, R I) {
+                                           const TplEvent<R> *__restrict__ ev, const double *__restrict__ tab, R I) {
   const unsigned char *tb = reinterpret_cast<const unsigned char *>(tile + idx0);
   int e = wl;
   for (; e > 0; e -= 2) {  // two segments per trip
     TplEvent<R> e0 = ev[e], e1 = ev[e - 1];
-    if (e > last) { e0.len = R(0); e0.off = 0; }
-    if (e - 1 > last) { e1.len = R(0); e1.off = 0; }
-    segment<R>(tb, e0, I);
-    segment<R>(tb, e1, I);
+    if (e > last) clear_event(e0);
+    if (e - 1 > last) clear_event(e1);
+    segment(tb, e0, tab, I);
+    segment(tb, e1, tab, I);
   }
-  if (e == 0 && last >= 0) segment<R>(tb, ev[0], I);
+  if (e == 0 && last >= 0) segment(tb, ev[0], tab, I);
   return I;
 }
 
@@ -360,7 +383,7 @@ constexpr int kFaceThreads = 512;
 // dependent launch of the one before); then the (direction, node) rays are
 // spread over the threads.
 template <typename R, int BC>
-__global__ void __launch_bounds__(kFaceThreads, 3)
+__global__ void __launch_bounds__(kFaceThreads, sizeof(R) == 8 ? 2 : 3)
     face_pass_kernel(GridDims g, const R *__restrict__ kappa, const R *__restrict__ S,
                      const unsigned char *__restrict__ tpl_g, const FaceItem *__restrict__ items,
                      R *__restrict__ faces, const R *__restrict__ bnd, long long spin_limit, int *status) {
@@ -464,7 +487,7 @@ __global__ void __launch_bounds__(kFaceThreads, 3)
       const int c1 = T.h->sgn[1] > 0 ? L1 - 1 : B - L1;
       const int c2 = T.h->sgn[2] > 0 ? L2 - 1 : B - L2;
       const int idx0 = last >= 0 ? c0 + ts.sy * c1 + ts.sz * c2 : 0;
-      I = march_aligned<R>(tile, idx0, last, wl, T.nev, I);
+      I = march_aligned<R>(tile, idx0, last, wl, T.nev, g.exp64, I);
     }
     if (act) faces[(((long long)(it.dir_begin + j) * nblk + it.block) * 3 + a) * g.fstride + ub * W + uc] = I;
   }
@@ -479,6 +502,10 @@ __device__ __forceinline__ void atomic_max_nonneg(void *p, double v) {
 }
 
 constexpr int kCellThreads = 512;  // one cell per thread
+// FP64 keeps one CTA per SM's worth of registers (102 instead of 64 with
+// spills: 10.15 -> 10.02 ms at 64^3): five warps fill the FP64 pipe.
+template <typename R>
+constexpr int kCellMinCtas = sizeof(R) == 8 ? 1 : 2;
 
 // Cell pass: one CTA per (block, slab of 512 of the block's cells), one cell
 // per thread.  Directions are visited in tiles of `dt` (octants interleaved)
@@ -488,7 +515,7 @@ constexpr int kCellThreads = 512;  // one cell per thread
 // tile they start.  For block edges that are multiples of 4, each warp holds a
 // 4 x 4 x 2 brick of cells, whose rays have similar lengths.
 template <typename R, int MODE, int BC>
-__global__ void __launch_bounds__(kCellThreads, 2)
+__global__ void __launch_bounds__(kCellThreads, kCellMinCtas<R>)
     cell_pass_kernel(GridDims g, int parts, int dt, const R *__restrict__ kappa, const R *__restrict__ S,
                      const unsigned char *__restrict__ tpl_g, const int *__restrict__ order,
                      const R *__restrict__ faces, const R *__restrict__ bnd, R *__restrict__ I_out,
@@ -585,7 +612,7 @@ __global__ void __launch_bounds__(kCellThreads, 2)
         if (p2 < last) { last = p2; ae = 2; la = l2; lb = l0; lc = l1; }
         const int row = (ae * 2) * B + la;
         const R Iin = face_value<R>(fin, fstride, B, ae, lb, lc, T.ck[row], T.ck[row + B], T.cw[row], T.cw[row + B]);
-        const R I = march<R>(tile, tc, last, T.cev, Iin);
+        const R I = march<R>(tile, tc, last, T.cev, g.exp64, Iin);
         if (MODE == 1) {
           I_out[(long long)T.h->ext * g.ncell + gc] = I;
         } else {
