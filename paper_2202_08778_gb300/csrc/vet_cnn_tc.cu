@@ -1,27 +1,32 @@
 // vet_cnn_tc.cu -- the learned closure's 3x3x3 convolutions on the 5th
 // generation tensor cores (tcgen05, accumulators in tensor memory).
 //
-// Implicit GEMM per output tile of 8 x 16 x 2 cells (x, y, z): for each of
-// the 27 taps and each 16-channel step of the input, one
-// tcgen05.mma.kind::f16 (BF16 x BF16 -> FP32) per z-slice with M = 128 cells
-// (8 x 16, one z), N = C_out, K = 16.  Both operands sit in shared memory in
-// the canonical K-major layout without swizzle: "core matrices" of 8 rows x
-// 16 bytes stored contiguously, addressed by a descriptor (start, leading
-// byte offset LBO between core matrices along K, stride byte offset SBO
-// between 8-row groups along M or N).
-//   A (activations): the tile's 10 x 18 x 4 input halo stored as
-//     [16-byte channel chunk][halo cell][16 B], so that 8 cells consecutive
-//     in x form one core matrix at every tap shift: start = the tap's first
-//     halo cell, LBO = one chunk plane (720 x 16 B), SBO = one halo row in y
-//     (10 x 16 B).
-//   B (weights): [tap][channel chunk][C_out][16 B], LBO = C_out x 16 B,
-//     SBO = 8 x 16 B.
-// One thread issues the 54 (C_in = 32) or 27 (C_in = 16) x 2 MMAs of a tile
-// and commits them to an mbarrier; the other warps wait (bounded) and then
-// read the accumulators back with tcgen05.ld (warp w reads tensor-memory
-// lanes 32 (w % 4).. of z-slice w / 4), apply the epilogue and store.
-// Tensor memory (2 x C_out columns) is allocated once per CTA and released
-// before the CTA exits, also when a wait gave up.
+// Implicit GEMM over columns of 8 x 16 cells (x, y) marched along z.  Each
+// input slice of a column (with its halo, 10 x 18 cells) is staged once and
+// serves the three output slices it touches in one go: their accumulators are
+// neighbouring column blocks of tensor memory and the weights of the three dz
+// taps are stacked along N, so that one tcgen05.mma.kind::f16 (BF16 x BF16 ->
+// FP32) per (dy, dx) tap and 16-channel step has M = 128 cells, N = 3 C_out,
+// K = 16.  Why: an M = 128, K = 16 MMA reads 4 KB of A from shared memory
+// and takes about 46 clocks whatever N up to 64, so one MMA per tap and output
+// slice (N = 32) reached 0.35 of the tensor rate; stacking issues a third of
+// the MMAs for the same products.  Every output still adds its taps in the
+// order dz, dy, dx, channel step: results are the same bits.
+// Both operands sit in shared memory in the canonical K-major layout without
+// swizzle: "core matrices" of 8 rows x 16 bytes stored contiguously, addressed
+// by a descriptor (start, leading byte offset LBO between core matrices along
+// K, stride byte offset SBO between 8-row groups along M or N).
+//   A (activations): a slice's halo as [16-byte channel chunk][halo cell][16 B],
+//     so that 8 cells consecutive in x form one core matrix at every tap
+//     shift: start = the tap's first halo cell, LBO = one chunk plane
+//     (180 x 16 B), SBO = one halo row in y (10 x 16 B).
+//   B (weights): [dy, dx][channel chunk][dz = +1, 0, -1][C_out][16 B],
+//     LBO = 3 C_out x 16 B, SBO = 8 x 16 B.
+// Tensor memory: a ring of 512 / C_out output slices (all 512 columns, one
+// CTA per SM), each zeroed by the epilogue that read it; a window of three
+// slices that wraps around the ring's end is issued as two sets of MMAs.
+// 128^3, ncu: 32 -> 32 channels 261 -> 95 us, 16 -> 32 150 -> 83 us, 32 -> 16
+// 248 -> 92 us; the network on one 128^3 grid 1144 -> 594 us.
 #include <cstdint>
 
 #include <cuda_bf16.h>
@@ -32,9 +37,11 @@ namespace vet {
 namespace cnn {
 namespace {
 
-constexpr int TX = 8, TY = 16, TZ = 2;     // output tile (x, y, z)
-constexpr int HX = 10, HY = 18, HZ = 4;    // input halo
-constexpr int HN = HX * HY * HZ;           // 720 halo cells
+constexpr int TX = 8, TY = 16;             // output tile of a slice (x, y)
+constexpr int HX = 10, HY = 18;            // input halo of a slice
+constexpr int HN = HX * HY;                // 180 halo cells
+constexpr int kRing = 6;                   // staged input slices (even: two loader groups take turns)
+constexpr uint32_t kTmemCols = 512;
 constexpr long long kWaitPolls = 1LL << 24;
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -63,16 +70,26 @@ __host__ __device__ constexpr uint32_t idesc_bf16(int M, int N) {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 
-__device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
+// D += A B; the descriptors as (low, high) words.
+__device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo, uint32_t b_hi,
+                                         uint32_t idesc) {
   asm volatile(
-      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-      " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d_tmem),
-      "l"(a), "l"(b), "r"(idesc), "r"(acc));
+      "{\n .reg .pred p;\n .reg .b64 a, b;\n setp.ne.b32 p, 1, 0;\n mov.b64 a, {%1, %2};\n mov.b64 b, {%3, %4};\n"
+      " tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %5, p;\n}\n" ::"r"(d_tmem),
+      "r"(a_lo), "r"(a_hi), "r"(b_lo), "r"(b_hi), "r"(idesc));
 }
 
-__device__ __forceinline__ void mma_commit(uint64_t *bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
-               : "memory");
+// One lane of a converged warp.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t r;
+  asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(r));
+  return r != 0;
+}
+// A value that is the same on every lane, known as such to the compiler.
+__device__ __forceinline__ uint32_t uniform(uint32_t v) { return __shfl_sync(0xffffffffu, v, 0); }
+
+__device__ __forceinline__ void mma_commit(uint32_t bar) {
+  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
 }
 
 __device__ __forceinline__ void mbar_init(uint64_t *bar, uint32_t count) {
@@ -95,29 +112,15 @@ __device__ __forceinline__ void fence_after_sync() { asm volatile("tcgen05.fence
 __device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void *src, uint32_t src_bytes) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(src_bytes) : "memory");
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(src_bytes) : "memory");
 }
 
-// 32 (or 16) consecutive FP32 columns of this thread's tensor-memory lane.
+// 16 (or 8) consecutive FP32 columns of this thread's tensor-memory lane,
+// which are then set to zero for the next output slice that takes them.
 template <int N>
-__device__ __forceinline__ void tmem_ld(uint32_t taddr, float (&v)[N]);
+__device__ __forceinline__ void tmem_take(uint32_t taddr, float (&v)[N]);
 template <>
-__device__ __forceinline__ void tmem_ld<32>(uint32_t taddr, float (&v)[32]) {
-  uint32_t r[32];
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
-      "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]),
-        "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
-        "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-      : "r"(taddr));
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-  for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
-}
-template <>
-__device__ __forceinline__ void tmem_ld<16>(uint32_t taddr, float (&v)[16]) {
+__device__ __forceinline__ void tmem_take<16>(uint32_t taddr, float (&v)[16]) {
   uint32_t r[16];
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
@@ -125,192 +128,298 @@ __device__ __forceinline__ void tmem_ld<16>(uint32_t taddr, float (&v)[16]) {
         "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
       : "r"(taddr));
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1};" ::"r"(taddr),
+               "r"(0u)
+               : "memory");
 #pragma unroll
   for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
+template <>
+__device__ __forceinline__ void tmem_take<8>(uint32_t taddr, float (&v)[8]) {
+  uint32_t r[8];
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+               : "r"(taddr));
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%1,%1,%1,%1,%1,%1,%1};" ::"r"(taddr), "r"(0u) : "memory");
+#pragma unroll
+  for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[i]);
+}
 
-struct Tile {
-  int v, tz, ty, tx;
+// A run of n output slices za .. za + n - 1 of one column.
+struct Run {
+  int v, ty, tx, za, n;
 };
 
-__device__ __forceinline__ Tile tile_of(long long t, const Vol &V) {
-  const int ntx = (V.nx + TX - 1) / TX, nty = (V.ny + TY - 1) / TY, ntz = (V.nz + TZ - 1) / TZ;
-  Tile r;
-  r.tx = (int)(t % ntx);
-  t /= ntx;
-  r.ty = (int)(t % nty);
-  t /= nty;
-  r.tz = (int)(t % ntz);
-  r.v = (int)(t / ntz);
-  return r;
-}
-
-// Columns of tensor memory: 2 accumulator sets x 2 z-slices x C_OUT, a
-// power of two >= 32 as tcgen05.alloc requires.
-template <int C_OUT>
-__host__ __device__ constexpr uint32_t tmem_cols() {
-  return 4 * C_OUT <= 32 ? 32 : (4 * C_OUT <= 64 ? 64 : 128);
-}
+// A CTA's share of the work: output slices [t, end) of the launch, numbered
+// column by column with z fastest, cut into runs at the column ends.  Run r of
+// n slices takes n + 2 steps, one per input slice za - 1 .. za + n (those
+// outside the volume are steps without a load or an MMA).
+struct Cursor {
+  long long t, end;
+  int step;
+  Run run;
+  __device__ __forceinline__ void load(const Vol &V) {
+    if (t >= end) return;
+    const int ntx = (V.nx + TX - 1) / TX, nty = (V.ny + TY - 1) / TY;
+    long long col = t / V.nz;
+    run.za = (int)(t - col * V.nz);
+    run.n = (int)min((long long)(V.nz - run.za), end - t);
+    run.tx = (int)(col % ntx);
+    col /= ntx;
+    run.ty = (int)(col % nty);
+    run.v = (int)(col / nty);
+  }
+  __device__ __forceinline__ Cursor(long long t0, long long t1, const Vol &V) : t(t0), end(t1), step(0), run{0, 0, 0, 0, 0} {
+    load(V);
+  }
+  __device__ __forceinline__ bool live() const { return t < end; }
+  __device__ __forceinline__ int z_in() const { return run.za - 1 + step; }
+  // true when the next step starts another run
+  __device__ __forceinline__ bool advance(const Vol &V) {
+    if (++step < run.n + 2) return false;
+    t += run.n;
+    step = 0;
+    load(V);
+    return true;
+  }
+};
 
 template <int C_IN>
-__host__ __device__ constexpr size_t halo_bytes() {
+__host__ __device__ constexpr size_t slice_bytes() {
   return (size_t)C_IN / 8 * HN * 16;
 }
 
-// Halo of tile ti into one buffer (cp.async, zero outside the volume), by
-// the `nthreads` threads 0 .. nthreads - 1 of the CTA.
-template <int C_IN>
-__device__ __forceinline__ void load_halo(uint32_t dst, const __nv_bfloat16 *__restrict__ x, const Vol &V,
-                                          const Tile &ti, int nthreads) {
-  constexpr int NCI = C_IN / 8;
-  const long long vol = (long long)V.nz * V.ny * V.nx;
-  for (int h = threadIdx.x; h < HN * NCI; h += nthreads) {
-    const int hc = h / NCI, c = h - hc * NCI;
-    const int hz = hc / (HX * HY), hy = (hc / HX) % HY, hx = hc % HX;
-    const int z = ti.tz * TZ + hz - 1, y = ti.ty * TY + hy - 1, xx = ti.tx * TX + hx - 1;
-    const bool in = z >= 0 && z < V.nz && y >= 0 && y < V.ny && xx >= 0 && xx < V.nx;
-    const long long cell = in ? (long long)ti.v * vol + ((long long)z * V.ny + y) * V.nx + xx : 0;
-    cp_async16(dst + (uint32_t)((c * HN + hc) * 16), x + cell * C_IN + c * 8, in ? 16u : 0u);
-  }
-  asm volatile("cp.async.commit_group;" ::: "memory");
-}
+// warp 0 issues the MMAs, warp 1 prepares them
+constexpr int kFirstLoader = 64;
+constexpr int kLoaders = 128;             // warps 2-5, 6-9: halo loads of the even and odd steps
+constexpr int kFirstEpi = kFirstLoader + 2 * kLoaders;
+constexpr int kEpiGroup = 256;            // warps 10-17, 18-25: epilogue of the even and odd output slices
+constexpr int kTcThreads = kFirstEpi + 2 * kEpiGroup;
+constexpr int kLoadLag = 1;               // steps of its own that a loader group waits behind its loads
 
-// The 27 x (C_IN / 16) x 2 MMAs of one tile (one thread).  Descriptor start
-// addresses are 16-byte units in their low 14 bits, so moving an operand by
-// b bytes adds b / 16 to the descriptor (no carry: shared memory < 256 KB).
-template <int C_IN, int C_OUT>
-__device__ __forceinline__ void issue_tile(uint32_t tmem_acc, uint64_t a0, uint64_t b0) {
+// Halo loads of one thread (cp.async, zero outside the volume): its up to
+// six 16-byte pieces sit at the same place in every slice of a column, so
+// the offsets are computed once per run.
+template <int C_IN>
+struct HaloLoader {
+  static constexpr int NCI = C_IN / 8, K = (HN * NCI + kLoaders - 1) / kLoaders;
+  long long off[K];  // elements from the slice's first cell; negative: outside
+  const __nv_bfloat16 *base;
+  long long plane;
+  __device__ __forceinline__ void set(const __nv_bfloat16 *__restrict__ x, const Vol &V, const Run &r) {
+    plane = (long long)V.ny * V.nx * C_IN;
+    base = x + (long long)r.v * V.nz * plane;
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+      const int h = ((int)threadIdx.x - kFirstLoader) % kLoaders + k * kLoaders, c = h / HN, hc = h - c * HN;
+      const int y = r.ty * TY + hc / HX - 1, xx = r.tx * TX + hc % HX - 1;
+      off[k] = y >= 0 && y < V.ny && xx >= 0 && xx < V.nx ? ((long long)y * V.nx + xx) * C_IN + c * 8 : -1;
+    }
+  }
+  __device__ __forceinline__ void load(uint32_t dst, const __nv_bfloat16 *__restrict__ x, int z) const {
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+      const int h = ((int)threadIdx.x - kFirstLoader) % kLoaders + k * kLoaders, c = h / HN, hc = h - c * HN;
+      if (h < HN * NCI)
+        cp_async16(dst + (uint32_t)((c * HN + hc) * 16), off[k] >= 0 ? base + z * plane + off[k] : x, off[k] >= 0 ? 16u : 0u);
+    }
+  }
+};
+
+// What the issuing warp does next: the MMAs of one input slice into a window
+// of neighbouring output slices (idesc 0: none), then the commits.
+struct alignas(16) MmaCommand {
+  uint32_t d, a, b, idesc;     // accumulator; low words of the descriptors; 0xffffffff: the end
+  uint32_t done, ready, pad0, pad1;  // shared addresses of the barriers to commit to (0: none)
+};
+
+// Named-barrier hand-over between the preparing and the issuing warp.
+__device__ __forceinline__ void pair_sync(int id) { asm volatile("barrier.cta.sync %0, 64;" ::"r"(id) : "memory"); }
+__device__ __forceinline__ void pair_arrive(int id) { asm volatile("barrier.cta.arrive %0, 64;" ::"r"(id) : "memory"); }
+constexpr int kBarLoad = 1, kBarEpi = 3, kBarReady = 5, kBarFree = 7;  // named barriers, two of each
+
+// The 9 x (C_IN / 16) MMAs of a command, issued by one lane of a converged
+// warp.  Descriptor start addresses are 16-byte units in their low 14 bits,
+// so moving an operand by b bytes adds b / 16 to the descriptor's low word (no
+// carry: shared memory < 256 KB).  The instruction takes its operands from
+// uniform registers: the bases are made uniform once and every tap is a
+// constant away (a base kept in ordinary registers is moved over for each
+// MMA: 94 clocks between MMAs, not 56).  `midway` runs between two halves of
+// the MMAs, while the tensor pipe has work queued.
+template <int C_IN, int C_OUT, typename F>
+__device__ __forceinline__ void issue_slice(const MmaCommand &c, uint32_t a_hi, uint32_t b_hi, F midway) {
   constexpr int NCI = C_IN / 8;
-  constexpr uint32_t IDESC = idesc_bf16(128, C_OUT);
+  const uint32_t idesc = uniform(c.idesc), d = uniform(c.d), al = uniform(c.a), bl = uniform(c.b);
 #pragma unroll
-  for (int tap = 0; tap < 27; ++tap) {
-    const int dz = tap / 9 - 1, dy = (tap / 3) % 3 - 1, dx = tap % 3 - 1;
+  for (int half = 0; half < 2; ++half) {
+    if (idesc && elect_one()) {
 #pragma unroll
-    for (int ks = 0; ks < NCI / 2; ++ks) {
-      const uint64_t bd = b0 + (uint64_t)((tap * NCI + 2 * ks) * C_OUT);
+      for (int tap = half ? 5 : 0; tap < (half ? 9 : 5); ++tap) {
 #pragma unroll
-      for (int z = 0; z < TZ; ++z) {
-        const int h0 = (z + dz + 1) * (HX * HY) + (dy + 1) * HX + (dx + 1);
-        mma_bf16(tmem_acc + z * C_OUT, a0 + (uint64_t)(2 * ks * HN + h0), bd, IDESC, (tap | ks) ? 1u : 0u);
+        for (int ks = 0; ks < NCI / 2; ++ks)
+          mma_bf16(d, al + (uint32_t)(2 * ks * HN + (tap / 3) * HX + tap % 3), a_hi,
+                   bl + (uint32_t)((tap * NCI + 2 * ks) * 3 * C_OUT), b_hi, idesc);
       }
     }
+    __syncwarp();
+    if (half == 0) midway();
   }
 }
 
+// One thread's part of the output slices of a run: cell r of the 128,
+// channels [c0, c0 + C_OUT / 2).
 template <int C_OUT, int EPI>
-__device__ __forceinline__ void epilogue(uint32_t taddr, const Tile &ti, const Vol &V, const float *__restrict__ sBias,
-                                         __nv_bfloat16 *__restrict__ pre_out, const __nv_bfloat16 *__restrict__ pre_in,
-                                         void *__restrict__ out, int r, int zs) {
-  float acc[C_OUT];
-  tmem_ld<C_OUT>(taddr, acc);
-  const long long vol = (long long)V.nz * V.ny * V.nx;
-  const int xx = ti.tx * TX + (r & 7), y = ti.ty * TY + (r >> 3), z = ti.tz * TZ + zs;
-  if (xx >= V.nx || y >= V.ny || z >= V.nz) return;
-  const long long cell = (long long)ti.v * vol + ((long long)z * V.ny + y) * V.nx + xx;
-  if (EPI == EPI_F32) {
-    float4 *dst = reinterpret_cast<float4 *>(reinterpret_cast<float *>(out) + cell * C_OUT);
-#pragma unroll
-    for (int i = 0; i < C_OUT / 4; ++i)
-      dst[i] = make_float4(acc[4 * i] + sBias[4 * i], acc[4 * i + 1] + sBias[4 * i + 1],
-                           acc[4 * i + 2] + sBias[4 * i + 2], acc[4 * i + 3] + sBias[4 * i + 3]);
-    return;
+struct Epilogue {
+  static constexpr int NC = C_OUT / 2;
+  long long at, plane;  // element of this thread's first channel in the run's slice 0, and per slice
+  bool in;
+  float bias[EPI == EPI_SILU_BWD ? 1 : NC];
+  int4 p[EPI == EPI_SILU_BWD ? NC / 8 : 1];
+  __device__ __forceinline__ void set(const Vol &V, const Run &run, int r, int c0) {
+    const int xx = run.tx * TX + (r & 7), y = run.ty * TY + (r >> 3);
+    in = xx < V.nx && y < V.ny;
+    plane = (long long)V.ny * V.nx * C_OUT;
+    at = ((((long long)run.v * V.nz + run.za) * V.ny + y) * V.nx + xx) * C_OUT + c0;
   }
-  __align__(16) __nv_bfloat162 o2[C_OUT / 2];
-  __align__(16) __nv_bfloat162 p2[C_OUT / 2];
-  if (EPI == EPI_SILU) {
+  // the pre-activations the backward epilogue needs, ahead of the wait
+  __device__ __forceinline__ void prefetch(const __nv_bfloat16 *__restrict__ pre_in, int j) {
+    if constexpr (EPI == EPI_SILU_BWD) {
+      if (!in) return;
 #pragma unroll
-    for (int i = 0; i < C_OUT / 2; ++i) {
-      const float z0 = acc[2 * i] + sBias[2 * i], z1 = acc[2 * i + 1] + sBias[2 * i + 1];
-      p2[i] = __floats2bfloat162_rn(z0, z1);
-      o2[i] = __floats2bfloat162_rn(silu(z0), silu(z1));
+      for (int i = 0; i < NC / 8; ++i) p[i] = reinterpret_cast<const int4 *>(pre_in + at + j * plane)[i];
     }
-    if (pre_out) {
-      int4 *pd = reinterpret_cast<int4 *>(pre_out + cell * C_OUT);
-#pragma unroll
-      for (int i = 0; i < C_OUT / 8; ++i) pd[i] = reinterpret_cast<const int4 *>(p2)[i];
-    }
-  } else {  // EPI_SILU_BWD
-    const int4 *ps = reinterpret_cast<const int4 *>(pre_in + cell * C_OUT);
-#pragma unroll
-    for (int i = 0; i < C_OUT / 8; ++i) reinterpret_cast<int4 *>(p2)[i] = ps[i];
-#pragma unroll
-    for (int i = 0; i < C_OUT / 2; ++i)
-      o2[i] = __floats2bfloat162_rn(acc[2 * i] * silu_grad(__bfloat162float(p2[i].x)),
-                                    acc[2 * i + 1] * silu_grad(__bfloat162float(p2[i].y)));
   }
-  int4 *od = reinterpret_cast<int4 *>(reinterpret_cast<__nv_bfloat16 *>(out) + cell * C_OUT);
+  __device__ __forceinline__ void store(const float (&acc)[NC], __nv_bfloat16 *__restrict__ pre_out,
+                                        void *__restrict__ out, int j) {
+    if (!in) return;
+    const long long e = at + j * plane;
+    if constexpr (EPI == EPI_F32) {
+      float4 *dst = reinterpret_cast<float4 *>(reinterpret_cast<float *>(out) + e);
 #pragma unroll
-  for (int i = 0; i < C_OUT / 8; ++i) od[i] = reinterpret_cast<const int4 *>(o2)[i];
-}
+      for (int i = 0; i < NC / 4; ++i)
+        dst[i] = make_float4(acc[4 * i] + bias[4 * i], acc[4 * i + 1] + bias[4 * i + 1], acc[4 * i + 2] + bias[4 * i + 2],
+                             acc[4 * i + 3] + bias[4 * i + 3]);
+    } else {
+      __align__(16) __nv_bfloat162 o2[NC / 2];
+      if constexpr (EPI == EPI_SILU) {
+        __align__(16) __nv_bfloat162 p2[NC / 2];
+#pragma unroll
+        for (int i = 0; i < NC / 2; ++i) {
+          const float z0 = acc[2 * i] + bias[2 * i], z1 = acc[2 * i + 1] + bias[2 * i + 1];
+          p2[i] = __floats2bfloat162_rn(z0, z1);
+          o2[i] = __floats2bfloat162_rn(silu(z0), silu(z1));
+        }
+        if (pre_out) {
+          int4 *pd = reinterpret_cast<int4 *>(pre_out + e);
+#pragma unroll
+          for (int i = 0; i < NC / 8; ++i) pd[i] = reinterpret_cast<const int4 *>(p2)[i];
+        }
+      } else {  // EPI_SILU_BWD
+        const __nv_bfloat162 *p2 = reinterpret_cast<const __nv_bfloat162 *>(p);
+#pragma unroll
+        for (int i = 0; i < NC / 2; ++i)
+          o2[i] = __floats2bfloat162_rn(acc[2 * i] * silu_grad(__bfloat162float(p2[i].x)),
+                                        acc[2 * i + 1] * silu_grad(__bfloat162float(p2[i].y)));
+      }
+      int4 *od = reinterpret_cast<int4 *>(reinterpret_cast<__nv_bfloat16 *>(out) + e);
+#pragma unroll
+      for (int i = 0; i < NC / 8; ++i) od[i] = reinterpret_cast<const int4 *>(o2)[i];
+    }
+  }
+};
 
-// Bounded wait on an mbarrier phase by a whole warp, giving up early when
+// Bounded wait of one thread on an mbarrier phase, giving up early when
 // another role has aborted (*abort set).
 __device__ __forceinline__ bool wait_or_abort(uint64_t *bar, uint32_t parity, volatile int *abort) {
-  bool done = false;
   for (long long i = 0; i < kWaitPolls; ++i) {
-    if (!done) done = mbar_try(bar, parity);
-    if (__all_sync(0xffffffffu, done)) return true;
-    if ((i & 1023) == 1023 && __any_sync(0xffffffffu, *abort != 0)) return false;
+    if (mbar_try(bar, parity)) return true;
+    if ((i & 1023) == 1023 && *abort != 0) return false;
   }
   return false;
+}
+
+// Named barrier over nthreads threads (whole warps) that also tells each
+// whether ok held for all of them: no shared-memory access.
+__device__ __forceinline__ bool group_all(int id, int nthreads, bool ok) {
+  uint32_t r;
+  asm volatile(
+      "{\n .reg .pred p, q;\n setp.ne.u32 p, %1, 0;\n barrier.cta.red.and.pred q, %2, %3, p;\n selp.u32 %0, 1, 0, q;\n}\n"
+      : "=r"(r)
+      : "r"((uint32_t)ok), "r"(id), "r"(nthreads)
+      : "memory");
+  return r != 0;
 }
 
 __device__ __forceinline__ void mbar_arrive(uint64_t *bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
 
-constexpr int kWorkers = 256;             // warps 0-7: halo loads and epilogue
-constexpr int kTcThreads = kWorkers + 32; // warp 8: issues the MMAs
-
-// Warp-specialised pipeline.  Tile i of this CTA uses halo buffer and
-// accumulator set s = i % 2.
-//   MMA warp (one lane): wait full[s] (halo of tile i landed) and, from
-//     i >= 2, empty[s] (tile i - 2's accumulators read); issue tile i's MMAs;
-//     commit them to done[s].
-//   Workers: wait done[s] (tile i's MMAs finished: buffer s is free, its
-//     accumulators ready); start the cp.async loads of tile i + 2 into buffer
-//     s; read and store tile i's outputs; arrive on empty[s]; complete the
-//     loads, fence them to the async proxy and arrive on full[s].
-// The tensor cores run tile i + 1 while the workers drain tile i and load
-// tile i + 2.  Every wait is bounded; a role that gives up sets `abort`,
-// which ends the other role's waits too.
+// Warp-specialised pipeline over the steps of this CTA's share (all roles walk
+// the same steps; step g uses ring buffer g % kRing, output o of the share,
+// counted over its runs, tensor-memory block o % (512 / C_OUT)).
+//   Loader groups, step g (even and odd ones): wait done[g - kRing] (the
+//     buffer is free); start the slice's loads; the loads of the group's step
+//     before have landed by then: fence them to the async proxy and arrive on
+//     full.
+//   MMA preparation, step g: wait full[g % kRing] and empty[block] of the
+//     output that joins, work out the window, hand a command to
+//   MMA issuer: issue the slice's MMAs; commit them to done[g % kRing] and to
+//     ready[block] of the output slice they complete.  Two warps, since the
+//     waits and the bookkeeping of a step (about 700 clocks on one warp) are
+//     more than the MMAs queued meanwhile (six, 340 clocks) hide.
+//   Epilogue groups, output o (even and odd ones): wait ready[block]; read,
+//     zero and store it (warp w: tensor-memory lanes 32 (w % 4) ..,
+//     channels of half w / 4); arrive on empty[block].
+// The MMAs read their operands at the full 128 bytes per clock of shared
+// memory (56 clocks for N = 96: 4 KB of A, 3 KB of B), so every other access
+// to it takes their time: one thread of a role polls a barrier and hands the
+// verdict to the others by a named barrier, and a warp arrives once.
+// What bounds a step (95 us: about 1640 clocks, of which the MMAs take 1225 with
+// their commits and windows cut in two): the hand-overs between the roles.
+// Every wait is bounded; a role that gives up sets `abort`, which ends the
+// other roles' waits too.
 template <int C_IN, int C_OUT, int EPI>
 __global__ void __launch_bounds__(kTcThreads, 1)
     conv3d_tc_kernel(const __nv_bfloat16 *__restrict__ x, const __nv_bfloat16 *__restrict__ W,
                      const float *__restrict__ b, Vol V, __nv_bfloat16 *__restrict__ pre_out,
                      const __nv_bfloat16 *__restrict__ pre_in, void *__restrict__ out, int *status) {
-  constexpr int NCI = C_IN / 8;
+  constexpr int NCI = C_IN / 8, NC = C_OUT / 2;
+  constexpr int kSlots = (int)kTmemCols / C_OUT;
   constexpr uint32_t A_LBO = HN * 16, A_SBO = HX * 16;
-  constexpr uint32_t B_LBO = C_OUT * 16, B_SBO = 8 * 16;
-  constexpr uint32_t TCOLS = tmem_cols<C_OUT>();
+  constexpr uint32_t B_LBO = 3 * C_OUT * 16, B_SBO = 8 * 16;
   extern __shared__ __align__(128) unsigned char smem[];
-  unsigned char *sA = smem;                                   // 2 x [NCI][HN][16 B]
-  unsigned char *sB = smem + 2 * halo_bytes<C_IN>();          // [27][NCI][C_OUT][16 B]
-  __shared__ __align__(8) uint64_t full[2], done[2], empty[2];
+  unsigned char *sA = smem;                                   // kRing x [NCI][HN][16 B]
+  unsigned char *sB = smem + kRing * slice_bytes<C_IN>();     // [9][NCI][3][C_OUT][16 B]
+  __shared__ __align__(8) uint64_t full[kRing], done[kRing], ready[kSlots], empty[kSlots];
+  __shared__ MmaCommand commands[2];
   __shared__ uint32_t tmem_base_slot;
   __shared__ volatile int abort_flag;
-  __shared__ int n_committed[2];  // MMA batches committed per accumulator set
-  __shared__ float sBias[C_OUT];
+  __shared__ int n_committed, n_next[2];  // steps whose MMAs were committed; first even and odd step the loaders did not see complete
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   for (int h = threadIdx.x; h < 27 * C_OUT * NCI; h += blockDim.x) {
     const int c = h % NCI, co = (h / NCI) % C_OUT, tap = h / (NCI * C_OUT);
     const int4 val = reinterpret_cast<const int4 *>(W + ((size_t)tap * C_OUT + co) * C_IN)[c];
-    *reinterpret_cast<int4 *>(sB + (((size_t)tap * NCI + c) * C_OUT + co) * 16) = val;
+    const int yx = tap % 9, k = 2 - tap / 9;
+    *reinterpret_cast<int4 *>(sB + ((((size_t)yx * NCI + c) * 3 + k) * C_OUT + co) * 16) = val;
   }
-  if (threadIdx.x < C_OUT) sBias[threadIdx.x] = b ? b[threadIdx.x] : 0.f;
   if (threadIdx.x == 0) {
-    for (int k = 0; k < 2; ++k) {
-      mbar_init(&full[k], kWorkers);
+    for (int k = 0; k < kRing; ++k) {
+      mbar_init(&full[k], kLoaders / 32);
       mbar_init(&done[k], 1);
-      mbar_init(&empty[k], kWorkers);
-      n_committed[k] = 0;
+    }
+    for (int k = 0; k < kSlots; ++k) {
+      mbar_init(&ready[k], 1);
+      mbar_init(&empty[k], kEpiGroup / 32);
     }
     abort_flag = 0;
+    n_committed = n_next[0] = 0;
+    n_next[1] = 1;
   }
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_slot)),
-                 "r"(TCOLS)
+                 "r"(kTmemCols)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
@@ -319,74 +428,178 @@ __global__ void __launch_bounds__(kTcThreads, 1)
   __syncthreads();
   fence_after_sync();
   const uint32_t tmem = tmem_base_slot;
-  const long long nt = (long long)V.n * ((V.nz + TZ - 1) / TZ) * ((V.ny + TY - 1) / TY) * ((V.nx + TX - 1) / TX);
-  const int ntile = blockIdx.x < nt ? (int)((nt - 1 - blockIdx.x) / gridDim.x + 1) : 0;  // tiles of this CTA
+  const long long nt = (long long)V.n * ((V.ny + TY - 1) / TY) * ((V.nx + TX - 1) / TX) * V.nz;
+  const long long t0 = nt * blockIdx.x / gridDim.x, t1 = nt * (blockIdx.x + 1) / gridDim.x;
   const uint32_t a_base = smem_u32(sA), b_base = smem_u32(sB);
+  auto wait = [&](uint64_t *bar, uint32_t parity) {  // one thread
+    if (wait_or_abort(bar, parity, &abort_flag)) return true;
+    atomicOr(status, 16);
+    abort_flag = 1;
+    return false;
+  };
+  auto wait_warp = [&](uint64_t *bar, uint32_t parity) {  // every lane of a warp, one verdict
+    return __all_sync(0xffffffffu, wait(bar, parity));
+  };
+  // the accumulators start at zero: each epilogue warp its lanes' quarter of the columns
+  if (warp >= kFirstEpi / 32) {
+    const int w = warp - kFirstEpi / 32;
+    const uint32_t t = tmem + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)((w >> 2) * ((int)kTmemCols / 4));
+    for (int k = 0; k < (int)kTmemCols / 4; k += 16)
+      asm volatile("tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1};" ::"r"(
+                       t + (uint32_t)k),
+                   "r"(0u)
+                   : "memory");
+    asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+  }
+  fence_before_sync();
+  __syncthreads();
+  fence_after_sync();
 
-  if (warp == kWorkers / 32) {
-    // ---- MMA issuer
-    const uint64_t a_desc0 = smem_desc(a_base, A_LBO, A_SBO);
-    const uint64_t a_desc1 = smem_desc(a_base + (uint32_t)halo_bytes<C_IN>(), A_LBO, A_SBO);
-    const uint64_t b_desc = smem_desc(b_base, B_LBO, B_SBO);
-    for (int i = 0; i < ntile; ++i) {
-      const int s = i & 1;
-      const uint32_t use = (uint32_t)(i >> 1);  // this is use number `use` of buffer / accumulator set s
-      bool ok = wait_or_abort(&full[s], use & 1u, &abort_flag);
-      if (ok && i >= 2) ok = wait_or_abort(&empty[s], (use - 1) & 1u, &abort_flag);
-      if (!ok) {
-        if (lane == 0) {
-          atomicOr(status, 16);
-          abort_flag = 1;
-        }
-        break;
-      }
+  if (warp == 0) {
+    // ---- MMA issuer: the next command is fetched halfway through the current one
+    const uint32_t a_hi = uniform((uint32_t)(smem_desc(a_base, A_LBO, A_SBO) >> 32));
+    const uint32_t b_hi = uniform((uint32_t)(smem_desc(b_base, B_LBO, B_SBO) >> 32));
+    MmaCommand cur, nxt;
+    int k = 0;
+    auto fetch = [&]() {
+      pair_sync(kBarReady + (k & 1));
+      nxt = commands[k & 1];
+      pair_arrive(kBarFree + (k & 1));
+      ++k;
+    };
+    fetch();
+    while (nxt.d != 0xffffffffu) {
+      cur = nxt;
       fence_after_sync();
-      if (lane == 0) {
-        issue_tile<C_IN, C_OUT>(tmem + (uint32_t)(s * 2 * C_OUT), s ? a_desc1 : a_desc0, b_desc);
-        mma_commit(&done[s]);
-        ++n_committed[s];
+      issue_slice<C_IN, C_OUT>(cur, a_hi, b_hi, fetch);
+      if (elect_one()) {
+        if (cur.done) mma_commit(cur.done);
+        if (cur.ready) mma_commit(cur.ready);
       }
       __syncwarp();
     }
-  }
-  int n_waited0 = 0, n_waited1 = 0;  // batches this worker saw complete, per set
-  if (warp != kWorkers / 32) {
-    // ---- workers
-    const int sp = warp & 3, zs = warp >> 2;  // TMEM lane quarter and z-slice of this warp
-    const int r = 32 * sp + lane;              // this thread's row of the 128-cell slice
-    // prologue: halos of tiles 0 and 1
-    for (int k = 0; k < 2 && k < ntile; ++k) {
-      load_halo<C_IN>(a_base + (uint32_t)(k * halo_bytes<C_IN>()), x, V,
-                      tile_of(blockIdx.x + (long long)k * gridDim.x, V), kWorkers);
-      asm volatile("cp.async.wait_group 0;" ::: "memory");
-      fence_proxy_async();
-      mbar_arrive(&full[k]);
-    }
-    for (int i = 0; i < ntile; ++i) {
-      const int s = i & 1;
-      const uint32_t use = (uint32_t)(i >> 1);
-      if (!wait_or_abort(&done[s], use & 1u, &abort_flag)) {
-        if (lane == 0) {
-          atomicOr(status, 16);
-          abort_flag = 1;
-        }
-        break;
-      }
-      if (s) ++n_waited1; else ++n_waited0;
-      fence_after_sync();
-      const bool more = i + 2 < ntile;
-      if (more)
-        load_halo<C_IN>(a_base + (uint32_t)(s * halo_bytes<C_IN>()), x, V,
-                        tile_of(blockIdx.x + (long long)(i + 2) * gridDim.x, V), kWorkers);
-      epilogue<C_OUT, EPI>(tmem + ((uint32_t)(32 * sp) << 16) + (uint32_t)(s * 2 * C_OUT + zs * C_OUT),
-                           tile_of(blockIdx.x + (long long)i * gridDim.x, V), V, sBias, pre_out, pre_in, out, r, zs);
+  } else if (warp == 1) {
+    // ---- MMA preparation: waits for a step's slice and accumulator, works out its window
+    const uint32_t a_lo = (uint32_t)smem_desc(a_base, A_LBO, A_SBO), b_lo = (uint32_t)smem_desc(b_base, B_LBO, B_SBO);
+    int o_run = 0;         // the run's first output, counted over the share
+    int s = 0, lap = 0;    // step g = lap kRing + s
+    int freed = kSlots;    // outputs below this index have a block to take
+    int k = 0;             // commands sent
+    auto send = [&](uint32_t d, uint32_t a, uint32_t b2, uint32_t idesc, uint32_t dn, uint32_t rd) {
+      if (k >= 2) pair_sync(kBarFree + (k & 1));
+      if (lane == 0) commands[k & 1] = MmaCommand{d, a, b2, idesc, dn, rd, 0, 0};
+      __syncwarp();
       fence_before_sync();
-      mbar_arrive(&empty[s]);
-      if (more) {
-        asm volatile("cp.async.wait_group 0;" ::: "memory");
-        fence_proxy_async();
-        mbar_arrive(&full[s]);
+      pair_arrive(kBarReady + (k & 1));
+      ++k;
+    };
+    for (Cursor cu(t0, t1, V); cu.live();) {
+      bool ok = wait_warp(&full[s], (uint32_t)lap & 1u);
+      if (ok && cu.step < cu.run.n && o_run + cu.step >= freed) {
+        // the next four blocks at once: each group reads its outputs in order,
+        // so the last one of either parity vouches for the other
+        const uint32_t ph = (uint32_t)(freed / kSlots - 1) & 1u;
+        ok = wait_warp(&empty[(freed + 2) % kSlots], ph) && wait_warp(&empty[(freed + 3) % kSlots], ph);
+        freed += 4;
       }
+      if (!ok) break;
+      fence_after_sync();
+      const int z = cu.z_in();
+      const uint32_t dn = smem_u32(&done[s]), rd = cu.step >= 2 ? smem_u32(&ready[(o_run + cu.step - 2) % kSlots]) : 0u;
+      if (z >= 0 && z < V.nz) {
+        // outputs z - 1 .. z + 1 that lie in the run; a window around the ring's end in two parts
+        const int lo = max(cu.step - 2, 0), hi = min(cu.step, cu.run.n - 1);
+        const int cnt = hi - lo + 1, slot = (o_run + lo) % kSlots, head = min(cnt, kSlots - slot);
+        const uint32_t ad = a_lo + (uint32_t)(s * (int)(slice_bytes<C_IN>() / 16));
+        const uint32_t bd = b_lo + (uint32_t)((lo - (cu.step - 2)) * C_OUT);
+        constexpr uint32_t kBlock = (uint32_t)(C_OUT >> 3) << 17;  // of the descriptor's N
+        const uint32_t id1 = idesc_bf16(128, C_OUT) - kBlock;
+        if (head < cnt) send(tmem + (uint32_t)(slot * C_OUT), ad, bd, id1 + (uint32_t)head * kBlock, 0u, 0u);
+        const int from = head < cnt ? head : 0;
+        send(tmem + (uint32_t)((slot + from) % kSlots * C_OUT), ad, bd + (uint32_t)(from * C_OUT),
+             id1 + (uint32_t)(cnt - from) * kBlock, dn, rd);
+      } else {
+        send(tmem, 0u, 0u, 0u, dn, rd);
+      }
+      if (++s == kRing) {
+        s = 0;
+        ++lap;
+      }
+      if (lane == 0) n_committed = lap * kRing + s;
+      const int n = cu.run.n;
+      if (cu.advance(V)) o_run += n;
+    }
+    send(0xffffffffu, 0u, 0u, 0u, 0u, 0u);
+  } else if (warp < kFirstEpi / 32) {
+    // ---- loaders
+    const int grp = ((int)threadIdx.x - kFirstLoader) / kLoaders;
+    const bool poller = ((int)threadIdx.x - kFirstLoader) % kLoaders == 0;
+    HaloLoader<C_IN> hl;
+    Cursor ld(t0, t1, V);
+    if (ld.live()) hl.set(x, V, ld.run);
+    auto next = [&]() {
+      if (ld.advance(V) && ld.live()) hl.set(x, V, ld.run);
+    };
+    auto landed = [&](int g) {  // this warp's part of step g's slice
+      fence_proxy_async();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&full[g % kRing]);
+    };
+    if (grp && ld.live()) next();
+    int g = grp;
+    for (; ld.live(); g += 2) {
+      if (g >= kRing) {
+        if (!group_all(kBarLoad + grp, kLoaders, !poller || wait(&done[g % kRing], (uint32_t)(g / kRing - 1) & 1u))) break;
+        if (poller) n_next[grp] = g - kRing + 2;
+      }
+      const int z = ld.z_in();
+      if (z >= 0 && z < V.nz) hl.load(a_base + (uint32_t)((g % kRing) * slice_bytes<C_IN>()), x, z);
+      asm volatile("cp.async.commit_group;" ::: "memory");
+      if (g >= 2 * kLoadLag + grp) {
+        asm volatile("cp.async.wait_group %0;" ::"n"(kLoadLag) : "memory");
+        landed(g - 2 * kLoadLag);
+      }
+      next();
+      if (ld.live()) next();
+    }
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    for (int k = max(g - 2 * kLoadLag, grp); k < g; k += 2) landed(k);
+  } else {
+    // ---- epilogue
+    const int w = warp - kFirstEpi / 32, grp = w / (kEpiGroup / 32);
+    const int sp = warp & 3, c0 = ((w >> 2) & 1) * NC;  // tensor-memory lane quarter, first channel
+    const int r = 32 * sp + lane;                    // this thread's cell of the slice
+    const uint32_t t_lane = tmem + ((uint32_t)(32 * sp) << 16) + (uint32_t)c0;
+    // the group's polling thread: a warp on another sub-partition than the MMAs'
+    const bool poller = w % (kEpiGroup / 32) == 1 && lane == 0;
+    Epilogue<C_OUT, EPI> ep;
+    if constexpr (EPI != EPI_SILU_BWD) {
+#pragma unroll
+      for (int i = 0; i < NC; ++i) ep.bias[i] = b[c0 + i];
+    }
+    int o = 0;
+    bool ok = true;
+    for (Cursor cu(t0, t1, V); ok && cu.live();) {
+      ep.set(V, cu.run, r, c0);
+      const int n = cu.run.n;
+      for (int j = (o + grp) & 1; j < n; j += 2) {
+        const int slot = (o + j) % kSlots;
+        ep.prefetch(pre_in, j);
+        ok = group_all(kBarEpi + grp, kEpiGroup, !poller || wait(&ready[slot], (uint32_t)((o + j) / kSlots) & 1u));
+        if (!ok) break;
+        fence_after_sync();
+        float acc[NC];
+        tmem_take<NC>(t_lane + (uint32_t)(slot * C_OUT), acc);
+        asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+        fence_before_sync();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&empty[slot]);
+        ep.store(acc, pre_out, out, j);
+        __syncwarp();
+      }
+      o += n;
+      cu.step = n + 1;  // to the next run
+      cu.advance(V);
     }
   }
   asm volatile("cp.async.wait_group 0;" ::: "memory");
@@ -394,23 +607,23 @@ __global__ void __launch_bounds__(kTcThreads, 1)
   fence_before_sync();
   __syncthreads();
   if (abort_flag && threadIdx.x == 0) {
-    // committed MMAs may still run: wait (bounded) for every batch committed
+    // committed MMAs may still run: wait (bounded) for every step committed
     // but not yet seen complete before tensor and shared memory are released
-    for (int k = 0; k < 2; ++k)
-      for (int ph = k ? n_waited1 : n_waited0; ph < n_committed[k]; ++ph)
-        for (long long n = 0; n < kWaitPolls && !mbar_try(&done[k], (uint32_t)ph & 1u); ++n) {
+    for (int q = 0; q < 2; ++q)
+      for (int g = n_next[q]; g < n_committed; g += 2)
+        for (long long n = 0; n < kWaitPolls && !mbar_try(&done[g % kRing], (uint32_t)(g / kRing) & 1u); ++n) {
         }
   }
   __syncthreads();
   if (warp == 0) {
     fence_after_sync();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TCOLS) : "memory");
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");
   }
 }
 
 }  // namespace
 
-size_t conv_tc_smem_bytes(int cin, int cout) { return 2 * (size_t)cin / 8 * HN * 16 + (size_t)27 * cout * cin * 2; }
+size_t conv_tc_smem_bytes(int cin, int cout) { return kRing * ((size_t)cin / 8 * HN * 16) + (size_t)27 * cout * cin * 2; }
 
 template <int C_IN, int C_OUT, int EPI>
 cudaError_t conv3d_tc(const __nv_bfloat16 *x, const __nv_bfloat16 *W, const float *b, const Vol &V,
@@ -419,16 +632,13 @@ cudaError_t conv3d_tc(const __nv_bfloat16 *x, const __nv_bfloat16 *W, const floa
   const void *fn = (const void *)conv3d_tc_kernel<C_IN, C_OUT, EPI>;
   cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   if (e != cudaSuccess) return e;
-  const long long nt = (long long)V.n * ((V.nz + TZ - 1) / TZ) * ((V.ny + TY - 1) / TY) * ((V.nx + TX - 1) / TX);
+  const long long nt = (long long)V.n * ((V.ny + TY - 1) / TY) * ((V.nx + TX - 1) / TX) * V.nz;
   if (nt < 1) return cudaSuccess;
-  int dev = 0, sms = 0, per = 0;
+  int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, fn, kTcThreads, sm) != cudaSuccess || per < 1) per = 1;
-  // tensor memory: at most 4 CTAs of <= 128 columns share an SM's 512
-  if (per > 4) per = 4;
-  long long g = (long long)per * sms;
-  if (g > nt) g = nt;
+  // one CTA per SM (it takes all of tensor memory), equal shares of the slices
+  const long long g = nt < sms ? nt : sms;
   conv3d_tc_kernel<C_IN, C_OUT, EPI><<<(int)g, kTcThreads, sm, st>>>(x, W, b, V, pre_out, pre_in, out, status);
   return cudaGetLastError();
 }
