@@ -1,16 +1,11 @@
 // vet_cnn.cu -- kernels of the learned closure (not in the VETTAM paper: a
 // 3D convolutional network predicting the Eddington tensor from local
-// features, with the exact ray tracer as fallback): features, the weight
-// gradient of the convolutions, head and loss, AdamW, indicator and block
-// list.  The convolutions themselves (forward and data gradient) run on the
-// tcgen05 tensor cores (vet_cnn_tc.cu).
+// features, with the exact ray tracer as fallback): features, head and loss,
+// AdamW, indicator and block list.  The convolutions and their weight gradients
+// run on the tcgen05 tensor cores (vet_cnn_tc.cu).
 //
 // Activations are stored cells-major, channels-minor ([volume][z][y][x][C],
-// BF16, C a multiple of 16).  The weight gradient is, per tap, a GEMM with
-// M = output channels, N = input channels and K = the 256 cells of an
-// 8 x 8 x 4 tile, on BF16 mma.sync (m16n8k16, FP32 accumulate) with
-// ldmatrix.trans operands from shared memory whose rows are XOR-swizzled in
-// 16-byte chunks (every ldmatrix phase touches 8 distinct bank groups).
+// BF16, C a multiple of 16).
 #include <cstdint>
 
 #include <cuda_bf16.h>
@@ -20,180 +15,6 @@
 namespace vet {
 namespace cnn {
 namespace {
-
-constexpr int TX = 8, TY = 8, TZ = 4;      // output tile
-constexpr int HX = 10, HY = 10, HZ = 6;    // input halo
-constexpr int HN = HX * HY * HZ;           // 600 halo cells
-constexpr int TN = TX * TY * TZ;           // 256 tile cells
-constexpr int kThreads = 256;
-
-__device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-// Byte offset of 16-byte chunk c of row `row` in a swizzled array whose rows
-// hold `nch` chunks (C/8 BF16 values each).
-__device__ __forceinline__ int swz_off(int row, int c, int nch) {
-  const int s = nch == 4 ? (c ^ ((row >> 1) & 3)) : (nch == 2 ? (c ^ ((row >> 2) & 1)) : c);
-  return row * nch * 16 + s * 16;
-}
-
-__device__ __forceinline__ void ldsm_x4_t(uint32_t addr, uint32_t &r0, uint32_t &r1, uint32_t &r2, uint32_t &r3) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
-               : "=r"(r0), "=r"(r1), "=r"(r2), "=r"(r3)
-               : "r"(addr));
-}
-
-__device__ __forceinline__ void mma_bf16(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0,
-                                         uint32_t b1) {
-  asm volatile(
-      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
-      "{%0,%1,%2,%3};"
-      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-      : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
-}
-
-
-struct TileIdx {
-  int v, tz, ty, tx;
-};
-
-__device__ __forceinline__ TileIdx tile_of(long long t, const Vol &V) {
-  const int ntx = (V.nx + TX - 1) / TX, nty = (V.ny + TY - 1) / TY, ntz = (V.nz + TZ - 1) / TZ;
-  TileIdx r;
-  r.tx = (int)(t % ntx);
-  t /= ntx;
-  r.ty = (int)(t % nty);
-  t /= nty;
-  r.tz = (int)(t % ntz);
-  r.v = (int)(t / ntz);
-  return r;
-}
-
-__device__ __forceinline__ long long ntiles_of(const Vol &V) {
-  return (long long)V.n * ((V.nz + TZ - 1) / TZ) * ((V.ny + TY - 1) / TY) * ((V.nx + TX - 1) / TX);
-}
-
-// Stage the 10 x 10 x 6 halo of tile `ti` of x (C channels) into smem;
-// cells outside the volume are zero (zero padding).
-template <int C>
-__device__ __forceinline__ void load_halo(unsigned char *sm, const __nv_bfloat16 *__restrict__ x, const Vol &V,
-                                          const TileIdx &ti) {
-  constexpr int NCH = C / 8;
-  const long long vol = (long long)V.nz * V.ny * V.nx;
-  for (int h = threadIdx.x; h < HN * NCH; h += blockDim.x) {
-    const int hc = h / NCH, c = h - hc * NCH;
-    const int hz = hc / (HX * HY), hy = (hc / HX) % HY, hx = hc % HX;
-    const int z = ti.tz * TZ + hz - 1, y = ti.ty * TY + hy - 1, xx = ti.tx * TX + hx - 1;
-    int4 val = make_int4(0, 0, 0, 0);
-    if (z >= 0 && z < V.nz && y >= 0 && y < V.ny && xx >= 0 && xx < V.nx) {
-      const long long cell = (long long)ti.v * vol + ((long long)z * V.ny + y) * V.nx + xx;
-      val = reinterpret_cast<const int4 *>(x + cell * C)[c];
-    }
-    *reinterpret_cast<int4 *>(sm + swz_off(hc, c, NCH)) = val;
-  }
-}
-
-// ---------------------------------------------------------- weight gradient
-// gW[tap][co][ci] += sum_cells gpre[cell][co] * x[cell + tap][ci];
-// gb[co] += sum_cells gpre[cell][co].  A GEMM per tap with M = C_OUT,
-// N = C_IN and K = the 256 cells of a tile; warp w owns taps w, w + 8, ...
-// and folds each tile's products into a shared FP32 accumulator (no other
-// warp writes those rows), flushed to global memory with atomics once per
-// CTA.  Accumulator rows are float2 pairs of input channels, the pair index
-// XOR-swizzled by the output channel so that a warp's fold is 2-way at most.
-template <int C_IN>
-__device__ __forceinline__ int acc_pair(int co, int p) {
-  return C_IN == 32 ? (p ^ ((co & 3) << 2)) : (p ^ (((co >> 1) & 1) << 2));
-}
-
-template <int C_IN, int C_OUT>
-__global__ void __launch_bounds__(kThreads, 1)
-    wgrad_kernel(const __nv_bfloat16 *__restrict__ x, const __nv_bfloat16 *__restrict__ gpre, Vol V,
-                 float *__restrict__ gW, float *__restrict__ gb) {
-  extern __shared__ __align__(128) unsigned char smem[];
-  constexpr int NCI = C_IN / 8, NCO = C_OUT / 8, MT = C_OUT / 16, NT = C_IN / 8, NP = C_IN / 2;
-  float2 *sAcc = reinterpret_cast<float2 *>(smem);             // [27][C_OUT][NP]
-  unsigned char *sX = smem + 27 * C_OUT * C_IN * 4;             // 600 halo rows of C_IN
-  unsigned char *sG = sX + HN * C_IN * 2;                       // 256 tile rows of C_OUT
-  for (int i = threadIdx.x; i < 27 * C_OUT * NP; i += blockDim.x) sAcc[i] = make_float2(0.f, 0.f);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int g = lane >> 2, t4 = lane & 3, q = lane >> 3, r8 = lane & 7;
-  constexpr int BSL = kThreads / C_OUT;  // bias: thread owns channel tid % C_OUT, cells tid / C_OUT + BSL j
-  const int bco = threadIdx.x % C_OUT, bks = threadIdx.x / C_OUT;
-  float bacc = 0.f;
-  const long long vol = (long long)V.nz * V.ny * V.nx;
-  const long long nt = ntiles_of(V);
-  for (long long tile = blockIdx.x; tile < nt; tile += gridDim.x) {
-    const TileIdx ti = tile_of(tile, V);
-    __syncthreads();
-    load_halo<C_IN>(sX, x, V, ti);
-    for (int h = threadIdx.x; h < TN * NCO; h += blockDim.x) {
-      const int k = h / NCO, c = h - k * NCO;
-      const int z = ti.tz * TZ + (k >> 6), y = ti.ty * TY + ((k >> 3) & 7), xx = ti.tx * TX + (k & 7);
-      int4 val = make_int4(0, 0, 0, 0);
-      if (z < V.nz && y < V.ny && xx < V.nx) {
-        const long long cell = (long long)ti.v * vol + ((long long)z * V.ny + y) * V.nx + xx;
-        val = reinterpret_cast<const int4 *>(gpre + cell * C_OUT)[c];
-      }
-      *reinterpret_cast<int4 *>(sG + swz_off(k, c, NCO)) = val;
-    }
-    __syncthreads();
-    for (int k = bks; k < TN; k += BSL)
-      bacc += __bfloat162float(*reinterpret_cast<const __nv_bfloat16 *>(sG + swz_off(k, bco >> 3, NCO) + (bco & 7) * 2));
-    for (int tap = warp; tap < 27; tap += kThreads / 32) {
-      const int dz = tap / 9 - 1, dy = (tap / 3) % 3 - 1, dx = tap % 3 - 1;
-      float acc[MT][NT][4];
-#pragma unroll
-      for (int mt = 0; mt < MT; ++mt)
-#pragma unroll
-        for (int j = 0; j < NT; ++j)
-#pragma unroll
-          for (int e = 0; e < 4; ++e) acc[mt][j][e] = 0.f;
-      for (int ks = 0; ks < TN / 16; ++ks) {
-        uint32_t a[MT][4];
-#pragma unroll
-        for (int mt = 0; mt < MT; ++mt) {
-          // A = gpre^T: rows co, k = cells; stored [cell][co] -> transposed load
-          const int k = 16 * ks + r8 + 8 * (q >> 1);
-          ldsm_x4_t(smem_u32(sG + swz_off(k, 2 * mt + (q & 1), NCO)), a[mt][0], a[mt][1], a[mt][2], a[mt][3]);
-        }
-#pragma unroll
-        for (int j = 0; j < NT; j += 2) {
-          // B = shifted input: k = cells, n = ci; stored [halo cell][ci]
-          const int k = 16 * ks + r8 + 8 * (q & 1);
-          const int hc = ((k >> 6) + 1 + dz) * (HX * HY) + (((k >> 3) & 7) + 1 + dy) * HX + ((k & 7) + 1 + dx);
-          uint32_t b0, b1, b2, b3;
-          ldsm_x4_t(smem_u32(sX + swz_off(hc, j + (q >> 1), NCI)), b0, b1, b2, b3);
-#pragma unroll
-          for (int mt = 0; mt < MT; ++mt) {
-            mma_bf16(acc[mt][j], a[mt][0], a[mt][1], a[mt][2], a[mt][3], b0, b1);
-            mma_bf16(acc[mt][j + 1], a[mt][0], a[mt][1], a[mt][2], a[mt][3], b2, b3);
-          }
-        }
-      }
-      float2 *row = sAcc + (size_t)tap * C_OUT * NP;
-#pragma unroll
-      for (int mt = 0; mt < MT; ++mt)
-#pragma unroll
-        for (int j = 0; j < NT; ++j)
-#pragma unroll
-          for (int half = 0; half < 2; ++half) {
-            const int co = 16 * mt + g + 8 * half, p = 4 * j + t4;
-            float2 &s = row[co * NP + acc_pair<C_IN>(co, p)];
-            s.x += acc[mt][j][2 * half];
-            s.y += acc[mt][j][2 * half + 1];
-          }
-    }
-  }
-  __syncthreads();
-  for (int i = threadIdx.x; i < 27 * C_OUT * NP; i += blockDim.x) {
-    const int tap = i / (C_OUT * NP), rem = i - tap * C_OUT * NP, co = rem / NP, p = rem - co * NP;
-    const float2 s = sAcc[(size_t)tap * C_OUT * NP + co * NP + acc_pair<C_IN>(co, p)];
-    float *dst = gW + ((long long)tap * C_OUT + co) * C_IN + 2 * p;
-    atomicAdd(dst, s.x);
-    atomicAdd(dst + 1, s.y);
-  }
-  atomicAdd(gb + bco, bacc);
-}
 
 // ---------------------------------------------------------------- features
 // Per (volume, block) CTA: mean and standard deviation (population) of
@@ -478,41 +299,6 @@ int grid_for(long long n, int threads) {
 
 }  // namespace
 
-size_t wgrad_smem_bytes(int cin, int cout) {
-  return (size_t)27 * cout * cin * 4 + (size_t)HN * cin * 2 + (size_t)TN * cout * 2;
-}
-long long tiles(const Vol &V) {
-  return (long long)V.n * ((V.nz + TZ - 1) / TZ) * ((V.ny + TY - 1) / TY) * ((V.nx + TX - 1) / TX);
-}
-
-namespace {
-// Persistent grid: resident CTAs per SM x SMs, capped by the tile count and
-// by `cap` when positive.
-int persistent_grid(const void *fn, size_t smem, long long nt, int cap) {
-  int dev = 0, sms = 0, per = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, fn, kThreads, smem) != cudaSuccess || per < 1) per = 1;
-  long long g = (long long)per * sms;
-  if (cap > 0 && g > cap) g = cap;
-  if (g > nt) g = nt;
-  return (int)g;
-}
-}  // namespace
-
-template <int C_IN, int C_OUT>
-cudaError_t wgrad(const __nv_bfloat16 *x, const __nv_bfloat16 *gpre, const Vol &V, float *gW, float *gb, int grid,
-                  cudaStream_t st) {
-  const size_t sm = wgrad_smem_bytes(C_IN, C_OUT);
-  const void *fn = (const void *)wgrad_kernel<C_IN, C_OUT>;
-  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-  if (e != cudaSuccess) return e;
-  const int g = persistent_grid(fn, sm, tiles(V), grid);
-  if (g < 1) return cudaSuccess;
-  wgrad_kernel<C_IN, C_OUT><<<g, kThreads, sm, st>>>(x, gpre, V, gW, gb);
-  return cudaGetLastError();
-}
-
 cudaError_t features(const float *kappa, const float *S, const float *E, const Vol &V, int B, double h, double *sums,
                      float *bstat, __nv_bfloat16 *x0, float *feat_out, cudaStream_t st) {
   if (V.n < 1) return cudaSuccess;
@@ -564,13 +350,6 @@ cudaError_t unpack_outputs(const float *o, const Vol &V, float *o_out, cudaStrea
   unpack_kernel<<<grid_for(n, 256), 256, 0, st>>>(o, V, o_out);
   return cudaGetLastError();
 }
-
-template cudaError_t wgrad<16, 32>(const __nv_bfloat16 *, const __nv_bfloat16 *, const Vol &, float *, float *, int,
-                                   cudaStream_t);
-template cudaError_t wgrad<32, 32>(const __nv_bfloat16 *, const __nv_bfloat16 *, const Vol &, float *, float *, int,
-                                   cudaStream_t);
-template cudaError_t wgrad<32, 16>(const __nv_bfloat16 *, const __nv_bfloat16 *, const Vol &, float *, float *, int,
-                                   cudaStream_t);
 
 }  // namespace cnn
 }  // namespace vet

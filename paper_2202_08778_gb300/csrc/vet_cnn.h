@@ -28,8 +28,6 @@ struct Vol {
 
 enum { EPI_SILU = 0, EPI_F32 = 1, EPI_SILU_BWD = 2 };
 
-size_t wgrad_smem_bytes(int cin, int cout);
-long long tiles(const Vol &V);
 
 // out = epi(conv3d(x, W) + b) on the tcgen05 tensor cores (vet_cnn_tc.cu):
 // tiles of 8 x 16 x 2 cells, accumulators in tensor memory.  Epilogues:
@@ -45,9 +43,10 @@ cudaError_t conv3d_tc(const __nv_bfloat16 *x, const __nv_bfloat16 *W, const floa
                       __nv_bfloat16 *pre_out, const __nv_bfloat16 *pre_in, void *out, int *status, cudaStream_t st);
 
 // gW[tap][co][ci] += sum_cells gpre[cell][co] x[cell + tap][ci], gb[co] +=
-// sum_cells gpre[cell][co] (FP32, accumulated into the given arrays).
+// sum_cells gpre[cell][co] (FP32, accumulated into the given arrays; 16-byte
+// aligned gW) on the tensor cores (vet_cnn_tc.cu), status as conv3d_tc's.
 template <int C_IN, int C_OUT>
-cudaError_t wgrad(const __nv_bfloat16 *x, const __nv_bfloat16 *gpre, const Vol &V, float *gW, float *gb, int grid,
+cudaError_t wgrad(const __nv_bfloat16 *x, const __nv_bfloat16 *gpre, const Vol &V, float *gW, float *gb, int *status,
                   cudaStream_t st);
 
 // Features of the learned closure into x0 [cells][16] BF16; sums [n][2]

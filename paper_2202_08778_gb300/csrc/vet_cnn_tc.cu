@@ -25,8 +25,8 @@
 // Tensor memory: a ring of 512 / C_out output slices (all 512 columns, one
 // CTA per SM), each zeroed by the epilogue that read it; a window of three
 // slices that wraps around the ring's end is issued as two sets of MMAs.
-// 128^3, ncu: 32 -> 32 channels 261 -> 95 us, 16 -> 32 150 -> 83 us, 32 -> 16
-// 248 -> 92 us; the network on one 128^3 grid 1144 -> 594 us.
+// 128^3, ncu: 32 -> 32 channels 261 -> 95 us, 16 -> 32 150 -> 77 us, 32 -> 16
+// 248 -> 95 us; the network on one 128^3 grid 1144 -> 588 us.
 #include <cstdint>
 
 #include <cuda_bf16.h>
@@ -146,6 +146,28 @@ __device__ __forceinline__ void tmem_take<8>(uint32_t taddr, float (&v)[8]) {
   for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[i]);
 }
 
+// Loads (no wait) and stores of 16 columns.
+__device__ __forceinline__ void tmem_load16(uint32_t taddr, uint32_t (&r)[16]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+      : "r"(taddr));
+}
+__device__ __forceinline__ void tmem_store16(uint32_t taddr, const uint32_t (&r)[16]) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};" ::"r"(taddr),
+               "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]),
+               "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
+               : "memory");
+}
+__device__ __forceinline__ void tmem_zero16(uint32_t taddr) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1};" ::"r"(taddr),
+               "r"(0u)
+               : "memory");
+}
+__device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+__device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+
 // A run of n output slices za .. za + n - 1 of one column.
 struct Run {
   int v, ty, tx, za, n;
@@ -196,7 +218,6 @@ constexpr int kLoaders = 128;             // warps 2-5, 6-9: halo loads of the e
 constexpr int kFirstEpi = kFirstLoader + 2 * kLoaders;
 constexpr int kEpiGroup = 256;            // warps 10-17, 18-25: epilogue of the even and odd output slices
 constexpr int kTcThreads = kFirstEpi + 2 * kEpiGroup;
-constexpr int kLoadLag = 1;               // steps of its own that a loader group waits behind its loads
 
 // Halo loads of one thread (cp.async, zero outside the volume): its up to
 // six 16-byte pieces sit at the same place in every slice of a column, so
@@ -212,7 +233,7 @@ struct HaloLoader {
     base = x + (long long)r.v * V.nz * plane;
 #pragma unroll
     for (int k = 0; k < K; ++k) {
-      const int h = ((int)threadIdx.x - kFirstLoader) % kLoaders + k * kLoaders, c = h / HN, hc = h - c * HN;
+      const int h = ((int)threadIdx.x - kFirstLoader) % kLoaders + k * kLoaders, hc = h / NCI, c = h - hc * NCI;
       const int y = r.ty * TY + hc / HX - 1, xx = r.tx * TX + hc % HX - 1;
       off[k] = y >= 0 && y < V.ny && xx >= 0 && xx < V.nx ? ((long long)y * V.nx + xx) * C_IN + c * 8 : -1;
     }
@@ -220,7 +241,7 @@ struct HaloLoader {
   __device__ __forceinline__ void load(uint32_t dst, const __nv_bfloat16 *__restrict__ x, int z) const {
 #pragma unroll
     for (int k = 0; k < K; ++k) {
-      const int h = ((int)threadIdx.x - kFirstLoader) % kLoaders + k * kLoaders, c = h / HN, hc = h - c * HN;
+      const int h = ((int)threadIdx.x - kFirstLoader) % kLoaders + k * kLoaders, hc = h / NCI, c = h - hc * NCI;
       if (h < HN * NCI)
         cp_async16(dst + (uint32_t)((c * HN + hc) * 16), off[k] >= 0 ? base + z * plane + off[k] : x, off[k] >= 0 ? 16u : 0u);
     }
@@ -231,7 +252,8 @@ struct HaloLoader {
 // of neighbouring output slices (idesc 0: none), then the commits.
 struct alignas(16) MmaCommand {
   uint32_t d, a, b, idesc;     // accumulator; low words of the descriptors; 0xffffffff: the end
-  uint32_t done, ready, pad0, pad1;  // shared addresses of the barriers to commit to (0: none)
+  uint32_t done, ready;              // shared addresses of the barriers to commit to (0: none)
+  uint32_t flags, pad;               // weight gradient: kFlush..
 };
 
 // Named-barrier hand-over between the preparing and the issuing warp.
@@ -555,15 +577,15 @@ __global__ void __launch_bounds__(kTcThreads, 1)
       const int z = ld.z_in();
       if (z >= 0 && z < V.nz) hl.load(a_base + (uint32_t)((g % kRing) * slice_bytes<C_IN>()), x, z);
       asm volatile("cp.async.commit_group;" ::: "memory");
-      if (g >= 2 * kLoadLag + grp) {
-        asm volatile("cp.async.wait_group %0;" ::"n"(kLoadLag) : "memory");
-        landed(g - 2 * kLoadLag);
+      if (g >= 2) {
+        asm volatile("cp.async.wait_group 1;" ::: "memory");
+        landed(g - 2);
       }
       next();
       if (ld.live()) next();
     }
     asm volatile("cp.async.wait_group 0;" ::: "memory");
-    for (int k = max(g - 2 * kLoadLag, grp); k < g; k += 2) landed(k);
+    if (g >= 2) landed(g - 2);
   } else {
     // ---- epilogue
     const int w = warp - kFirstEpi / 32, grp = w / (kEpiGroup / 32);
@@ -621,6 +643,403 @@ __global__ void __launch_bounds__(kTcThreads, 1)
   }
 }
 
+// ---------------------------------------------------------- weight gradient
+// gW[dz, dy, dx][co][ci] += sum_cells g[cell][co] x[cell + (dx, dy, dz)][ci],
+// gb[co] += sum_cells g[cell][co]: a contraction over cells.  Same march along
+// the columns; per slice of g (8 x 16 cells) and dy one tcgen05.mma per 16
+// cells, with
+//   M = (dx, co), 3 C_out of 128 rows: the cells c of the column's tile read
+//     g[c - dx], from three copies of the g slice shifted in x (a tap's shift
+//     in y is an offset of whole rows in the copies),
+//   N = (dz, ci), 3 C_in: three neighbouring slices of x in their ring,
+//   K = 16 cells, two rows of the tile,
+// both operands MN-major (8 channels of a cell are the 16 contiguous bytes, the
+// cells of a row follow each other): core matrices of 8 cells x 16 bytes, SBO
+// between 8-channel chunks, LBO between rows of 8 cells.  The tensor core's
+// FP32 accumulation truncates, so chains are kept to kFlushSlices slices (16
+// MMAs): the accumulators of a dy (3 C_in columns) are then added, rounded, to
+// sums that live in the rest of tensor memory and, for what does not fit there,
+// in registers, while the MMAs of the other two dy run (chains over a CTA's
+// whole share were off by 1.4e-5 on 4 x 64^3).  The sums are added to gW
+// at the share's end by 16-byte reductions.
+// What the MMAs need: their operands' 24 x 56 clocks a slice (C_in = 32), 40 us on
+// 4 x 64^3; measured there, ncu: 32 -> 32 channels 327 -> 110 us, 32 -> 16 260 -> 88 us,
+// 16 -> 32 210 -> 84 us (before: a tap at a time by mma.sync into
+// shared-memory accumulators, the tensor pipe 28% busy).  What is left over: the
+// hand-overs of a step and the sums (20 us).
+constexpr int kWgRing = 4;   // staged g slices (even: two loader groups take turns)
+constexpr int kWgX = 8;      // staged x slices: a step's slice is read by it and the next two
+static_assert(kWgRing + 2 <= kWgX, "the wait for a g buffer must cover the x buffer");
+constexpr int kWgSum = 128;  // warps 10-13: sums of the accumulators
+constexpr int kWgBias = 64;  // warps 14, 15: bias sums
+constexpr int kWgThreads = kFirstLoader + 2 * kLoaders + kWgSum + kWgBias;
+constexpr int kFlushSlices = 2;
+constexpr uint32_t kFlush = 1, kAfterFlush = 2, kFlushOdd = 4;  // command flags: a chain ends / starts here; parity
+constexpr int kGRows = TY + 2;                      // rows of a g copy: y - 1 .. y + 16
+constexpr int kGPlane = kGRows * TX * 16, kXPlane = TY * TX * 16;  // bytes of one channel chunk
+
+template <int C_IN, int C_OUT>
+__host__ __device__ constexpr size_t wg_g_bytes() {
+  return (size_t)3 * (C_OUT / 8) * kGPlane;
+}
+template <int C_IN, int C_OUT>
+__host__ __device__ constexpr size_t wg_x_bytes() {
+  return (size_t)(C_IN / 8) * kXPlane;
+}
+// The M = 128 MMAs read 16 chunks from the last g buffer on: its own 3 C_out / 8
+// and what follows (the x ring), whose rows of the result nobody reads.
+template <int C_IN, int C_OUT>
+__host__ __device__ constexpr size_t wg_smem() {
+  return kWgRing * wg_g_bytes<C_IN, C_OUT>() + kWgX * wg_x_bytes<C_IN, C_OUT>();
+}
+
+// Loads of one thread, in 16-byte pieces from a slice's first cell (negative:
+// outside the volume, zero).
+template <int C_IN, int C_OUT>
+struct WgradLoader {
+  static constexpr int NCI = C_IN / 8, NCO = C_OUT / 8;
+  static constexpr int NG = 3 * NCO * kGRows * TX, NX = NCI * TY * TX;
+  static constexpr int KG = (NG + kLoaders - 1) / kLoaders, KX = NX / kLoaders;
+  static_assert(NX % kLoaders == 0, "x pieces divide evenly");
+  int og[KG], ox[KX];
+  const __nv_bfloat16 *gb, *xb;
+  long long plane;  // cells of a slice
+  __device__ __forceinline__ void set(const __nv_bfloat16 *__restrict__ x, const __nv_bfloat16 *__restrict__ g, const Vol &V,
+                                      const Run &r, int tid) {
+    plane = (long long)V.ny * V.nx;
+    gb = g + (long long)r.v * V.nz * plane * C_OUT;
+    xb = x + (long long)r.v * V.nz * plane * C_IN;
+#pragma unroll
+    for (int k = 0; k < KG; ++k) {
+      // a warp's lanes take whole cells: [dx][row][x][chunk]
+      const int h = tid + k * kLoaders, c = h % NCO, xc = (h / NCO) % TX, row = (h / (NCO * TX)) % kGRows;
+      const int xx = r.tx * TX + xc - (h / (NCO * TX * kGRows) - 1), y = r.ty * TY + row - 1;
+      og[k] = xx >= 0 && xx < V.nx && y >= 0 && y < V.ny ? (y * V.nx + xx) * NCO + c : -1;
+    }
+#pragma unroll
+    for (int k = 0; k < KX; ++k) {
+      const int h = tid + k * kLoaders, c = h % NCI, xc = (h / NCI) % TX, row = h / (NCI * TX);
+      const int xx = r.tx * TX + xc, y = r.ty * TY + row;
+      ox[k] = xx < V.nx && y < V.ny ? (y * V.nx + xx) * NCI + c : -1;
+    }
+  }
+  __device__ __forceinline__ void load_g(uint32_t dst, int z, int tid) const {
+    const __nv_bfloat16 *src = gb + z * plane * C_OUT;
+#pragma unroll
+    for (int k = 0; k < KG; ++k) {
+      const int h = tid + k * kLoaders;
+      if (NG % kLoaders == 0 || h < NG)
+        cp_async16(dst + (uint32_t)((h / (NCO * TX * kGRows) * NCO + h % NCO) * kGPlane + (h / NCO) % (TX * kGRows) * 16), og[k] >= 0 ? src + (long long)og[k] * 8 : gb, og[k] >= 0 ? 16u : 0u);
+    }
+  }
+  __device__ __forceinline__ void load_x(uint32_t dst, int z, int tid) const {
+    const __nv_bfloat16 *src = xb + z * plane * C_IN;
+#pragma unroll
+    for (int k = 0; k < KX; ++k)
+      cp_async16(dst + (uint32_t)((tid + k * kLoaders) % NCI * kXPlane + (tid + k * kLoaders) / NCI * 16), ox[k] >= 0 ? src + (long long)ox[k] * 8 : xb,
+                 ox[k] >= 0 ? 16u : 0u);
+  }
+};
+
+// dst[0..3] += v by one reduction.
+__device__ __forceinline__ void red_add4(float *dst, float a, float b, float c, float d) {
+  asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(dst), "f"(a), "f"(b), "f"(c), "f"(d) : "memory");
+}
+
+// Roles as in conv3d_tc_kernel; step g of a run loads x slice za - 1 + step and,
+// from step 2 on, g slice za + step - 2, whose MMAs it issues.
+template <int C_IN, int C_OUT>
+__global__ void __launch_bounds__(kWgThreads, 1)
+    wgrad_tc_kernel(const __nv_bfloat16 *__restrict__ x, const __nv_bfloat16 *__restrict__ gpre, Vol V,
+                    float *__restrict__ gW, float *__restrict__ gb, int *status) {
+  constexpr int NCO = C_OUT / 8;
+  // accumulators in columns [0, kAcc); the sums of the first kTm of them in
+  // [kAcc, kAcc + kTm), of the others in registers
+  constexpr int kAcc = 9 * C_IN, kDy = 3 * C_IN, kTm = kAcc < (int)kTmemCols - kAcc ? kAcc : (int)kTmemCols - kAcc;
+  static_assert(kTm % 16 == 0 && kDy % 16 == 0, "whole pieces of 16 columns");
+  constexpr size_t kG = wg_g_bytes<C_IN, C_OUT>(), kX = wg_x_bytes<C_IN, C_OUT>();
+  extern __shared__ __align__(128) unsigned char smem[];
+  __shared__ __align__(8) uint64_t full[kWgRing], done[kWgRing], ready[3], zeroed[3];
+  __shared__ MmaCommand commands[2];
+  __shared__ uint32_t tmem_base_slot;
+  __shared__ volatile int abort_flag;
+  __shared__ int n_committed, n_next[2];
+  __shared__ float sBias[C_OUT];
+
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (threadIdx.x < C_OUT) sBias[threadIdx.x] = 0.f;
+  if (threadIdx.x == 0) {
+    for (int k = 0; k < kWgRing; ++k) {
+      mbar_init(&full[k], kLoaders / 32);
+      mbar_init(&done[k], 1);
+    }
+    for (int k = 0; k < 3; ++k) {
+      mbar_init(&ready[k], 1);
+      mbar_init(&zeroed[k], kWgSum / 32);
+    }
+    abort_flag = 0;
+    n_committed = n_next[0] = 0;
+    n_next[1] = 1;
+  }
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_slot)),
+                 "r"(kTmemCols)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  fence_proxy_async();
+  fence_before_sync();
+  __syncthreads();
+  fence_after_sync();
+  const uint32_t tmem = tmem_base_slot;
+  const long long nt = (long long)V.n * ((V.ny + TY - 1) / TY) * ((V.nx + TX - 1) / TX) * V.nz;
+  const long long t0 = nt * blockIdx.x / gridDim.x, t1 = nt * (blockIdx.x + 1) / gridDim.x;
+  const uint32_t g_base = smem_u32(smem), x_base = g_base + (uint32_t)(kWgRing * kG);
+  auto wait = [&](uint64_t *bar, uint32_t parity) {  // one thread
+    if (wait_or_abort(bar, parity, &abort_flag)) return true;
+    atomicOr(status, 16);
+    abort_flag = 1;
+    return false;
+  };
+  constexpr int kFirstSum = (kFirstLoader + 2 * kLoaders) / 32;
+  constexpr int kFirstBias = kFirstSum + kWgSum / 32;
+  if (warp >= kFirstSum && warp < kFirstBias) {  // the accumulators and their sums start at zero
+    for (int k = 0; k < (int)kTmemCols; k += 16) tmem_zero16(tmem + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)k);
+    tmem_wait_st();
+  }
+  fence_before_sync();
+  __syncthreads();
+  fence_after_sync();
+
+  if (warp == 0) {
+    // ---- MMA issuer
+    const uint32_t a_hi = uniform((uint32_t)(smem_desc(g_base, 128, kGPlane) >> 32));
+    const uint32_t b_hi = uniform((uint32_t)(smem_desc(x_base, 128, kXPlane) >> 32));
+    MmaCommand cur, nxt;
+    int k = 0;
+    auto fetch = [&]() {
+      pair_sync(kBarReady + (k & 1));
+      nxt = commands[k & 1];
+      pair_arrive(kBarFree + (k & 1));
+      ++k;
+    };
+    fetch();
+    bool ok = true;  // once a wait gave up, commands are taken and not carried out
+    while (nxt.d != 0xffffffffu) {
+      cur = nxt;
+      fence_after_sync();
+      const uint32_t idesc = uniform(cur.idesc), d = uniform(cur.d), al = uniform(cur.a), bl = uniform(cur.b),
+                     flags = uniform(cur.flags);
+#pragma unroll
+      for (int dy = 0; dy < 3; ++dy) {
+        if (flags & kAfterFlush) {
+          ok = ok && __all_sync(0xffffffffu, wait(&zeroed[dy], flags & kFlushOdd ? 1u : 0u));
+          fence_after_sync();
+        }
+        if (idesc && ok && elect_one()) {
+#pragma unroll
+          for (int ks = 0; ks < TY / 2; ++ks)
+            mma_bf16(d + (uint32_t)(dy * kDy), al + (uint32_t)((2 * ks + 2 - dy) * TX), a_hi, bl + (uint32_t)(2 * ks * TX), b_hi,
+                     idesc);
+          if (flags & kFlush) mma_commit(smem_u32(&ready[dy]));
+        }
+        __syncwarp();
+        if (dy == 1) fetch();
+      }
+      if (cur.done && ok && elect_one()) mma_commit(cur.done);
+      __syncwarp();
+    }
+  } else if (warp == 1) {
+    // ---- MMA preparation
+    const uint32_t a_lo = (uint32_t)smem_desc(g_base, 128, kGPlane), b_lo = (uint32_t)smem_desc(x_base, 128, kXPlane);
+    int g = 0, k = 0;
+    auto send = [&](uint32_t d, uint32_t a, uint32_t b2, uint32_t idesc, uint32_t dn, uint32_t flags) {
+      if (k >= 2) pair_sync(kBarFree + (k & 1));
+      if (lane == 0) commands[k & 1] = MmaCommand{d, a, b2, idesc, dn, 0u, flags, 0u};
+      __syncwarp();
+      fence_before_sync();
+      pair_arrive(kBarReady + (k & 1));
+      ++k;
+    };
+    int i = 0;  // g slices done
+    for (Cursor cu(t0, t1, V); cu.live(); ++g) {
+      const int s = g % kWgRing;
+      if (!__all_sync(0xffffffffu, wait(&full[s], (uint32_t)(g / kWgRing) & 1u))) break;
+      fence_after_sync();
+      const int step = cu.step, zg = cu.run.za + step - 2;
+      const uint32_t dn = smem_u32(&done[s]);
+      if (step >= 2) {
+        // x slices zg - 1 .. zg + 1 in the volume; a window around the ring's end in two parts
+        const int lo = zg > 0 ? 0 : 1, hi = zg < V.nz - 1 ? 2 : 1, cnt = hi - lo + 1;
+        const int first = (g - 2 + lo) % kWgX, head = min(cnt, kWgX - first);
+        const uint32_t ad = a_lo + (uint32_t)(s * (int)(kG / 16));
+        const uint32_t fl = i % kFlushSlices == kFlushSlices - 1 || i == (int)(t1 - t0) - 1 ? kFlush : 0u;
+        uint32_t af = i && i % kFlushSlices == 0 ? kAfterFlush | ((i / kFlushSlices - 1) & 1 ? kFlushOdd : 0u) : 0u;
+        // bits 15, 16: both operands MN-major
+        const uint32_t id0 = idesc_bf16(128, 0) | (1u << 15) | (1u << 16);
+        constexpr uint32_t kBlock = (uint32_t)(C_IN >> 3) << 17;
+        if (head < cnt) {
+          send(tmem + (uint32_t)(lo * C_IN), ad, b_lo + (uint32_t)(first * (int)(kX / 16)), id0 + (uint32_t)head * kBlock, 0u, af);
+          af = 0u;
+        }
+        const int from = head < cnt ? head : 0;
+        send(tmem + (uint32_t)((lo + from) * C_IN), ad, b_lo + (uint32_t)((first + from) % kWgX * (int)(kX / 16)),
+             id0 + (uint32_t)(cnt - from) * kBlock, dn, fl | af);
+        ++i;
+      } else {
+        send(tmem, 0u, 0u, 0u, dn, 0u);
+      }
+      if (lane == 0) n_committed = g + 1;
+      cu.advance(V);
+    }
+    send(0xffffffffu, 0u, 0u, 0u, 0u, 0u);
+  } else if (warp < kFirstSum) {
+    // ---- loaders
+    const int grp = ((int)threadIdx.x - kFirstLoader) / kLoaders, tid = ((int)threadIdx.x - kFirstLoader) % kLoaders;
+    WgradLoader<C_IN, C_OUT> wl;
+    Cursor ld(t0, t1, V);
+    if (ld.live()) wl.set(x, gpre, V, ld.run, tid);
+    auto next = [&]() {
+      if (ld.advance(V) && ld.live()) wl.set(x, gpre, V, ld.run, tid);
+    };
+    auto landed = [&](int g) {
+      fence_proxy_async();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&full[g % kWgRing]);
+    };
+    if (grp && ld.live()) next();
+    int g = grp;
+    for (; ld.live(); g += 2) {
+      if (g >= 2) {
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+        landed(g - 2);
+      }
+      if (g >= kWgRing) {
+        if (!group_all(kBarLoad + grp, kLoaders, tid != 0 || wait(&done[g % kWgRing], (uint32_t)(g / kWgRing - 1) & 1u))) break;
+        if (tid == 0) n_next[grp] = g - kWgRing + 2;
+      }
+      const int z = ld.z_in();
+      if (z >= 0 && z < V.nz) wl.load_x(x_base + (uint32_t)((g % kWgX) * kX), z, tid);
+      if (ld.step >= 2) wl.load_g(g_base + (uint32_t)((g % kWgRing) * kG), z - 1, tid);
+      asm volatile("cp.async.commit_group;" ::: "memory");
+      next();
+      if (ld.live()) next();
+    }
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    if (g >= 2) landed(g - 2);
+  } else if (warp < kFirstBias) {
+    // ---- sums of the accumulators
+    const int tid = (int)threadIdx.x - 32 * kFirstSum;
+    const uint32_t t_lane = tmem + ((uint32_t)(32 * (warp & 3)) << 16);
+    constexpr int kRegs = kAcc > kTm ? kAcc - kTm : 1;
+    float sum[kRegs];
+#pragma unroll
+    for (int q = 0; q < kRegs; ++q) sum[q] = 0.f;
+    const int flushes = (int)((t1 - t0 + kFlushSlices - 1) / kFlushSlices);
+    bool ok = true;
+    for (int f = 0; f < flushes && ok; ++f) {
+#pragma unroll
+      for (int dy = 0; dy < 3; ++dy) {
+        ok = ok && group_all(kBarEpi, kWgSum, tid != 0 || wait(&ready[dy], (uint32_t)f & 1u));
+        if (!ok) break;
+        fence_after_sync();
+#pragma unroll
+        for (int q = dy * kDy; q < (dy + 1) * kDy; q += 16) {
+          uint32_t v[16], u[16];
+          tmem_load16(t_lane + (uint32_t)q, v);
+          if (q < kTm) {
+            tmem_load16(t_lane + (uint32_t)(kAcc + q), u);
+            tmem_wait_ld();
+#pragma unroll
+            for (int e = 0; e < 16; ++e) u[e] = __float_as_uint(__uint_as_float(u[e]) + __uint_as_float(v[e]));
+            tmem_store16(t_lane + (uint32_t)(kAcc + q), u);
+          } else {
+            tmem_wait_ld();
+#pragma unroll
+            for (int e = 0; e < 16; ++e) sum[q >= kTm ? q - kTm + e : 0] += __uint_as_float(v[e]);
+          }
+          tmem_zero16(t_lane + (uint32_t)q);
+        }
+        tmem_wait_st();
+        fence_before_sync();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&zeroed[dy]);
+      }
+    }
+    if (ok) {
+      const int row = 32 * (warp & 3) + lane, dx = row / C_OUT, co = row - dx * C_OUT;
+#pragma unroll
+      for (int q = 0; q < kAcc; q += 16) {
+        const int dy = q / kDy, dz = (q - dy * kDy) / C_IN, ci = q % C_IN;
+        uint32_t u[16];
+        if (q < kTm) {
+          tmem_load16(t_lane + (uint32_t)(kAcc + q), u);
+          tmem_wait_ld();
+        } else {
+#pragma unroll
+          for (int e = 0; e < 16; ++e) u[e] = __float_as_uint(sum[q >= kTm ? q - kTm + e : 0]);
+        }
+        float *dst = gW + ((long long)(dz * 9 + dy * 3 + dx) * C_OUT + co) * C_IN + ci;
+        if (dx < 3) {
+#pragma unroll
+          for (int e = 0; e < 16; e += 4)
+            red_add4(dst + e, __uint_as_float(u[e]), __uint_as_float(u[e + 1]), __uint_as_float(u[e + 2]), __uint_as_float(u[e + 3]));
+        }
+        __syncwarp();
+      }
+    }
+  } else {
+    // ---- bias sums: thread = (channel chunk, cells j, j + kWgBias / NCO, ...) of every g slice
+    const int tid = (int)threadIdx.x - 32 * kFirstBias, c = tid % NCO;
+    float acc[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) acc[i] = 0.f;
+    for (Cursor cu(t0, t1, V); cu.live();) {
+      const long long plane = (long long)V.ny * V.nx;
+#pragma unroll 1
+      for (int j = tid / NCO; j < TX * TY; j += kWgBias / NCO) {
+        const int xx = cu.run.tx * TX + j % TX, y = cu.run.ty * TY + j / TX;
+        if (xx >= V.nx || y >= V.ny) continue;
+        const int4 *src = reinterpret_cast<const int4 *>(
+                              gpre + ((((long long)cu.run.v * V.nz + cu.run.za) * V.ny + y) * V.nx + xx) * C_OUT) +
+                          c;
+#pragma unroll 4
+        for (int z = 0; z < cu.run.n; ++z) {
+          const int4 q = src[z * plane * NCO];
+          const __nv_bfloat162 *h = reinterpret_cast<const __nv_bfloat162 *>(&q);
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const float2 f = __bfloat1622float2(h[i]);
+            acc[2 * i] += f.x;
+            acc[2 * i + 1] += f.y;
+          }
+        }
+      }
+      cu.step = cu.run.n + 1;  // to the next run
+      cu.advance(V);
+    }
+#pragma unroll
+    for (int i = 0; i < 8; ++i) atomicAdd(&sBias[c * 8 + i], acc[i]);
+  }
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
+  __syncwarp();
+  fence_before_sync();
+  __syncthreads();
+  if (threadIdx.x < C_OUT && !abort_flag) atomicAdd(gb + threadIdx.x, sBias[threadIdx.x]);
+  if (abort_flag && threadIdx.x == 0) {
+    // committed MMAs may still run (see conv3d_tc_kernel)
+    for (int q = 0; q < 2; ++q)
+      for (int g = n_next[q]; g < n_committed; g += 2)
+        for (long long n = 0; n < kWaitPolls && !mbar_try(&done[g % kWgRing], (uint32_t)(g / kWgRing) & 1u); ++n) {
+        }
+  }
+  __syncthreads();
+  if (warp == 0) {
+    fence_after_sync();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");
+  }
+}
+
 }  // namespace
 
 size_t conv_tc_smem_bytes(int cin, int cout) { return kRing * ((size_t)cin / 8 * HN * 16) + (size_t)27 * cout * cin * 2; }
@@ -643,6 +1062,24 @@ cudaError_t conv3d_tc(const __nv_bfloat16 *x, const __nv_bfloat16 *W, const floa
   return cudaGetLastError();
 }
 
+template <int C_IN, int C_OUT>
+cudaError_t wgrad(const __nv_bfloat16 *x, const __nv_bfloat16 *gpre, const Vol &V, float *gW, float *gb, int *status,
+                  cudaStream_t st) {
+  constexpr size_t sm = wg_smem<C_IN, C_OUT>();
+  static_assert((kWgRing - 1) * wg_g_bytes<C_IN, C_OUT>() + 16 * kGPlane <= sm, "the MMAs' 16 chunks stay in shared memory");
+  const void *fn = (const void *)wgrad_tc_kernel<C_IN, C_OUT>;
+  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  if (e != cudaSuccess) return e;
+  const long long nt = (long long)V.n * ((V.ny + TY - 1) / TY) * ((V.nx + TX - 1) / TX) * V.nz;
+  if (nt < 1) return cudaSuccess;
+  int dev = 0, sms = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const long long g = nt < sms ? nt : sms;
+  wgrad_tc_kernel<C_IN, C_OUT><<<(int)g, kWgThreads, sm, st>>>(x, gpre, V, gW, gb, status);
+  return cudaGetLastError();
+}
+
 #define VET_TC_INST(CI, CO, EPI)                                                                                  \
   template cudaError_t conv3d_tc<CI, CO, EPI>(const __nv_bfloat16 *, const __nv_bfloat16 *, const float *,       \
                                               const Vol &, __nv_bfloat16 *, const __nv_bfloat16 *, void *, int *, \
@@ -652,6 +1089,13 @@ VET_TC_INST(32, 32, EPI_SILU)
 VET_TC_INST(32, 16, EPI_F32)
 VET_TC_INST(16, 32, EPI_SILU_BWD)
 VET_TC_INST(32, 32, EPI_SILU_BWD)
+
+#define VET_WG_INST(CI, CO)                                                                                    \
+  template cudaError_t wgrad<CI, CO>(const __nv_bfloat16 *, const __nv_bfloat16 *, const Vol &, float *, float *, \
+                                     int *, cudaStream_t);
+VET_WG_INST(16, 32)
+VET_WG_INST(32, 32)
+VET_WG_INST(32, 16)
 
 }  // namespace cnn
 }  // namespace vet

@@ -486,16 +486,16 @@ VET_API vet_status vet_model_backward(vet_model *m, const float *f_ref, const ui
   cudaError_t e = cudaMemsetAsync(m->g, 0, sizeof(float) * m->meta.total, st);
   if (!e) e = head_loss(m->o, f_ref, mask, V, lam, m->count, m->loss, m->go, st);
   // layer 4: gradient of its output is go
-  if (!e) e = wgrad<kHidden, kOutPad>(m->act[2], m->go, V, gW(m, 3), gb(m, 3), 0, st);
+  if (!e) e = wgrad<kHidden, kOutPad>(m->act[2], m->go, V, gW(m, 3), gb(m, 3), m->status, st);
   if (!e) e = conv3d_tc<kOutPad, kHidden, EPI_SILU_BWD>(m->go, Wt(m, 3), nullptr, V, nullptr, m->pre[2], m->g1, m->status, st);
   // layer 3
-  if (!e) e = wgrad<kHidden, kHidden>(m->act[1], m->g1, V, gW(m, 2), gb(m, 2), 0, st);
+  if (!e) e = wgrad<kHidden, kHidden>(m->act[1], m->g1, V, gW(m, 2), gb(m, 2), m->status, st);
   if (!e) e = conv3d_tc<kHidden, kHidden, EPI_SILU_BWD>(m->g1, Wt(m, 2), nullptr, V, nullptr, m->pre[1], m->g2, m->status, st);
   // layer 2
-  if (!e) e = wgrad<kHidden, kHidden>(m->act[0], m->g2, V, gW(m, 1), gb(m, 1), 0, st);
+  if (!e) e = wgrad<kHidden, kHidden>(m->act[0], m->g2, V, gW(m, 1), gb(m, 1), m->status, st);
   if (!e) e = conv3d_tc<kHidden, kHidden, EPI_SILU_BWD>(m->g2, Wt(m, 1), nullptr, V, nullptr, m->pre[0], m->g1, m->status, st);
   // layer 1 (its input gradient is not needed)
-  if (!e) e = wgrad<kInPad, kHidden>(m->x0, m->g1, V, gW(m, 0), gb(m, 0), 0, st);
+  if (!e) e = wgrad<kInPad, kHidden>(m->x0, m->g1, V, gW(m, 0), gb(m, 0), m->status, st);
   if (!e && loss_out) e = cudaMemcpyAsync(loss_out, m->loss, sizeof(double), cudaMemcpyDeviceToDevice, st);
   if (e) return cuda_fail(m, e, "backward launch");
   m->have_backward = true;
