@@ -2,7 +2,7 @@
 //
 // Activation layout: cells-major, channels-minor, [volume][z][y][x][C] with
 // C a multiple of 16 (BF16 rows of 32 or 64 bytes).  Network outputs are FP32
-// rows of 16 (7 used).  Weights of a layer: [27][C_out][C_in] with
+// rows of 8 (7 used).  Weights of a layer: [27][C_out][C_in] with
 // tap = (dz + 1) * 9 + (dy + 1) * 3 + (dx + 1); the data-gradient pass uses
 // the flipped transpose Wt[tap][C_in][C_out] = W[26 - tap][C_out][C_in].
 #pragma once
@@ -18,7 +18,8 @@ namespace cnn {
 constexpr int kIn = 6;      // real input features
 constexpr int kOut = 7;     // real outputs: D (6) and log error
 constexpr int kInPad = 16;  // stored input channels
-constexpr int kOutPad = 16; // stored output channels
+constexpr int kOutPad = 16; // output channels of the tensor-core layers (their gradient is stored so)
+constexpr int kOutRow = 8;  // stored output channels
 constexpr int kHidden = 32; // hidden channels
 
 // n volumes of nz x ny x nx cells.
@@ -32,7 +33,7 @@ enum { EPI_SILU = 0, EPI_F32 = 1, EPI_SILU_BWD = 2 };
 // out = epi(conv3d(x, W) + b) on the tcgen05 tensor cores (vet_cnn_tc.cu):
 // tiles of 8 x 16 x 2 cells, accumulators in tensor memory.  Epilogues:
 //   EPI_SILU:     pre = acc + b (stored BF16 if pre_out), out = SiLU(pre) BF16
-//   EPI_F32:      out = acc + b, FP32
+//   EPI_F32:      out = acc + b, FP32, the first kOutRow channels
 //   EPI_SILU_BWD: out = acc * SiLU'(pre_in) BF16 (data gradient through the
 //                 previous layer's activation), no bias
 // A bounded wait that gives up ORs 16 into *status (device) and the kernel
@@ -88,7 +89,7 @@ cudaError_t indicator(const float *o, const Vol &V, int B, float thr, float *f_o
 // number (one CTA).
 cudaError_t compact_flags(const unsigned int *flags, int n, int *list, int *count, cudaStream_t st);
 
-// Output rows [cells][16] FP32 -> [n][7][cells] FP32.
+// Output rows [cells][8] FP32 -> [n][7][cells] FP32.
 cudaError_t unpack_outputs(const float *o, const Vol &V, float *o_out, cudaStream_t st);
 
 }  // namespace cnn

@@ -294,15 +294,17 @@ __device__ __forceinline__ void issue_slice(const MmaCommand &c, uint32_t a_hi, 
 template <int C_OUT, int EPI>
 struct Epilogue {
   static constexpr int NC = C_OUT / 2;
+  static_assert(EPI != EPI_F32 || kOutRow % NC == 0, "whole halves are stored");
   long long at, plane;  // element of this thread's first channel in the run's slice 0, and per slice
   bool in;
   float bias[EPI == EPI_SILU_BWD ? 1 : NC];
   int4 p[EPI == EPI_SILU_BWD ? NC / 8 : 1];
   __device__ __forceinline__ void set(const Vol &V, const Run &run, int r, int c0) {
     const int xx = run.tx * TX + (r & 7), y = run.ty * TY + (r >> 3);
-    in = xx < V.nx && y < V.ny;
-    plane = (long long)V.ny * V.nx * C_OUT;
-    at = ((((long long)run.v * V.nz + run.za) * V.ny + y) * V.nx + xx) * C_OUT + c0;
+    constexpr int kRow = EPI == EPI_F32 ? kOutRow : C_OUT;  // stored channels
+    in = xx < V.nx && y < V.ny && c0 < kRow;
+    plane = (long long)V.ny * V.nx * kRow;
+    at = ((((long long)run.v * V.nz + run.za) * V.ny + y) * V.nx + xx) * kRow + c0;
   }
   // the pre-activations the backward epilogue needs, ahead of the wait
   __device__ __forceinline__ void prefetch(const __nv_bfloat16 *__restrict__ pre_in, int j) {

@@ -145,7 +145,7 @@ vet_status ensure_cells(vet_model *m, long long cells, bool train) {
   cudaError_t e = cudaMalloc((void **)&m->x0, n * h16);
   if (!e) e = cudaMalloc((void **)&m->act[0], n * h32);
   if (!e) e = cudaMalloc((void **)&m->act[1], n * h32);
-  if (!e) e = cudaMalloc((void **)&m->o, n * sizeof(float) * cnn::kOutPad);
+  if (!e) e = cudaMalloc((void **)&m->o, n * sizeof(float) * cnn::kOutRow);
   if (!e) e = cudaMalloc((void **)&m->r, n * sizeof(float));
   if (!e && want_train) {
     e = cudaMalloc((void **)&m->act[2], n * h32);

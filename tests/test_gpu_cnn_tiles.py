@@ -60,3 +60,38 @@ def _reference(params, x, f_ref):
     loss = (d * d).mean() + 0.01 * ((a[:, 6] - target) ** 2).mean()
     loss.backward()
     return a.detach().numpy(), [(W.grad.numpy(), b.grad.numpy()) for W, b in P], float(loss.detach())
+
+
+@pytest.mark.parametrize("B", [1, 3, 32, 33])
+def test_features_block_edges(B):
+    """Block statistics on both sides of the 32-cell edge where the block's
+    indices are found another way, and of blocks of equal cells."""
+    rng = np.random.default_rng(B)
+    shape = (B, 2 * B, B)
+    kappa, S, E = _fields(rng, 2, shape)
+    kappa[1, :, :B] = 3.7  # one uniform block: standard deviation 0
+    h = 0.25
+    model = vet.Model()
+    feat = torch.empty(2 * 6 * kappa[0].size, device="cuda")
+    model.features(shape, B, h, _dev(kappa), _dev(S), _dev(E), nvol=2, feat_out=feat)
+    got = feat.cpu().numpy().reshape(2, 6, *shape)
+    for v in range(2):
+        ref = cnn.features(kappa[v], S[v], E[v], h, B)
+        assert np.abs(got[v] - ref.reshape(got[v].shape)).max() < 2e-5
+    assert np.abs(got[1, 5, :, :B]).max() == 0.0
+
+
+def test_features_of_infinite_fields():
+    """An infinite opacity or source reaches the features as it does in plain
+    sums: the block's mean depth, the volume's mean source."""
+    shape, B = (4, 4, 8), 4
+    kappa, S, E = (np.full((1, *shape), x, np.float32) for x in (2.0, 3.0, 5.0))
+    kappa[0, 1, 2, 1] = np.inf
+    S[0, 3, 3, 7] = np.inf
+    model = vet.Model()
+    feat = torch.empty(6 * S.size, device="cuda")
+    model.features(shape, B, 1.0, _dev(kappa), _dev(S), _dev(E), feat_out=feat)
+    got = feat.cpu().numpy().reshape(6, *shape)
+    assert np.isposinf(got[1, 1, 2, 1]) and np.isposinf(got[4, :, :, :4]).all()
+    assert np.isfinite(got[4, :, :, 4:]).all() and np.isfinite(got[3]).all()
+    assert np.isneginf(np.delete(got[2].ravel(), 127)).all()
