@@ -46,7 +46,8 @@ struct vet_ctx {
   long long spin = 0;            // polls per device-side wait
   void *d_stage = nullptr;       // staging of host-pointer arguments
   size_t stage_bytes = 0;
-  vet::TailSplit split;          // scratch of the cell pass's tail split (none: split.nsm = 0)
+  bool want_split = true;        // lone grids: split the cell pass to fill the SMs
+  vet::TailSplit split;          // scratch of the cell pass's split (none: split.nsm = 0)
   long long cell_segs = 0, face_segs = 0;
   int ob[9] = {0};                // octant ranges of the internal direction order
   int face_group = vet::kFaceGroup;  // directions per face-pass item (tunable)
@@ -72,6 +73,8 @@ vet_status cuda_err(vet_ctx *c, cudaError_t e, const char *what) {
   return set_err(c, e == cudaErrorMemoryAllocation ? VET_ENOMEM : VET_ECUDA,
                  std::string(what) + ": " + cudaGetErrorString(e));
 }
+
+size_t round256(size_t x) { return (x + 255) & ~size_t(255); }
 
 // Switches to the context's device for the duration of a call.
 struct DeviceGuard {
@@ -103,8 +106,6 @@ void free_ctx(vet_ctx *c) {
   cudaFree(c->d_bnd);
   cudaFree(c->d_status);
   cudaFree(c->d_stage);
-  cudaFree(c->split.part);
-  cudaFree(c->split.count);
   delete c;
 }
 
@@ -175,39 +176,26 @@ vet_status build_schedule(vet_ctx *c, int group) {
   return VET_OK;
 }
 
-// Scratch of the paired cell pass's tail split for the whole grid (the
-// largest plan over the direction tiles the tuning can pick); the split is
-// left off when the pass is not paired or the plan does not split.
-vet_status enable_tail_split(vet_ctx *c) {
-  if (!c->dims.paired || c->split.part) return VET_OK;
+// The paired cell pass's split for the whole grid (the largest plan over the
+// direction tiles the tuning can pick): its scratch (part) and counters lie
+// behind the face intensities, in their allocation.  No scratch where the
+// pass is not paired or no plan splits (the trace's splits need none); off
+// for grids of a batch, whose closures share the GPU: a lone grid's last
+// wave leaves SMs idle, a batch's does not.
+vet::TailPlan split_plan(vet_ctx *c) {
+  vet::TailPlan best;
   int nsm = 0;
+  if (!c->want_split || !c->dims.paired) return best;
   if (cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, c->cfg.device) != cudaSuccess) {
     cudaGetLastError();
-    return VET_OK;
+    return best;
   }
-  vet::TailPlan best;
   for (int dt = 2; dt <= vet::kMaxTune; dt += 2) {
-    const vet::TailPlan p = vet::plan_tail_split(c->grid.block, c->nblk, nsm, (c->N + dt - 1) / dt);
+    const vet::TailPlan p = vet::plan_tail_split(c->grid.block, c->nblk, nsm, c->N, dt);
     if (p.part_bytes > best.part_bytes) best = p;
   }
   c->split.nsm = nsm;
-  if (best.k <= 1) return VET_OK;  // trace-mode splits need no scratch
-  cudaError_t e;
-  if ((e = cudaMalloc((void **)&c->split.part, best.part_bytes))) return cuda_err(c, e, "cudaMalloc(tail split)");
-  if ((e = cudaMalloc((void **)&c->split.count, sizeof(int) * best.slots)))
-    return cuda_err(c, e, "cudaMalloc(tail split counts)");
-  if ((e = cudaMemset(c->split.count, 0, sizeof(int) * best.slots))) return cuda_err(c, e, "cudaMemset(tail split)");
-  c->split.part_bytes = best.part_bytes;
-  c->split.slots = best.slots;
-  return VET_OK;
-}
-
-// Off for grids of a batch, whose closures share the GPU: a lone grid's last
-// wave leaves SMs idle, a batch's does not.
-void disable_tail_split(vet_ctx *c) {
-  cudaFree(c->split.part);
-  cudaFree(c->split.count);
-  c->split = vet::TailSplit();
+  return best;
 }
 
 template <typename R>
@@ -276,9 +264,19 @@ vet_status build_context(vet_ctx *c) {
   c->dims.fstride = vet::face_stride_elems<R>(B);
   const size_t face_elems = (size_t)N * c->nblk * 3 * c->dims.fstride;
   if ((e = cudaMalloc(&c->d_tpl, tpl.size()))) return cuda_err(c, e, "cudaMalloc(templates)");
-  if ((e = cudaMalloc(&c->d_faces, sizeof(R) * face_elems))) return cuda_err(c, e, "cudaMalloc(face intensities)");
+  // faces, then the split's counters and scratch
+  const vet::TailPlan plan = split_plan(c);
+  const size_t face_bytes = round256(sizeof(R) * face_elems), count_bytes = round256(sizeof(int) * plan.slots);
+  if ((e = cudaMalloc(&c->d_faces, face_bytes + count_bytes + plan.part_bytes)))
+    return cuda_err(c, e, "cudaMalloc(face intensities)");
   // the padding row and column of every stored face stay zero for good
-  if ((e = cudaMemset(c->d_faces, 0, sizeof(R) * face_elems))) return cuda_err(c, e, "cudaMemset(face intensities)");
+  if ((e = cudaMemset(c->d_faces, 0, face_bytes + count_bytes))) return cuda_err(c, e, "cudaMemset(face intensities)");
+  if (plan.k > 1) {
+    c->split.count = (int *)((char *)c->d_faces + face_bytes);
+    c->split.slots = plan.slots;
+    c->split.part = (float *)((char *)c->d_faces + face_bytes + count_bytes);
+    c->split.part_bytes = plan.part_bytes;
+  }
   if ((e = cudaMalloc(&c->d_emax, 8))) return cuda_err(c, e, "cudaMalloc(emax)");
   if ((e = cudaMalloc(&c->d_E, sizeof(R) * c->dims.ncell))) return cuda_err(c, e, "cudaMalloc(E)");
   if ((e = cudaMalloc(&c->d_coef, sizeof(R) * coef.size()))) return cuda_err(c, e, "cudaMalloc(coef)");
@@ -315,15 +313,19 @@ vet_status build_context(vet_ctx *c) {
   if ((e = cudaMemcpy(c->d_coef, coef.data(), sizeof(R) * coef.size(), cudaMemcpyHostToDevice)))
     return cuda_err(c, e, "upload coefficients");
   if (c->fp64) {
-    std::vector<double> tab(vet::kExp64TableDoubles);
-    vet::exp64_fill_table(tab.data());
+    // computed once per process: 1 ms of long double functions on Arm
+    static const std::vector<double> tab = [] {
+      std::vector<double> t(vet::kExp64TableDoubles);
+      vet::exp64_fill_table(t.data());
+      return t;
+    }();
     if ((e = cudaMalloc((void **)&c->d_exp64, sizeof(double) * tab.size()))) return cuda_err(c, e, "cudaMalloc(exp table)");
     if ((e = cudaMemcpy(c->d_exp64, tab.data(), sizeof(double) * tab.size(), cudaMemcpyHostToDevice)))
       return cuda_err(c, e, "upload exp table");
     c->dims.exp64 = c->d_exp64;
   }
   if ((e = vet::prepare_kernels())) return cuda_err(c, e, "cudaFuncSetAttribute");
-  return enable_tail_split(c);
+  return VET_OK;
 }
 
 bool is_device_ptr(const void *p) {
@@ -366,8 +368,6 @@ vet_status reserve_stage(vet_ctx *c, size_t bytes) {
   c->stage_bytes = bytes;
   return VET_OK;
 }
-
-size_t round256(size_t x) { return (x + 255) & ~size_t(255); }
 
 template <typename R>
 vet_status check_ctx(vet_ctx *c, bool want_fp64) {
@@ -620,7 +620,7 @@ vet_status vet::exact_on_blocks(vet_ctx *c, const float *kappa, const float *S, 
   return VET_OK;
 }
 
-VET_API vet_status vet_create(vet_ctx **out, const vet_grid *grid, const vet_config *cfg) {
+static vet_status create_context(vet_ctx **out, const vet_grid *grid, const vet_config *cfg, bool split) {
   if (!out) return set_err(nullptr, VET_EINVAL, "out is NULL");
   *out = nullptr;
   if (!grid || !cfg) return set_err(nullptr, VET_EINVAL, "grid and cfg are required");
@@ -651,6 +651,7 @@ VET_API vet_status vet_create(vet_ctx **out, const vet_grid *grid, const vet_con
   if (!c) return set_err(nullptr, VET_ENOMEM, "host allocation failed");
   c->grid = g;
   c->cfg = *cfg;
+  c->want_split = split;
   c->spin = cfg->spin_limit > 0 ? cfg->spin_limit : (1LL << 22);
   c->fp64 = fp64;
   c->N = 12 * cfg->nside * cfg->nside;
@@ -683,6 +684,10 @@ VET_API vet_status vet_create(vet_ctx **out, const vet_grid *grid, const vet_con
   }
   *out = c;
   return VET_OK;
+}
+
+VET_API vet_status vet_create(vet_ctx **out, const vet_grid *grid, const vet_config *cfg) {
+  return create_context(out, grid, cfg, true);
 }
 
 VET_API vet_status vet_destroy(vet_ctx *ctx) {
@@ -1058,13 +1063,12 @@ VET_API vet_status vet_batch_create(vet_batch **out, int n, const vet_grid *grid
       return set_err(nullptr, VET_EINVAL, "a batch holds FP32 grids on one device");
     }
     vet_ctx *c = nullptr;
-    vet_status st = vet_create(&c, &grids[i], &cfgs[i]);
+    vet_status st = create_context(&c, &grids[i], &cfgs[i], false);
     if (st != VET_OK) {
       g_create_err = "grid " + std::to_string(i) + ": " + g_create_err;
       free_batch(b);
       return st;
     }
-    disable_tail_split(c);
     b->ctx.push_back(c);
   }
   DeviceGuard dg(b->device);

@@ -195,13 +195,24 @@ cudaError_t launch_face_level(const GridDims &g, const R *kappa, const R *S, con
 // ([slot][share][28][threads] floats) and the last share of a slot to
 // finish (counted in `count`, which it resets) adds the others' and writes
 // the outputs.
+//
+// A grid of fewer CTAs than one wave (total < wave) is split whole, every CTA
+// into as many shares as fill the wave, so that a small grid's cell pass does
+// not take one CTA's time on a part of the SMs.  Its results are the unsplit
+// pass's bits (a small grid's closure equals the same grid's in a batch, or
+// its blocks' in the learned closure's fallback): the shares store each
+// antipodal pair's sum and difference of intensities, and the last share of
+// an item adds them in the unsplit order (`ordered`).
 struct TailPlan {
   int nfull = 0;          // CTAs that run whole (total - r)
   int k = 1;              // shares per split work item (1: no split)
   int slots = 0;          // r
   size_t part_bytes = 0;  // scratch the moments of the shares need
+  bool ordered = false;   // total < wave: per-pair values instead of partial moments
 };
-TailPlan plan_tail_split(int B, int nblk, int nsm, int ntiles);
+TailPlan plan_tail_split(int B, int nblk, int nsm, int ndir, int dir_tile);
+// Largest scratch of an ordered split (beyond: the grid runs unsplit).
+constexpr size_t kOrderedSplitMax = (size_t)128 << 20;
 
 // One grid of a merged launch of the paired FP32 cell pass (the batched
 // closure): what a single grid's launch passes as arguments.  M_out null:

@@ -997,7 +997,8 @@ static_assert(offsetof(TplHead<float>, sgn) == 16 && offsetof(TplHead<float>, ex
                   offsetof(TplHead<float>, mirror) == 32 && offsetof(TplHead<float>, cp) % 16 == 0,
               "TplHead<float> layout");
 
-template <int MODE, int BC, bool MERGED>
+// ORDERED (moment modes): every CTA is one share of a work item, see TailPlan.
+template <int MODE, int BC, bool MERGED, bool ORDERED = false>
 __global__ void __launch_bounds__(pair_threads(BC), pair_min_ctas(BC))
     cell_pair_kernel(GridDims g_arg, int parts, int dt, int nstage, const float *__restrict__ kappa_arg,
                      const float *__restrict__ S_arg, const unsigned char *__restrict__ tpl_arg,
@@ -1205,6 +1206,13 @@ __global__ void __launch_bounds__(pair_threads(BC), pair_min_ctas(BC))
         I_out[(long long)hb.w * g.ncell + gc2] = m1.y;
         I_out[(long long)hb.w * g.ncell + gc1] = m2.x;
         I_out[(long long)ha.w * g.ncell + gc2] = m2.y;
+      } else if (ORDERED) {
+        // this pair's place in the item's list: pairs are consecutive in the order
+        const int pair = ((tile0 + t) * dt + j) >> 1;
+        float2 *dst = reinterpret_cast<float2 *>(split_part) +
+                      ((size_t)slot * (g.ndir >> 1) + pair) * 2 * NT + threadIdx.x;
+        __stcg(dst, __fadd2_rn(m1, m2));
+        if (kWantF) __stcg(dst + NT, __fadd2_rn(m1, neg2(m2)));
       } else {
         // E and P take I(d) + I(-d), F takes I(d) - I(-d), with the primary
         // direction's coefficient pairs
@@ -1226,7 +1234,7 @@ __global__ void __launch_bounds__(pair_threads(BC), pair_min_ctas(BC))
         mom[9] = __ffma2_rn(make_float2(c89.z, c89.w), sum, mom[9]);
       }
     }
-    if (MODE != 1) {  // the tile's plain partial sums into the compensated ones
+    if (MODE != 1 && !ORDERED) {  // the tile's plain partial sums into the compensated ones
       const float2 one = make_float2(1.f, 1.f);
       kahan2(mom[0], nc[0], one, pk[0]);
       kahan2(mom[4], nc[1], one, pk[1]);
@@ -1248,7 +1256,51 @@ __global__ void __launch_bounds__(pair_threads(BC), pair_min_ctas(BC))
     for (int t = consumed; t < issued; ++t)
       if (!mbar_wait_sleep(full_s + 8 * (t % nstage), (uint32_t)((t / nstage) & 1), kDrainPolls)) atomicOr(status, 8);
   }
-  if (MODE != 1 && slot >= 0) {
+  if (MODE != 1 && ORDERED) {
+    // the share that finishes last adds every pair's values, tile by tile as
+    // the unsplit pass does, and writes the outputs
+    __shared__ int s_last;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) s_last = atomicAdd(split_count + slot, 1) == ksplit - 1;
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    const float2 one = make_float2(1.f, 1.f);
+    const float2 *src = reinterpret_cast<const float2 *>(split_part) + (size_t)slot * (g.ndir >> 1) * 2 * NT + threadIdx.x;
+    for (int d0 = 0; d0 < g.ndir; d0 += dt) {
+      const int nd = min(dt, g.ndir - d0);
+#pragma unroll 4
+      for (int j = 0; j < nd; j += 2) {
+        const int pair = (d0 + j) >> 1;
+        const float2 sum = __ldcg(src + (size_t)pair * 2 * NT);
+        const float2 dif = kWantF ? __ldcg(src + (size_t)pair * 2 * NT + NT) : one;
+        const int v = ord_smem ? s_ord[d0 + j] : order[d0 + j];
+        const float4 *cp = reinterpret_cast<const float4 *>(tpl_g + (size_t)order_dir(v) * TL.bytes +
+                                                            offsetof(TplHead<float>, cp));
+        const float4 c01 = __ldg(cp), c23 = __ldg(cp + 1), c45 = __ldg(cp + 2), c67 = __ldg(cp + 3), c89 = __ldg(cp + 4);
+        pk[0] = __ffma2_rn(make_float2(c01.x, c01.y), sum, pk[0]);
+        if (kWantF) {
+          mom[1] = __ffma2_rn(make_float2(c01.z, c01.w), dif, mom[1]);
+          mom[2] = __ffma2_rn(make_float2(c23.x, c23.y), dif, mom[2]);
+          mom[3] = __ffma2_rn(make_float2(c23.z, c23.w), dif, mom[3]);
+        }
+        pk[1] = __ffma2_rn(make_float2(c45.x, c45.y), sum, pk[1]);
+        pk[2] = __ffma2_rn(make_float2(c45.z, c45.w), sum, pk[2]);
+        pk[3] = __ffma2_rn(make_float2(c67.x, c67.y), sum, pk[3]);
+        mom[7] = __ffma2_rn(make_float2(c67.z, c67.w), sum, mom[7]);
+        mom[8] = __ffma2_rn(make_float2(c89.x, c89.y), sum, mom[8]);
+        mom[9] = __ffma2_rn(make_float2(c89.z, c89.w), sum, mom[9]);
+      }
+      kahan2(mom[0], nc[0], one, pk[0]);
+      kahan2(mom[4], nc[1], one, pk[1]);
+      kahan2(mom[5], nc[2], one, pk[2]);
+      kahan2(mom[6], nc[3], one, pk[3]);
+#pragma unroll
+      for (int m = 0; m < 4; ++m) pk[m] = make_float2(0.f, 0.f);
+    }
+    if (threadIdx.x == 0) split_count[slot] = 0;  // ready for the next call
+  } else if (MODE != 1 && slot >= 0) {
     // one share of a split work item: its partial sums go to the slot's
     // scratch, and the share that finishes last adds the others' (the
     // compensated sums as compensated sums) and writes the outputs
@@ -1748,13 +1800,26 @@ inline void pair_staging(int B, int want, int &dt, int &nstage) {
 
 }  // namespace
 
-TailPlan plan_tail_split(int B, int nblk, int nsm, int ntiles) {
+TailPlan plan_tail_split(int B, int nblk, int nsm, int ndir, int dir_tile) {
   TailPlan p;
   if (B != 8 && B != 16) return p;
-  const int parts = B * B * B / 2 / pair_threads(B), total = nblk * parts;
+  const int parts = B * B * B / 2 / pair_threads(B), total = nblk * parts, ntiles = (ndir + dir_tile - 1) / dir_tile;
   p.nfull = total;
   const int wave = nsm * pair_min_ctas(B);
-  if (nsm <= 0 || total < wave) return p;
+  if (nsm <= 0) return p;
+  if (total < wave) {
+    // whole shares per item that still fit one wave.  32^3 cells in 8^3 blocks, 48
+    // directions (64 CTAs on 608 places, 6 shares): closure 137 -> 72 us
+    const int k = std::min(ntiles, wave / total);
+    const size_t bytes = (size_t)total * (ndir / 2) * 4 * pair_threads(B) * sizeof(float);
+    if (k < 2 || bytes > kOrderedSplitMax) return p;
+    p.k = k;
+    p.nfull = 0;
+    p.slots = total;
+    p.part_bytes = bytes;
+    p.ordered = true;
+    return p;
+  }
   const int r = total % wave;
   if (r == 0) return p;
   // tail time in CTA times, with each share's own start (tile load, first
@@ -1790,7 +1855,7 @@ void pair_launch(const GridDims &g, const float *kappa, const float *S, const un
   TailPlan tp;
   tp.nfull = nblk * parts;
   if (split && !block_list) {
-    const TailPlan q = plan_tail_split(BC, nblk, split->nsm, (g.ndir + dt - 1) / dt);
+    const TailPlan q = plan_tail_split(BC, nblk, split->nsm, g.ndir, dt);
     const bool room = MODE == 1 || (split->part && split->count && q.part_bytes <= split->part_bytes &&
                                     q.slots <= split->slots);
     if (q.k > 1 && room) tp = q;
@@ -1806,9 +1871,12 @@ void pair_launch(const GridDims &g, const float *kappa, const float *S, const un
   cfg.stream = st;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  cudaLaunchKernelEx(&cfg, cell_pair_kernel<MODE, BC, false>, g, parts, dt, nstage, kappa, S, tpl, order, faces, bnd, I_out,
-                     M_out, E_out, f_out, emax_bits, spin, status, block_list, tp.nfull, tp.k,
-                     split ? split->part : nullptr, split ? split->count : nullptr, nullptr, nullptr);
+  auto *kernel = cell_pair_kernel<MODE, BC, false>;
+  if constexpr (MODE != 1)
+    if (tp.ordered) kernel = cell_pair_kernel<MODE, BC, false, true>;
+  cudaLaunchKernelEx(&cfg, kernel, g, parts, dt, nstage, kappa, S, tpl, order, faces, bnd, I_out, M_out, E_out, f_out,
+                     emax_bits, spin, status, block_list, tp.nfull, tp.k, split ? split->part : nullptr,
+                     split ? split->count : nullptr, nullptr, nullptr);
 }
 
 // One launch of the paired cell pass over the blocks of several grids of
@@ -1851,6 +1919,8 @@ cudaError_t set_smem_attrs() {
                         (const void *)cell_pair_kernel<2, 8, false>,  (const void *)cell_pair_kernel<2, 16, false>,
                         (const void *)cell_pair_kernel<0, 8, true>,   (const void *)cell_pair_kernel<0, 16, true>,
                         (const void *)cell_pair_kernel<2, 8, true>,   (const void *)cell_pair_kernel<2, 16, true>,
+                        (const void *)cell_pair_kernel<0, 8, false, true>, (const void *)cell_pair_kernel<0, 16, false, true>,
+                        (const void *)cell_pair_kernel<2, 8, false, true>, (const void *)cell_pair_kernel<2, 16, false, true>,
                         (const void *)face_pair_kernel<8>,            (const void *)face_pair_kernel<16>};
   for (const void *f : pfns) {  // less their static shared memory
     cudaFuncAttributes fa;
