@@ -1654,23 +1654,41 @@ __global__ void floor_fix_blocks_kernel(const GridDims g, const int *__restrict_
   }
 }
 
+// Sum of FP32 values as three floats: two exact sums (TwoSum, Knuth) carry
+// their roundings on, the third collects what is below 2^-48 of the total, so
+// the result is within an FP64 rounding of the exact sum.  13 FP32 additions a
+// value, where an FP64 addition and the conversion before it hold the SM's
+// two-lane FP64 pipe for 32 clocks per warp.
+struct FloatSum {
+  float a = 0.f, b = 0.f, c = 0.f;
+  static __device__ __forceinline__ float two_sum(float &s, float x) {  // s += x, returns the rounding
+    const float r = __fadd_rn(s, x), t = __fsub_rn(r, s);
+    const float e = __fadd_rn(__fsub_rn(s, __fsub_rn(r, t)), __fsub_rn(x, t));
+    s = r;
+    return e;
+  }
+  __device__ __forceinline__ void add(float x) { c = __fadd_rn(c, two_sum(b, two_sum(a, x))); }
+  __device__ __forceinline__ double value() const { return (double)a + ((double)b + (double)c); }
+};
+
 // Quadratures of stored intensities (Eqs. 10-12, c = 1): M[m][c] =
 // sum_k coef[k][m] I[k][c].  HBM-bound (4 bytes of I per 10 FMAs): one thread
 // per V consecutive cells with V-wide loads, directions unrolled by 4 so that
 // several loads are in flight, coefficients of a chunk of 64 directions in
-// shared memory.  The FP32 version keeps pairs of cells in packed f32x2
-// accumulators against (c, c) coefficient pairs.
+// shared memory.  With E64 the sum of I goes through FloatSum and V is 2 (96 x
+// 64 x 48 cells, 192 directions, L2 flushed: 234 -> 72 us against FP64 additions of
+// every value; without E64 79 -> 58 us by two cells a thread).
 template <typename R, int V, bool WITH_E64>
 __global__ void __launch_bounds__(256, 4) moments_kernel(long long ncell, int ndir, const R *__restrict__ I,
                                                       const R *__restrict__ coef, R *__restrict__ M,
                                                       double *__restrict__ E64, double w64) {
+  static_assert(!WITH_E64 || sizeof(R) == 4, "E64 is the FP32 path's");
   __shared__ R cs[64][10];
   const long long c = (blockIdx.x * (long long)blockDim.x + threadIdx.x) * V;
   R acc[V][10];
-  double e64[V];  // E in FP64: the weights are equal, so the sum of I times w
+  FloatSum fs[WITH_E64 ? V : 1];  // E in FP64: the weights are equal, so the sum of I times w
 #pragma unroll
   for (int v = 0; v < V; ++v) {
-    e64[v] = 0.0;
 #pragma unroll
     for (int m = 0; m < 10; ++m) acc[v][m] = R(0);
   }
@@ -1684,12 +1702,12 @@ __global__ void __launch_bounds__(256, 4) moments_kernel(long long ncell, int nd
       for (int k = 0; k < nk; ++k) {
         R v[V];
         const R *src = I + (long long)(k0 + k) * ncell + c;
-        if (V == 4) {
+        if constexpr (V == 4) {
           const float4 q = *reinterpret_cast<const float4 *>(src);
-          v[0] = q.x; v[1] = q.y; v[V > 2 ? 2 : 0] = q.z; v[V > 3 ? 3 : 0] = q.w;
-        } else if (V == 2) {
-          const double2 q = *reinterpret_cast<const double2 *>(src);
-          v[0] = q.x; v[V > 1 ? 1 : 0] = q.y;
+          v[0] = q.x; v[1] = q.y; v[2] = q.z; v[3] = q.w;
+        } else if constexpr (V == 2) {
+          const vec2_t<R> q = *reinterpret_cast<const vec2_t<R> *>(src);
+          v[0] = q.x; v[1] = q.y;
         } else {
           v[0] = src[0];
         }
@@ -1701,7 +1719,7 @@ __global__ void __launch_bounds__(256, 4) moments_kernel(long long ncell, int nd
         }
         if constexpr (WITH_E64) {
 #pragma unroll
-          for (int j = 0; j < V; ++j) e64[j] += (double)v[j];
+          for (int j = 0; j < V; ++j) fs[j].add(v[j]);
         }
       }
     }
@@ -1709,17 +1727,25 @@ __global__ void __launch_bounds__(256, 4) moments_kernel(long long ncell, int nd
   if (c >= ncell) return;
   if constexpr (WITH_E64) {
 #pragma unroll
-    for (int j = 0; j < V; ++j)
-      if (c + j < ncell) E64[c + j] = w64 * e64[j];
+    for (int j = 0; j < V; ++j) {
+      double e = fs[j].value();
+      if (!isfinite(e)) {  // an infinity, a NaN or a sum beyond FP32's range
+        e = 0.0;
+        for (int k = 0; k < ndir; ++k) e += (double)I[(long long)k * ncell + c + j];
+      }
+      E64[c + j] = w64 * e;
+    }
   }
 #pragma unroll
   for (int m = 0; m < 10; ++m) {
     R *dst = M + m * ncell + c;
-    if (V == 4) {
-      *reinterpret_cast<float4 *>(dst) = make_float4(acc[0][m], acc[V > 1 ? 1 : 0][m], acc[V > 2 ? 2 : 0][m],
-                                                     acc[V > 3 ? 3 : 0][m]);
-    } else if (V == 2) {
-      *reinterpret_cast<double2 *>(dst) = make_double2(acc[0][m], acc[V > 1 ? 1 : 0][m]);
+    if constexpr (V == 4) {
+      *reinterpret_cast<float4 *>(dst) = make_float4(acc[0][m], acc[1][m], acc[2][m], acc[3][m]);
+    } else if constexpr (V == 2) {
+      vec2_t<R> q;
+      q.x = acc[0][m];
+      q.y = acc[1][m];
+      *reinterpret_cast<vec2_t<R> *>(dst) = q;
     } else {
       dst[0] = acc[0][m];
     }
@@ -2038,23 +2064,32 @@ template <typename R>
 cudaError_t launch_moments(long long ncell, int ndir, const R *I, const R *coef, R *M_out, cudaStream_t st,
                            double *E64, double w64) {
   const int threads = 256;
-  // vector loads need every direction's row to start 16-byte aligned
-  constexpr int VW = 16 / (int)sizeof(R);
-  const bool vec = ncell % VW == 0 && (reinterpret_cast<uintptr_t>(I) & 15) == 0 &&
-                   (reinterpret_cast<uintptr_t>(M_out) & 15) == 0;
-  const long long per = vec ? VW : 1;
-  const long long blocks = ((ncell + per - 1) / per + threads - 1) / threads;
+  // vector loads need every direction's row to start aligned to them
+  auto fits = [&](int v) {
+    return ncell % v == 0 && ((reinterpret_cast<uintptr_t>(I) | reinterpret_cast<uintptr_t>(M_out)) & (v * sizeof(R) - 1)) == 0;
+  };
+  // four FP32 cells a thread where that still gives the SMs enough loads in
+  // flight (threads of 152 SMs x 1024), else two; two with E64 (registers)
+  int v = 1;
+  if (sizeof(R) == 4 && !E64 && fits(4) && ncell >= 4LL * 152 * 1024) v = 4;
+  else if (fits(2)) v = 2;
+  const long long blocks = ((ncell + v - 1) / v + threads - 1) / threads;
   if (blocks < 1) return cudaSuccess;
-  if (E64) {
-    if (vec)
-      moments_kernel<R, VW, true><<<(unsigned)blocks, threads, 0, st>>>(ncell, ndir, I, coef, M_out, E64, w64);
-    else
-      moments_kernel<R, 1, true><<<(unsigned)blocks, threads, 0, st>>>(ncell, ndir, I, coef, M_out, E64, w64);
-  } else if (vec) {
-    moments_kernel<R, VW, false><<<(unsigned)blocks, threads, 0, st>>>(ncell, ndir, I, coef, M_out, E64, w64);
-  } else {
-    moments_kernel<R, 1, false><<<(unsigned)blocks, threads, 0, st>>>(ncell, ndir, I, coef, M_out, E64, w64);
+#define VET_MOM(V, WE) moments_kernel<R, V, WE><<<(unsigned)blocks, threads, 0, st>>>(ncell, ndir, I, coef, M_out, E64, w64)
+  if constexpr (sizeof(R) == 4) {
+    if (E64) {
+      if (v == 2) VET_MOM(2, true);
+      else VET_MOM(1, true);
+      return cudaGetLastError();
+    }
+    if (v == 4) {
+      VET_MOM(4, false);
+      return cudaGetLastError();
+    }
   }
+  if (v == 2) VET_MOM(2, false);
+  else VET_MOM(1, false);
+#undef VET_MOM
   return cudaGetLastError();
 }
 
