@@ -35,7 +35,7 @@ struct vet_ctx {
   void *d_tpl = nullptr;         // N template blobs, internal (octant-sorted) order
   FaceItem *d_items = nullptr;
   int *d_cell_order = nullptr;   // cell-pass visiting order of internal directions
-  uint16_t *d_node_order = nullptr;  // paired face pass: face nodes by ray length (dims.node_order)
+  void *d_rec = nullptr;         // ray records: nodes, then cells (dims.node_rec, dims.cell_rec)
   double *d_exp64 = nullptr;     // FP64: tables of the segment weight
   void *d_faces = nullptr;       // [N][blocks][3][fstride], upwind frame, padded
   void *d_emax = nullptr;        // 8 bytes: bit pattern of max E (nonnegative)
@@ -97,7 +97,7 @@ void free_ctx(vet_ctx *c) {
   cudaFree(c->d_tpl);
   cudaFree(c->d_items);
   cudaFree(c->d_cell_order);
-  cudaFree(c->d_node_order);
+  cudaFree(c->d_rec);
   cudaFree(c->d_exp64);
   cudaFree(c->d_faces);
   cudaFree(c->d_emax);
@@ -304,11 +304,21 @@ vet_status build_context(vet_ctx *c) {
     std::vector<uint16_t> nord((size_t)N * 6 * NN);
     for (int i = 0; i < N; ++i)
       vet::geom::node_order<R>(tpl.data() + (size_t)i * tbytes, B, nord.data() + (size_t)i * 6 * NN);
-    if ((e = cudaMalloc((void **)&c->d_node_order, sizeof(uint16_t) * nord.size())))
-      return cuda_err(c, e, "cudaMalloc(node order)");
-    if ((e = cudaMemcpy(c->d_node_order, nord.data(), sizeof(uint16_t) * nord.size(), cudaMemcpyHostToDevice)))
+    const size_t node_bytes = round256(sizeof(uint2) * vet::node_rec_count(N, B));
+    const size_t cell_bytes = round256(sizeof(uint32_t) * vet::cell_rec_count(N, B));
+    // the order's upload goes behind the records, in their allocation
+    if ((e = cudaMalloc(&c->d_rec, node_bytes + cell_bytes + sizeof(uint16_t) * nord.size())))
+      return cuda_err(c, e, "cudaMalloc(ray records)");
+    uint2 *node_rec = (uint2 *)c->d_rec;
+    uint32_t *cell_rec = (uint32_t *)((char *)c->d_rec + node_bytes);
+    uint16_t *order_dev = (uint16_t *)((char *)cell_rec + cell_bytes);
+    if ((e = cudaMemcpy(order_dev, nord.data(), sizeof(uint16_t) * nord.size(), cudaMemcpyHostToDevice)))
       return cuda_err(c, e, "upload node order");
-    c->dims.node_order = c->d_node_order;
+    if ((e = vet::launch_ray_records<R>(c->dims, (const unsigned char *)c->d_tpl, order_dev, cell_rec, node_rec, nullptr)) ||
+        (e = cudaStreamSynchronize(nullptr)))
+      return cuda_err(c, e, "ray records");
+    c->dims.node_rec = node_rec;
+    c->dims.cell_rec = cell_rec;
   }
   if ((e = cudaMemcpy(c->d_coef, coef.data(), sizeof(R) * coef.size(), cudaMemcpyHostToDevice)))
     return cuda_err(c, e, "upload coefficients");

@@ -129,13 +129,42 @@ struct GridDims {
   int dir_tile;       // directions per cell-pass tile (0: default)
   int paired;         // 1: the cell order lists antipodal pairs (d, -d), see the paired cell pass
   int face_paired;    // 1: face-pass items are mirrored block pairs, see the paired face pass
-  // face passes: per template (internal order), the (B+1)^2 face nodes of
-  // each face axis by ascending node-ray length, then the node codes of all
-  // three faces merged the same way, [N][6][(B+1)^2] (geom::node_order;
-  // null: row order)
-  const uint16_t *node_order;
+  const uint32_t *cell_rec;  // ray records, see CellRec and NodeRec
+  const uint2 *node_rec;
   const double *exp64;  // FP64 passes: tables of the segment weight (vet_exp64.h)
 };
+
+// Ray records.  Where a ray leaves its block, through which entry of the exit
+// tables, and at which node of the incoming faces it starts depend on the
+// direction and the cell (or face node) alone, not on the block; a table of
+// them, made once per context by ray_records_kernel, replaces the passes' per-ray
+// search of the plane events and its index arithmetic.
+//   cells: [N][B^3] words (internal direction order; cells in cell_rec_index order)
+//   nodes: [N][6][(B+1)^2] words pairs: the nodes of each face axis, then of the
+//     three faces merged, each in geom::node_order's order (null: row order)
+struct CellRec {
+  uint32_t v;  // exit event index 8 bits, row of the weight table 8, face entry (element of the three faces) 16
+  __host__ __device__ int last() const { return (int)(v & 255u); }
+  __host__ __device__ int row() const { return (int)((v >> 8) & 255u); }
+  __host__ __device__ int face() const { return (int)(v >> 16); }
+};
+struct NodeRec {
+  uint2 v;  // x: exit event index + 1, row, face entry as above; y: start cell in the tile 16 bits, stored node 16
+  __host__ __device__ int last() const { return (int)(v.x & 255u) - 1; }
+  __host__ __device__ int row() const { return (int)((v.x >> 8) & 255u); }
+  __host__ __device__ int face() const { return (int)(v.x >> 16); }
+  __host__ __device__ int start() const { return (int)(v.y & 65535u); }
+  __host__ __device__ int out() const { return (int)(v.y >> 16); }
+};
+// Place of a block's cell in a direction's records: where the edge is a
+// multiple of 4, the 4 x 4 x 2 bricks that the warps of the cell passes take,
+// one after another; else row by row.
+__host__ __device__ inline int cell_rec_index(int B, int x, int y, int z) {
+  if (B % 4 || B % 2) return (z * B + y) * B + x;
+  return (((z >> 1) * (B / 4) + (y >> 2)) * (B / 4) + (x >> 2)) * 32 + (z & 1) * 16 + (y & 3) * 4 + (x & 3);
+}
+inline size_t cell_rec_count(int N, int B) { return (size_t)N * B * B * B; }
+inline size_t node_rec_count(int N, int B) { return (size_t)N * 6 * (B + 1) * (B + 1); }
 
 // Shared-memory kappa/S tiles of a block, in entries of 8 bytes (kappa, S) or,
 // for the FP32 mirrored passes, 16 bytes (kappa, kappa', S, S').  Face pass:
@@ -261,6 +290,12 @@ cudaError_t launch_cell_pass(const GridDims &g, int mode, const R *kappa, const 
 template <typename R>
 cudaError_t launch_floor_fix_blocks(const GridDims &g, const int *block_list, int nlist, const R *E,
                                     const void *emax_bits, double floor_rel, R *f_out, cudaStream_t st);
+
+// The ray records of every direction's template (node_order: device, may be
+// null).
+template <typename R>
+cudaError_t launch_ray_records(const GridDims &g, const unsigned char *tpl, const uint16_t *node_order, uint32_t *cell_rec,
+                               uint2 *node_rec, cudaStream_t st);
 
 // bnd[face][d] <- constant Ib[face][ext(d)] (or 0 when Ib is NULL).
 template <typename R>

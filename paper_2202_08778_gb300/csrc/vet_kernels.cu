@@ -154,20 +154,6 @@ struct Tpl {
         nw(reinterpret_cast<const vec2_t<R> *>(base + L.nw)) {}
 };
 
-// Bilinear interpolation on incoming face ae (Sec. 2.2.5 reading: short
-// characteristics between blocks).  The face is staged in the upwind frame
-// with row stride B + 2 (node B + 1 is zero padding, reached only with weight
-// 0).  lb, lc are the ray's upwind-frame coordinates along the two in-plane
-// axes, kb/kc and wb/wc its exit-table entries (floor and (f, 1-f)).
-template <typename R>
-__device__ __forceinline__ R face_value(const R *__restrict__ fin, int fstride, int B, int ae, int lb, int lc,
-                                        int kb, int kc, vec2_t<R> wb, vec2_t<R> wc) {
-  const int W = B + 2;
-  const int ib = max(lb + kb, 0), ic = max(lc + kc, 0);
-  const R *F = fin + ae * fstride + ib * W + ic;
-  return wb.y * (wc.y * F[0] + wc.x * F[1]) + wb.x * (wc.y * F[W] + wc.x * F[W + 1]);
-}
-
 // ------------------------------------------------ TMA bulk copies + mbarriers
 __device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
@@ -372,8 +358,99 @@ int cell_dir_tile(int B, int want) {
   return dt;
 }
 
+// -------------------------------------------------------------- ray records
+// One direction per block row (y); x over its cells and node entries.
+template <typename R>
+__global__ void __launch_bounds__(256) ray_records_kernel(GridDims g, const unsigned char *__restrict__ tpl_g,
+                                                          const uint16_t *__restrict__ node_order,
+                                                          uint32_t *__restrict__ cell_rec, uint2 *__restrict__ node_rec) {
+  const int B = g.B, W = B + 2, N1 = B + 1, NN = N1 * N1, B3 = B * B * B, d = blockIdx.y;
+  const TplLayout TL = tpl_layout<R>(B);
+  const Tpl<R> T(tpl_g + (size_t)d * TL.bytes, TL);
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < B3 + 6 * NN; i += gridDim.x * blockDim.x) {
+    if (i < B3) {
+      const int x = i % B, y = (i / B) % B, z = i / (B * B);
+      // upwind-frame coordinates; the exit axis ae is the one whose plane
+      // event comes first, (lb, lc) the other two in increasing axis order
+      const int l0 = T.h->sgn[0] > 0 ? x : B - 1 - x;
+      const int l1 = T.h->sgn[1] > 0 ? y : B - 1 - y;
+      const int l2 = T.h->sgn[2] > 0 ? z : B - 1 - z;
+      const int p0 = T.cpos[l0], p1 = T.cpos[B + l1], p2 = T.cpos[2 * B + l2];
+      int last = p0, ae = 0, la = l0, lb = l1, lc = l2;
+      if (p1 < last) { last = p1; ae = 1; la = l1; lb = l0; }
+      if (p2 < last) { last = p2; ae = 2; la = l2; lb = l0; lc = l1; }
+      const int row = (ae * 2) * B + la;
+      const int ib = max(lb + T.ck[row], 0), ic = max(lc + T.ck[row + B], 0);
+      cell_rec[(size_t)d * B3 + cell_rec_index(B, x, y, z)] =
+          (uint32_t)last | (uint32_t)row << 8 | (uint32_t)(ae * g.fstride + ib * W + ic) << 16;
+      continue;
+    }
+    const int k = i - B3;  // entry: k < 3 NN: face k / NN; else the merged order
+    int a, r;
+    if (k < 3 * NN) {
+      a = k / NN;
+      r = node_order ? node_order[(size_t)d * 6 * NN + k] : k - a * NN;
+    } else {
+      const int code = node_order ? node_order[(size_t)d * 6 * NN + k] : k - 3 * NN;
+      a = code / NN;
+      r = code - a * NN;
+    }
+    const int ub = r / N1, uc = r - ub * N1;  // upwind-frame node on the downwind face of axis a
+    // upwind-frame node coordinates (L0, L1, L2): B along the face's axis
+    const int L0 = a == 0 ? B : ub;
+    const int L1 = a == 1 ? B : (a == 0 ? ub : uc);
+    const int L2 = a == 2 ? B : uc;
+    const int p0 = T.npos[L0], p1 = T.npos[N1 + L1], p2 = T.npos[2 * N1 + L2];
+    int last = p0, ae = 0, la = L0, lb = L1, lc = L2;
+    if (p1 < last) { last = p1; ae = 1; la = L1; lb = L0; }
+    if (p2 < last) { last = p2; ae = 2; la = L2; lb = L0; lc = L1; }
+    const int row = (ae * 2) * N1 + la;
+    const int ib = max(lb + T.nk[row], 0), ic = max(lc + T.nk[row + N1], 0);
+    // where last >= 0, every L >= 1 and the start cell is inside the block
+    const TileShape ts = node_tile(B);
+    const int c0 = T.h->sgn[0] > 0 ? L0 - 1 : B - L0;
+    const int c1 = T.h->sgn[1] > 0 ? L1 - 1 : B - L1;
+    const int c2 = T.h->sgn[2] > 0 ? L2 - 1 : B - L2;
+    const int start = last >= 0 ? c0 + ts.sy * c1 + ts.sz * c2 : 0;
+    node_rec[(size_t)d * 6 * NN + k] =
+        make_uint2((uint32_t)(last + 1) | (uint32_t)row << 8 | (uint32_t)(ae * g.fstride + ib * W + ic) << 16,
+                   (uint32_t)start | (uint32_t)(a * g.fstride + ub * W + uc) << 16);
+  }
+}
+
+// Bilinear interpolation at a record's face entry (Sec. 2.2.5 reading: short
+// characteristics between blocks).  The face is staged in the upwind frame
+// with row stride B + 2 (node B + 1 is zero padding, reached only with weight
+// 0); wb/wc are the exit-table weights (f, 1-f).
+template <typename R>
+__device__ __forceinline__ R face_value(const R *__restrict__ F, int W, vec2_t<R> wb, vec2_t<R> wc) {
+  return wb.y * (wc.y * F[0] + wc.x * F[1]) + wb.x * (wc.y * F[W] + wc.x * F[W + 1]);
+}
+
 // ---------------------------------------------------------------- face pass
 constexpr int kFaceThreads = 512;
+
+// The record of the w-th node ray of a face item: the k-th node by length of
+// face ai (or where all three faces are computed, of the three merged), every
+// other face (or direction) of the item taken from its longest ray down, so
+// that a warp that straddles two joins rays of similar length too; j: the
+// ray's direction in the item.
+template <int BC>
+__device__ __forceinline__ NodeRec node_record(const GridDims &g, int dir_begin, int live, int nlive, int w, int &j) {
+  const int NN = BC ? (BC + 1) * (BC + 1) : g.nnode;
+  int e;
+  if (nlive == 3) {
+    j = w / (3 * NN);
+    const int k = w - j * (3 * NN);
+    e = 3 * NN + ((j & 1) ? 3 * NN - 1 - k : k);
+  } else {
+    const int q = w / NN, k = w - q * NN;
+    j = nlive == 1 ? q : q >> 1;
+    const int a = (live >> (2 * (q - j * nlive))) & 3;
+    e = a * NN + ((q & 1) ? NN - 1 - k : k);
+  }
+  return {__ldg(g.node_rec + (size_t)(dir_begin + j) * (6 * NN) + e)};
+}
 
 // Face pass: one CTA per item (a block and up to kFaceGroup directions of one
 // octant at the same wavefront level).  The CTA loads the block's kappa/S
@@ -440,38 +517,13 @@ __global__ void __launch_bounds__(kFaceThreads, sizeof(R) == 8 ? 2 : 3)
     const int wr = w0 + ((int)threadIdx.x & 31);
     const bool act = wr < total;
     const int w = act ? wr : total - 1;
-    // w = (j * nlive + ai) * NN + r; NN is a compile-time constant for a
-    // templated block edge, and q / nlive (q < 3 * kMaxTune, nlive <= 3) is
-    // a multiply-shift instead of a runtime division
-    const int q = w / NN, k = w - q * NN;
-    const int j = nlive == 1 ? q : (nlive == 2 ? q >> 1 : (q * 21846) >> 16);
-    const int ai = q - j * nlive;
+    int j;
+    const NodeRec rec = node_record<BC>(g, it.dir_begin, live, nlive, w, j);
     const Tpl<R> T(slots + sb * j, TL);
     const R *fin = reinterpret_cast<const R *>(slots + sb * j + TL.node_bytes);
-    // the k-th node ray by length, as in the paired face pass
-    int a = (live >> (2 * ai)) & 3, r = k;
-    if (g.node_order) {
-      const uint16_t *no = g.node_order + (size_t)(it.dir_begin + j) * (6 * NN);
-      if (nlive == 3) {
-        const int k3 = w - j * (3 * NN);
-        const int code = __ldg(no + 3 * NN + ((j & 1) ? 3 * NN - 1 - k3 : k3));
-        a = code / NN;
-        r = code - a * NN;
-      } else {
-        r = __ldg(no + a * NN + ((q & 1) ? NN - 1 - k : k));
-      }
-    }
-    const int ub = r / N1, uc = r - ub * N1;  // upwind-frame node on the downwind face of axis a
-    // upwind-frame node coordinates (L0, L1, L2): B along the face's axis
-    const int L0 = a == 0 ? B : ub;
-    const int L1 = a == 1 ? B : (a == 0 ? ub : uc);
-    const int L2 = a == 2 ? B : uc;
-    const int p0 = T.npos[L0], p1 = T.npos[N1 + L1], p2 = T.npos[2 * N1 + L2];
-    int last = p0, ae = 0, la = L0, lb = L1, lc = L2;
-    if (p1 < last) { last = p1; ae = 1; la = L1; lb = L0; }
-    if (p2 < last) { last = p2; ae = 2; la = L2; lb = L0; lc = L1; }
-    const int row = (ae * 2) * N1 + la;
-    R I = face_value<R>(fin, g.fstride, B, ae, lb, lc, T.nk[row], T.nk[row + N1], T.nw[row], T.nw[row + N1]);
+    const int row = rec.row();
+    R I = face_value<R>(fin + rec.face(), W, T.nw[row], T.nw[row + N1]);
+    int last = rec.last();
     if (!act) last = -1;
     // The lanes march in lockstep aligned at the downwind end: the warp runs
     // from its largest `last` down to event 0, and a lane whose own ray is
@@ -481,15 +533,8 @@ __global__ void __launch_bounds__(kFaceThreads, sizeof(R) == 8 ? 2 : 3)
     // at the same step, so their tile addresses are one common offset from
     // neighbouring start cells (few shared-memory bank conflicts).
     const int wl = __reduce_max_sync(0xffffffffu, last);
-    if (wl >= 0) {
-      // where last >= 0, every L >= 1 and the start cell is inside the block
-      const int c0 = T.h->sgn[0] > 0 ? L0 - 1 : B - L0;
-      const int c1 = T.h->sgn[1] > 0 ? L1 - 1 : B - L1;
-      const int c2 = T.h->sgn[2] > 0 ? L2 - 1 : B - L2;
-      const int idx0 = last >= 0 ? c0 + ts.sy * c1 + ts.sz * c2 : 0;
-      I = march_aligned<R>(tile, idx0, last, wl, T.nev, g.exp64, I);
-    }
-    if (act) faces[(((long long)(it.dir_begin + j) * nblk + it.block) * 3 + a) * g.fstride + ub * W + uc] = I;
+    if (wl >= 0) I = march_aligned<R>(tile, rec.start(), last, wl, T.nev, g.exp64, I);
+    if (act) faces[((long long)(it.dir_begin + j) * nblk + it.block) * 3 * g.fstride + rec.out()] = I;
   }
 }
 
@@ -575,6 +620,10 @@ __global__ void __launch_bounds__(kCellThreads, kCellMinCtas<R>)
     cz = lc / B2;
   }
   const int tc = cx + ts.sy * cy + ts.sz * cz;  // tile index
+  // this cell's record of the direction after the current one is on its way
+  // while the current ray is marched
+  const uint32_t *cell_rec = g.cell_rec + cell_rec_index(B, cx, cy, cz);
+  uint32_t next_rec = __ldg(cell_rec + (size_t)order_dir(order[0]) * B3);
   const long long gc = ((long long)(bz * B + cz) * g.ny + (by * B + cy)) * g.nx + (bx * B + cx);
   // Moments over all directions: a plain partial sum over the directions of
   // one tile, folded into the totals once per tile.  The fold of E, Pxx, Pyy
@@ -601,17 +650,10 @@ __global__ void __launch_bounds__(kCellThreads, kCellMinCtas<R>)
       for (int j = 0; j < nd; ++j) {
         const Tpl<R> T(buf + sb * j, TL);
         const R *fin = reinterpret_cast<const R *>(buf + sb * j + TL.bytes);
-        // upwind-frame coordinates; the exit axis ae is the one whose plane
-        // event comes first, (lb, lc) the other two in increasing axis order
-        const int l0 = T.h->sgn[0] > 0 ? cx : B - 1 - cx;
-        const int l1 = T.h->sgn[1] > 0 ? cy : B - 1 - cy;
-        const int l2 = T.h->sgn[2] > 0 ? cz : B - 1 - cz;
-        const int p0 = T.cpos[l0], p1 = T.cpos[B + l1], p2 = T.cpos[2 * B + l2];
-        int last = p0, ae = 0, la = l0, lb = l1, lc = l2;
-        if (p1 < last) { last = p1; ae = 1; la = l1; lb = l0; }
-        if (p2 < last) { last = p2; ae = 2; la = l2; lb = l0; lc = l1; }
-        const int row = (ae * 2) * B + la;
-        const R Iin = face_value<R>(fin, fstride, B, ae, lb, lc, T.ck[row], T.ck[row + B], T.cw[row], T.cw[row + B]);
+        const CellRec rec{next_rec};
+        next_rec = __ldg(cell_rec + (size_t)order_dir(order[min(t * dt + j + 1, g.ndir - 1)]) * B3);
+        const int last = rec.last(), row = rec.row();
+        const R Iin = face_value<R>(fin + rec.face(), B + 2, T.cw[row], T.cw[row + B]);
         const R I = march<R>(tile, tc, last, T.cev, g.exp64, Iin);
         if (MODE == 1) {
           I_out[(long long)T.h->ext * g.ncell + gc] = I;
@@ -997,6 +1039,38 @@ static_assert(offsetof(TplHead<float>, sgn) == 16 && offsetof(TplHead<float>, ex
                   offsetof(TplHead<float>, mirror) == 32 && offsetof(TplHead<float>, cp) % 16 == 0,
               "TplHead<float> layout");
 
+// A thread's lower-half cell (z < B/2): 4 x 4 x 2 bricks, warp-major.  Layer
+// pair lp holds z = 2 lp, 2 lp + 1 of the lower half; with two parts of a 16^3
+// block, part 0 takes layer pairs 0 and 3 and part 1 takes 1 and 2 (85e3 and
+// 89e3 warp steps over 192 directions, where z-order parts differ by 15%), so
+// that the CTAs of a wave carry about equal work.
+template <int B>
+struct PairCell {
+  int q, x, y, z;  // place among the part's cells; the cell
+  __device__ __forceinline__ PairCell(int part, int parts, uint32_t tid) {
+    q = part * pair_threads(B) + (int)tid;
+    const int qb = q >> 5, ln = q & 31;
+    x = 4 * (qb % (B / 4)) + (ln & 3);
+    y = 4 * ((qb / (B / 4)) % (B / 4)) + ((ln >> 2) & 3);
+    int lp = qb / (B * B / 16);
+    if (B == 16 && parts == 2) lp = (0x2130 >> (4 * lp)) & 15;
+    z = 2 * lp + (ln >> 4);
+  }
+  __device__ __forceinline__ long long cell(const GridDims &g, int bx, int by, int bz) const {
+    return ((long long)(bz * B + z) * g.ny + (by * B + y)) * g.nx + (bx * B + x);
+  }
+  __device__ __forceinline__ long long mirror(const GridDims &g, int bx, int by, int bz) const {
+    return ((long long)(bz * B + B - 1 - z) * g.ny + (by * B + B - 1 - y)) * g.nx + (bx * B + B - 1 - x);
+  }
+};
+// threadIdx.x read anew: what is only needed after the marches is worked out
+// there instead of being held in registers through them.
+__device__ __forceinline__ uint32_t fresh_tid() {
+  uint32_t t;
+  asm volatile("mov.u32 %0, %%tid.x;" : "=r"(t));
+  return t;
+}
+
 // ORDERED (moment modes): every CTA is one share of a work item, see TailPlan.
 template <int MODE, int BC, bool MERGED, bool ORDERED = false>
 __global__ void __launch_bounds__(pair_threads(BC), pair_min_ctas(BC))
@@ -1082,24 +1156,9 @@ __global__ void __launch_bounds__(pair_threads(BC), pair_min_ctas(BC))
   if (threadIdx.x == 0) tile[B] = make_float4(0.f, 0.f, 0.f, 0.f);  // identity entry (padding, x = B)
   __syncthreads();
 
-  // this thread's lower-half cell (z < B/2): 4 x 4 x 2 bricks, warp-major
-  const int q = part * NT + (int)threadIdx.x;
-  const int qb = q >> 5, ln = q & 31;
-  const int cx = 4 * (qb % (B / 4)) + (ln & 3);
-  const int cy = 4 * ((qb / (B / 4)) % (B / 4)) + ((ln >> 2) & 3);
-  // layer pair lp holds z = 2 lp, 2 lp + 1 of the lower half; with two parts
-  // of a 16^3 block, part 0 takes layer pairs 0 and 3 and part 1 takes 1 and
-  // 2 (85e3 and 89e3 warp steps over 192 directions, where z-order parts
-  // differ by 15%), so that the CTAs of a wave carry about equal work
-  int lp = qb / (B2 / 16);
-  if (B == 16 && parts == 2) lp = (0x2130 >> (4 * lp)) & 15;
-  const int cz = 2 * lp + (ln >> 4);
-  const int mx = B - 1 - cx, my = B - 1 - cy, mz = B - 1 - cz;  // the mirror cell
+  const PairCell<BC> pc(part, parts, threadIdx.x);
   const uint32_t tile_s = smem_u32(tile);
-  const uint32_t t1 = tile_s + 16u * (uint32_t)(cx + ts.sy * cy + ts.sz * cz);
-  const uint32_t t2 = tile_s + 16u * (uint32_t)(mx + ts.sy * my + ts.sz * mz);
-  const long long gc1 = ((long long)(bz * B + cz) * g.ny + (by * B + cy)) * g.nx + (bx * B + cx);
-  const long long gc2 = ((long long)(bz * B + mz) * g.ny + (by * B + my)) * g.nx + (bx * B + mx);
+  const uint32_t t1 = tile_s + 16u * (uint32_t)(pc.x + ts.sy * pc.y + ts.sz * pc.z);
   constexpr bool kWantF = MODE == 0;
   // moments of (c, c') as packed pairs: E, Fx, Fy, Fz, Pxx, Pyy, Pzz, Pxy,
   // Pxz, Pyz; compensated E and Pii (nc: their negated compensations), which
@@ -1119,23 +1178,14 @@ __global__ void __launch_bounds__(pair_threads(BC), pair_min_ctas(BC))
   constexpr int W = B + 2;
   const uint32_t fW = 4u * W;
 
-  // Exit lookup and entry value of the ray(s) of one march: primary slot ps
-  // (its template), upwind-frame coordinates l0..l2; returns the pair of
-  // entry intensities from faces f1 (primary) and f2 (the pair's second ray).
-  auto entry = [&](uint32_t ps, int l0, int l1, int l2, uint32_t f1, uint32_t f2, int &last) -> float2 {
-    const int p0 = lds_s16(ps + CS.cpos + 2 * l0), p1 = lds_s16(ps + CS.cpos + 2 * (B + l1)),
-              p2 = lds_s16(ps + CS.cpos + 2 * (2 * B + l2));
-    int ae = 0, la = l0, lb = l1, lc = l2;
-    last = p0;
-    if (p1 < last) { last = p1; ae = 1; la = l1; lb = l0; }
-    if (p2 < last) { last = p2; ae = 2; la = l2; lb = l0; lc = l1; }
-    const int row = (ae * 2) * B + la;
-    const int kb = lds_s16(ps + CS.ck + 2 * row), kc = lds_s16(ps + CS.ck + 2 * (row + B));
-    const uint2 ub = lds_2x32(ps + CS.cw + 8 * row), uc = lds_2x32(ps + CS.cw + 8 * (row + B));
+  // Entry value of the ray(s) of one march, by its record: primary slot ps
+  // (its weights), faces f1 (primary) and f2 (the pair's second ray).
+  auto entry = [&](uint32_t ps, CellRec rec, uint32_t f1, uint32_t f2) -> float2 {
+    const uint32_t wa = ps + CS.cw + 8 * (uint32_t)rec.row();
+    const uint2 ub = lds_2x32(wa), uc = lds_2x32(wa + 8 * B);
     const float wbx = __uint_as_float(ub.x), wby = __uint_as_float(ub.y);
     const float wcx = __uint_as_float(uc.x), wcy = __uint_as_float(uc.y);
-    const int ib = max(lb + kb, 0), ic = max(lc + kc, 0);
-    const uint32_t fo = 4u * (uint32_t)(ae * fstride + ib * W + ic);
+    const uint32_t fo = 4u * (uint32_t)rec.face();
     const uint32_t a1 = f1 + fo, a2 = f2 + fo;
     const float I1 = wby * (wcy * lds_f32(a1) + wcx * lds_f32(a1 + 4)) +
                      wbx * (wcy * lds_f32(a1 + fW) + wcx * lds_f32(a1 + fW + 4));
@@ -1143,15 +1193,24 @@ __global__ void __launch_bounds__(pair_threads(BC), pair_min_ctas(BC))
                      wbx * (wcy * lds_f32(a2 + fW) + wcx * lds_f32(a2 + fW + 4));
     return make_float2(I1, I2);
   };
+  // This cell's records: that of a march is on its way during the one before.
+  const uint32_t rec_at = (uint32_t)cell_rec_index(B, pc.x, pc.y, pc.z);
+  auto record = [&](int k) {  // of the k-th direction of the order
+    const int v = ord_smem ? s_ord[k] : __ldg(order + k);
+    return __ldg(g.cell_rec + ((uint32_t)order_dir(v) * (uint32_t)(B * B2) + rec_at));
+  };
+  uint32_t next_a = record(tile0 * dt);
   // one ray of a pair that is not an exact mirror image: its own template
-  // (slot ps, signs sg), start cell (x, y, z), entry face f
-  auto single = [&](uint32_t ps, uint4 hd, int x, int y, int z, uint32_t tstart) -> float {
-    const int l0 = (int)hd.x > 0 ? x : B - 1 - x;
-    const int l1 = (int)hd.y > 0 ? y : B - 1 - y;
-    const int l2 = (int)hd.z > 0 ? z : B - 1 - z;
-    int last;
-    const float2 Iin = entry(ps, l0, l1, l2, ps + CS.faces, ps + CS.faces, last);
-    return march_one(tstart, ps + CS.cev, last, Iin.x);
+  // (slot ps), the record of its start cell in that direction
+  auto single = [&](uint32_t ps, int k, bool mirror_cell) -> float {
+    const int v = ord_smem ? s_ord[k] : __ldg(order + k);
+    const PairCell<BC> c(part, parts, fresh_tid());
+    const int x = mirror_cell ? B - 1 - c.x : c.x, y = mirror_cell ? B - 1 - c.y : c.y, z = mirror_cell ? B - 1 - c.z : c.z;
+    const uint32_t tstart = tile_s + 16u * (uint32_t)(x + ts.sy * y + ts.sz * z);
+    const uint32_t *r = g.cell_rec + (size_t)order_dir(v) * (B * B2) + cell_rec_index(B, x, y, z);
+    const CellRec rec{__ldg(r)};
+    const float2 Iin = entry(ps, rec, ps + CS.faces, ps + CS.faces);
+    return march_one(tstart, ps + CS.cev, rec.last(), Iin.x);
   };
 
   bool ok = true;
@@ -1178,34 +1237,33 @@ __global__ void __launch_bounds__(pair_threads(BC), pair_min_ctas(BC))
     const uint32_t buf = ring_s + (uint32_t)(st * stage_bytes);
     for (int j = 0; j < nd; j += 2) {  // the antipodal pair (j, j + 1)
       const uint32_t sa = buf + (uint32_t)(CS.bytes * j), sb = sa + (uint32_t)CS.bytes;
-      const uint4 ha = lds_4x32(sa + 16), hb = lds_4x32(sb + 16);  // (sgn0, sgn1, sgn2, ext)
       const int mirror = (int)lds_2x32(sa + 32).x;
+      const int k = (tile0 + t) * dt + j;
+      const CellRec rb{record(k + 1)};
       float2 m1, m2;  // m1 = (I(c, d), I(c', -d)), m2 = (I(c, -d), I(c', d))
       if (mirror) {
-        // upwind-frame coordinates of c in the primary direction; the mirror
-        // cell in the antipode has the same ones (each flips to B - 1 - c)
-        int last;
-        {
-          const int l0 = (int)ha.x > 0 ? cx : mx, l1 = (int)ha.y > 0 ? cy : my, l2 = (int)ha.z > 0 ? cz : mz;
-          const float2 Iin = entry(sa, l0, l1, l2, sa + CS.faces, sb + CS.faces, last);
-          m1 = march_pair(t1, id_s, sa + CS.cev, last, Iin);
-        }
-        {
-          const int l0 = (int)hb.x > 0 ? cx : mx, l1 = (int)hb.y > 0 ? cy : my, l2 = (int)hb.z > 0 ? cz : mz;
-          const float2 Iin = entry(sb, l0, l1, l2, sb + CS.faces, sa + CS.faces, last);
-          m2 = march_pair(t1, id_s, sb + CS.cev, last, Iin);
-        }
+        // the mirror cell's ray in the antipode has the upwind-frame
+        // coordinates of c's in the primary direction: one record for both
+        const CellRec ra{next_a};
+        const float2 I1 = entry(sa, ra, sa + CS.faces, sb + CS.faces);
+        m1 = march_pair(t1, id_s, sa + CS.cev, ra.last(), I1);
+        next_a = record(min(k + 2, g.ndir - 2));
+        const float2 I2 = entry(sb, rb, sb + CS.faces, sa + CS.faces);
+        m2 = march_pair(t1, id_s, sb + CS.cev, rb.last(), I2);
       } else {
         // the pair's templates differ (near-tied plane crossings ordered
         // differently): each ray follows its own direction's template
-        m1 = make_float2(single(sa, ha, cx, cy, cz, t1), single(sb, hb, mx, my, mz, t2));
-        m2 = make_float2(single(sb, hb, cx, cy, cz, t1), single(sa, ha, mx, my, mz, t2));
+        m1 = make_float2(single(sa, k, false), single(sb, k + 1, true));
+        m2 = make_float2(single(sb, k + 1, false), single(sa, k, true));
+        next_a = record(min(k + 2, g.ndir - 2));
       }
       if (MODE == 1) {
-        I_out[(long long)ha.w * g.ncell + gc1] = m1.x;
-        I_out[(long long)hb.w * g.ncell + gc2] = m1.y;
-        I_out[(long long)hb.w * g.ncell + gc1] = m2.x;
-        I_out[(long long)ha.w * g.ncell + gc2] = m2.y;
+        const int ea = (int)lds_2x32(sa + 24).y, eb = (int)lds_2x32(sb + 24).y;  // the directions' public indices
+        const long long gc1 = pc.cell(g, bx, by, bz), gc2 = pc.mirror(g, bx, by, bz);
+        I_out[(long long)ea * g.ncell + gc1] = m1.x;
+        I_out[(long long)eb * g.ncell + gc2] = m1.y;
+        I_out[(long long)eb * g.ncell + gc1] = m2.x;
+        I_out[(long long)ea * g.ncell + gc2] = m2.y;
       } else if (ORDERED) {
         // this pair's place in the item's list: pairs are consecutive in the order
         const int pair = ((tile0 + t) * dt + j) >> 1;
@@ -1362,11 +1420,12 @@ __global__ void __launch_bounds__(pair_threads(BC), pair_min_ctas(BC))
         Ms[1][m] = mom[m].y;
       }
       float *st = reinterpret_cast<float *>(ring);
-      const int zs = 2 * (qb / (B2 / 16) - part * (L / 2)) + (ln >> 4);  // the lower cell's z slot
-      const int li[2] = {(zs * B + cy) * B + cx, ((L + zs) * B + my) * B + mx};
+      const PairCell<BC> c(part, parts, fresh_tid());
+      const int zs = 2 * ((c.q >> 5) / (B2 / 16) - part * (L / 2)) + ((c.q & 31) >> 4);  // the lower cell's z slot
+      const int li[2] = {(zs * B + c.y) * B + c.x, ((L + zs) * B + B - 1 - c.y) * B + B - 1 - c.x};
 #pragma unroll
       for (int r = 0; r < 2; ++r) {
-        const long long gc = r ? gc2 : gc1;
+        const long long gc = r ? c.mirror(g, bx, by, bz) : c.cell(g, bx, by, bz);
         const float E = Ms[r][0];
         float v[NV];
         if (kWantF) {
@@ -1519,45 +1578,18 @@ __global__ void __launch_bounds__(kFaceThreads, 2)
     const int wr = w0 + ((int)threadIdx.x & 31);
     const bool act = wr < total;
     const int w = act ? wr : total - 1;
-    const int q = w / NN, k = w - q * NN;
-    const int j = nlive == 1 ? q : (nlive == 2 ? q >> 1 : (q * 21846) >> 16);
-    const int ai = q - j * nlive;
+    int j;
+    const NodeRec rec = node_record<BC>(g, it.dir_begin, live, nlive, w, j);
     // 32-bit shared addresses of the slot's template parts and both rays'
     // incoming faces
     const uint32_t ps = slots_s + (uint32_t)(sb * j);
     const uint32_t f1 = ps + (uint32_t)TL.node_bytes, f2 = slots_s + (uint32_t)(sb * cnt + fb3 * j);
-    // the k-th node ray by length: of the face, or where all three faces
-    // are computed, of the three merged; every other face (or direction)
-    // of the item taken from its longest ray down, so that a warp that
-    // straddles two joins rays of similar length too
-    int a = (live >> (2 * ai)) & 3, r = k;
-    if (g.node_order) {
-      const uint16_t *no = g.node_order + (size_t)(it.dir_begin + j) * (6 * NN);
-      if (nlive == 3) {
-        const int k3 = w - j * (3 * NN);
-        const int code = __ldg(no + 3 * NN + ((j & 1) ? 3 * NN - 1 - k3 : k3));
-        a = code / NN;
-        r = code - a * NN;
-      } else {
-        r = __ldg(no + a * NN + ((q & 1) ? NN - 1 - k : k));
-      }
-    }
-    const int ub = r / N1, uc = r - ub * N1;
-    const int L0 = a == 0 ? B : ub;
-    const int L1 = a == 1 ? B : (a == 0 ? ub : uc);
-    const int L2 = a == 2 ? B : uc;
-    const uint32_t pp = ps + (uint32_t)TL.npos;
-    const int p0 = lds_s16(pp + 2 * L0), p1 = lds_s16(pp + 2 * (N1 + L1)), p2 = lds_s16(pp + 2 * (2 * N1 + L2));
-    int last = p0, ae = 0, la = L0, lb = L1, lc = L2;
-    if (p1 < last) { last = p1; ae = 1; la = L1; lb = L0; }
-    if (p2 < last) { last = p2; ae = 2; la = L2; lb = L0; lc = L1; }
-    const int row = (ae * 2) * N1 + la;
-    const int kb = lds_s16(ps + TL.nk + 2 * row), kc = lds_s16(ps + TL.nk + 2 * (row + N1));
-    const uint2 wbu = lds_2x32(ps + TL.nw + 8 * row), wcu = lds_2x32(ps + TL.nw + 8 * (row + N1));
+    int last = rec.last();
+    const uint32_t wa = ps + (uint32_t)TL.nw + 8 * (uint32_t)rec.row();
+    const uint2 wbu = lds_2x32(wa), wcu = lds_2x32(wa + 8 * N1);
     const float wbx = __uint_as_float(wbu.x), wby = __uint_as_float(wbu.y);
     const float wcx = __uint_as_float(wcu.x), wcy = __uint_as_float(wcu.y);
-    const int ib = max(lb + kb, 0), ic = max(lc + kc, 0);
-    const uint32_t fo = 4u * (uint32_t)(ae * g.fstride + ib * W + ic);
+    const uint32_t fo = 4u * (uint32_t)rec.face();
     const uint32_t a1 = f1 + fo, a2 = f2 + fo;
     float2 I = make_float2(wby * (wcy * lds_f32(a1) + wcx * lds_f32(a1 + 4)) +
                                wbx * (wcy * lds_f32(a1 + 4 * W) + wcx * lds_f32(a1 + 4 * W + 4)),
@@ -1570,11 +1602,7 @@ __global__ void __launch_bounds__(kFaceThreads, 2)
     // four at a time in 16-byte pairs
     const int wl = __reduce_max_sync(0xffffffffu, last);
     if (wl >= 0) {
-      const uint4 hd = lds_4x32(ps + 16);  // (sgn0, sgn1, sgn2, ext)
-      const int c0 = (int)hd.x > 0 ? L0 - 1 : B - L0;
-      const int c1 = (int)hd.y > 0 ? L1 - 1 : B - L1;
-      const int c2 = (int)hd.z > 0 ? L2 - 1 : B - L2;
-      const uint32_t tb = last >= 0 ? tile_s + 16u * (uint32_t)(c0 + ts.sy * c1 + ts.sz * c2) : id_s;
+      const uint32_t tb = last >= 0 ? tile_s + 16u * (uint32_t)rec.start() : id_s;
       const uint32_t ev = ps + (uint32_t)TL.nev;
       int e = wl;
       if (!(e & 1)) {  // to an odd index: event pairs (e - 1, e) are 16-byte aligned
@@ -1597,10 +1625,9 @@ __global__ void __launch_bounds__(kFaceThreads, 2)
       }
     }
     if (act) {
-      const float I1 = I.x, I2 = I.y;
-      const int node = ub * W + uc;
-      faces[(((long long)(it.dir_begin + j) * nblk + it.block) * 3 + a) * g.fstride + node] = I1;
-      faces[(((long long)(it.mirror_begin + j) * nblk + mblock) * 3 + a) * g.fstride + node] = I2;
+      const int out = rec.out();
+      faces[((long long)(it.dir_begin + j) * nblk + it.block) * 3 * g.fstride + out] = I.x;
+      faces[((long long)(it.mirror_begin + j) * nblk + mblock) * 3 * g.fstride + out] = I.y;
     }
   }
 }
@@ -2036,6 +2063,14 @@ cudaError_t launch_cell_pass(const GridDims &g, int mode, const R *kappa, const 
 }
 
 template <typename R>
+cudaError_t launch_ray_records(const GridDims &g, const unsigned char *tpl, const uint16_t *node_order, uint32_t *cell_rec,
+                               uint2 *node_rec, cudaStream_t st) {
+  const int per_dir = g.B * g.B * g.B + 6 * (g.B + 1) * (g.B + 1);
+  ray_records_kernel<R><<<dim3((per_dir + 255) / 256, g.ndir), 256, 0, st>>>(g, tpl, node_order, cell_rec, node_rec);
+  return cudaGetLastError();
+}
+
+template <typename R>
 cudaError_t launch_fill_boundary(const GridDims &g, const unsigned char *tpl, const R *Ib, R *bnd, cudaStream_t st) {
   fill_boundary_kernel<R><<<dim3(g.ndir, 6), 128, 0, st>>>(g, tpl, tpl_layout<R>(g.B).bytes, Ib, bnd);
   return cudaGetLastError();
@@ -2129,6 +2164,8 @@ cudaError_t prepare_kernels() {
                                            const TailSplit *);                                               \
   template cudaError_t launch_floor_fix_blocks<R>(const GridDims &, const int *, int, const R *, const void *, \
                                                   double, R *, cudaStream_t);                                \
+  template cudaError_t launch_ray_records<R>(const GridDims &, const unsigned char *, const uint16_t *, uint32_t *, \
+                                             uint2 *, cudaStream_t);                                        \
   template cudaError_t launch_fill_boundary<R>(const GridDims &, const unsigned char *, const R *, R *,      \
                                                cudaStream_t);                                                \
   template cudaError_t launch_floor_fix<R>(long long, const R *, long long, const void *, double, R *,     \

@@ -30,6 +30,12 @@ namespace {
 
 static __device__ __align__(256) unsigned char g_scratch[VET_NOALLOC_SCRATCH_BYTES];
 
+// Ray records of the largest direction set and block edge, beside the scratch
+// array (whose size is part of the interface): nodes, then cells.
+constexpr size_t kNodeRecMax = 192u * 6u * 17u * 17u, kCellRecMax = 192u * 16u * 16u * 16u;
+static __device__ __align__(256) uint2 g_node_rec[kNodeRecMax];
+static __device__ __align__(256) uint32_t g_cell_rec[kCellRecMax];
+
 constexpr int kMaxDevices = 64;
 constexpr int kMaxDirs = 192;            // nside <= 4
 constexpr int kMaxEdge = 16;             // block edge <= 16
@@ -39,6 +45,7 @@ constexpr int kMaxLevels = 4096;
 
 std::mutex g_mutex;                     // one host thread stages at a time
 void *g_addr[kMaxDevices];              // device address of g_scratch per device
+void *g_rec_addr[kMaxDevices][2];       // of the record arrays
 
 // fixed host staging (no heap)
 alignas(16) unsigned char h_tpl[kMaxDirs * kTplMax];
@@ -168,6 +175,11 @@ VET_API vet_status vet_closure_noalloc(const vet_grid *grid, const vet_config *c
       void *p = nullptr;
       e = cudaGetSymbolAddress(&p, g_scratch);
       if (e != cudaSuccess) { result = fail(VET_ECUDA, std::string("cudaGetSymbolAddress: ") + cudaGetErrorString(e)); break; }
+      if ((e = cudaGetSymbolAddress(&g_rec_addr[cfg->device][0], g_node_rec)) ||
+          (e = cudaGetSymbolAddress(&g_rec_addr[cfg->device][1], g_cell_rec))) {
+        result = fail(VET_ECUDA, std::string("cudaGetSymbolAddress: ") + cudaGetErrorString(e));
+        break;
+      }
       e = vet::prepare_kernels();
       if (e != cudaSuccess) { result = fail(VET_ECUDA, std::string("cudaFuncSetAttribute: ") + cudaGetErrorString(e)); break; }
       g_addr[cfg->device] = p;
@@ -192,6 +204,11 @@ VET_API vet_status vet_closure_noalloc(const vet_grid *grid, const vet_config *c
     if ((e = cudaMemsetAsync(d_emax, 0, 8, st))) break;
     if ((e = cudaMemsetAsync(d_status, 0, sizeof(int), st))) break;
     const long long spin = cfg->spin_limit > 0 ? cfg->spin_limit : (1LL << 22);
+    auto *node_rec = static_cast<uint2 *>(g_rec_addr[cfg->device][0]);
+    auto *cell_rec = static_cast<uint32_t *>(g_rec_addr[cfg->device][1]);
+    if ((e = vet::launch_ray_records<float>(dims, d_tpl, nullptr, cell_rec, node_rec, st))) break;
+    dims.node_rec = node_rec;
+    dims.cell_rec = cell_rec;
     if ((e = vet::launch_fill_boundary<float>(dims, d_tpl, Ib, d_bnd, st))) break;
     for (int L = 0; L < nlevels && !e; ++L)
       e = vet::launch_face_level<float>(dims, kappa, S, d_tpl, d_items + h_level_off[L],
