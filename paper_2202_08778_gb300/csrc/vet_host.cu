@@ -205,9 +205,9 @@ vet_status build_context(vet_ctx *c) {
   int ob[9];
   vet::geom::internal_order(N, c->dirs_ext.data(), order.data(), ob);
   // FP32 face pass on mirrored block pairs: antipodes at equal positions of
-  // opposite octants (block edges 8 and 16, no zero direction component)
+  // opposite octants (block edges up to kMaxPairBlock, no zero direction component)
   const bool mirror_order =
-      !c->fp64 && (B == 8 || B == 16) && vet::geom::mirror_octant_order(N, c->dirs_ext.data(), order.data(), ob);
+      !c->fp64 && B <= vet::kMaxPairBlock && vet::geom::mirror_octant_order(N, c->dirs_ext.data(), order.data(), ob);
   const int tbytes = vet::tpl_layout<R>(B).bytes;
   std::vector<unsigned char> tpl((size_t)tbytes * N);
   long long cs_tot = 0, ns_tot = 0;
@@ -226,9 +226,9 @@ vet_status build_context(vet_ctx *c) {
   std::vector<int> cell_order(N);
   vet::geom::interleaved_order(ob, cell_order.data());
   // FP32 cell pass on mirrored ray pairs where the set is closed under
-  // negation (block edges 8 and 16)
+  // negation (block edges kMinPairBlock to kMaxPairBlock)
   c->dims.paired = 0;
-  if (!c->fp64 && (B == 8 || B == 16) && vet::geom::antipodal_order(N, c->dirs_ext.data(), order.data(),
+  if (!c->fp64 && B >= vet::kMinPairBlock && B <= vet::kMaxPairBlock && vet::geom::antipodal_order(N, c->dirs_ext.data(), order.data(),
                                                                      cell_order.data())) {
     c->dims.paired = 1;
     // pairs whose templates are not exact mirrors, or with a zero direction

@@ -160,7 +160,7 @@ struct NodeRec {
 // multiple of 4, the 4 x 4 x 2 bricks that the warps of the cell passes take,
 // one after another; else row by row.
 __host__ __device__ inline int cell_rec_index(int B, int x, int y, int z) {
-  if (B % 4 || B % 2) return (z * B + y) * B + x;
+  if (B % 4) return (z * B + y) * B + x;
   return (((z >> 1) * (B / 4) + (y >> 2)) * (B / 4) + (x >> 2)) * 32 + (z & 1) * 16 + (y & 3) * 4 + (x & 3);
 }
 inline size_t cell_rec_count(int N, int B) { return (size_t)N * B * B * B; }
@@ -170,16 +170,20 @@ inline size_t node_rec_count(int N, int B) { return (size_t)N * 6 * (B + 1) * (B
 // for the FP32 mirrored passes, 16 bytes (kappa, kappa', S, S').  Face pass:
 // cell (x, y, z) at x + (B+1) y + (B+1)^2 z; the three strides are odd, so a
 // warp walking a row, column or pillar of a face (and any uniform shift of
-// it) touches distinct banks.  Cell pass: x + (B+4) y + (B+4) B z; with B a
-// multiple of 8 the y stride is 4 or 12 mod 16 entries of 8 bytes (a 4 x 4
-// layer of a warp's 4 x 4 x 2 cell brick is conflict free) and 4 mod 8
-// entries of 16 bytes (each quarter warp, 4 x 2 cells, covers the 32 banks
-// once).
+// it) touches distinct banks.  Cell pass: where B is a multiple of 4, the y
+// stride is the first above B that is 4 mod 8 entries (12 for 8, 20 for 12 and
+// 16): a 4 x 4 layer of a warp's 4 x 4 x 2 cell brick is conflict free in 8-byte
+// entries, a quarter warp's 4 x 2 cells in 16-byte ones.  Other edges are
+// walked row by row and stored without padding.  The last entry is the cell
+// pass's identity segment.
 struct TileShape {
   int sy, sz, elems;
 };
 __host__ __device__ inline TileShape node_tile(int B) { return {B + 1, (B + 1) * (B + 1), (B + 1) * (B + 1) * B}; }
-__host__ __device__ inline TileShape cell_tile(int B) { return {B + 4, (B + 4) * B, (B + 4) * B * B}; }
+__host__ __device__ inline TileShape cell_tile(int B) {
+  const int sy = B % 4 ? B : B + 8 - (B + 4) % 8;
+  return {sy, sy * B, sy * B * B + 1};
+}
 
 // Stored faces: node (ub, uc) of a face, in the upwind frame of the direction
 // (the in-plane axes flipped where the direction component is negative), at
@@ -230,8 +234,8 @@ cudaError_t launch_face_level(const GridDims &g, const R *kappa, const R *S, con
 // not take one CTA's time on a part of the SMs.  Its results are the unsplit
 // pass's bits (a small grid's closure equals the same grid's in a batch, or
 // its blocks' in the learned closure's fallback): the shares store each
-// antipodal pair's sum and difference of intensities, and the last share of
-// an item adds them in the unsplit order (`ordered`).
+// antipodal pair's intensities, and the last share of an item adds
+// them in the unsplit order (`ordered`).
 struct TailPlan {
   int nfull = 0;          // CTAs that run whole (total - r)
   int k = 1;              // shares per split work item (1: no split)
@@ -328,6 +332,14 @@ size_t cell_smem_bytes(int B, int nslots, bool fp64);
 // Directions per face-pass item (default; a context may be tuned to 1..8).
 constexpr int kFaceGroup = 4;
 constexpr int kMaxTune = 8;
+// Largest block edge of the mirrored (paired) FP32 passes: their 16-byte tiles
+// and staged directions fit a CTA's shared memory.
+constexpr int kMaxPairBlock = 16;
+// Smallest block edge of the paired cell pass: below, a CTA's few cells do not
+// pay for its pairs of staged directions (cell pass, paired against unpaired: edge 4
+// 0.42 and 0.38 ms, 5 0.36 and 0.34, 6 0.42 and 0.56, 12 1.5 and 2.7; the paired
+// face pass is ahead from 2 on, 0.59 and 0.67 ms).
+constexpr int kMinPairBlock = 6;
 
 // Per-device kernel attributes; call with the context's device current.
 cudaError_t prepare_kernels();

@@ -14,8 +14,9 @@
 // Both passes stage the block's kappa/S tile, the directions' ray templates
 // and the incoming faces in shared memory.  Faces are stored by the face pass
 // already in the consumer's upwind frame and padded, so staging is a plain
-// 16-byte copy.  Kernels are compiled for the block edges 8 and 16 (index
-// arithmetic folds to shifts) and for a runtime edge.
+// 16-byte copy.  Every pass is compiled for the block edges 8 and 16 (index
+// arithmetic folds to shifts) and for a runtime edge; the mirrored FP32 passes
+// take edges up to 16 (cell pass: from 6).
 #include <algorithm>
 #include <cstddef>
 #include <cstdint>
@@ -438,13 +439,15 @@ constexpr int kFaceThreads = 512;
 template <int BC>
 __device__ __forceinline__ NodeRec node_record(const GridDims &g, int dir_begin, int live, int nlive, int w, int &j) {
   const int NN = BC ? (BC + 1) * (BC + 1) : g.nnode;
+  // w < 2^15; a runtime edge divides by a multiplication (exact there)
+  auto div = [&](int n, int d) { return BC ? n / d : (int)__umulhi((unsigned)n, 0xffffffffu / (unsigned)d + 1u); };
   int e;
   if (nlive == 3) {
-    j = w / (3 * NN);
+    j = div(w, 3 * NN);
     const int k = w - j * (3 * NN);
     e = 3 * NN + ((j & 1) ? 3 * NN - 1 - k : k);
   } else {
-    const int q = w / NN, k = w - q * NN;
+    const int q = div(w, NN), k = w - q * NN;
     j = nlive == 1 ? q : q >> 1;
     const int a = (live >> (2 * (q - j * nlive))) & 3;
     e = a * NN + ((q & 1) ? NN - 1 - k : k);
@@ -725,8 +728,8 @@ __global__ void __launch_bounds__(kCellThreads, kCellMinCtas<R>)
 }
 
 // --------------------------------------------- cell pass, mirrored ray pairs
-// FP32 cell pass for block edges 8 and 16 and direction sets closed under
-// negation (HEALPix sets are, rotated or not).  The ray from cell c in
+// FP32 cell pass for block edges kMinPairBlock to 16 and direction sets closed
+// under negation (HEALPix sets are, rotated or not).  The ray from cell c in
 // direction d and the ray from the point-mirrored cell c' = (B-1-x, B-1-y,
 // B-1-z) in direction -d are mirror images (and so are (c, -d) and (c', d)):
 // in their own upwind frames both start at the same coordinates along every
@@ -747,8 +750,21 @@ __global__ void __launch_bounds__(kCellThreads, kCellMinCtas<R>)
 // shared-memory addressing is 32-bit (the state of a march is a handful of
 // registers: the pair's intensities, the tile address of the start entries
 // and the event index, which is the same for the whole warp).
-__host__ __device__ constexpr int pair_threads(int B) { return B == 16 ? 1024 : 256; }
-__host__ __device__ constexpr int pair_min_ctas(int B) { return B == 16 ? 1 : 4; }
+// Other edges (BC = 0): the lower half's (B^3 + 1) / 2 cells (of an odd edge's
+// middle cell both rays are its own) over CTAs of up to 512 threads.  Closures
+// of 192 directions in FP32, one ray a thread before, paired now: edge 6, 60^3
+// cells, 1.17 and 0.95 ms; 7, 63^3, 1.35 and 0.96; 10, 80^3, 1.97 and 1.29; 12,
+// 96^3, 3.42 and 2.17; 14, 98^3, 3.96 and 2.68.
+__host__ __device__ constexpr int pair_parts(int B) { return B == 16 ? 2 : (B == 8 ? 1 : ((B * B * B + 1) / 2 + 511) / 512); }
+__host__ __device__ constexpr int pair_threads(int B) {  // whole warps of cells
+  return (((B * B * B + 1) / 2 + pair_parts(B) - 1) / pair_parts(B) + 31) / 32 * 32;
+}
+__host__ __device__ constexpr int pair_min_ctas(int B) {
+  return B == 16 ? 1 : (B == 8 ? 4 : (1024 / pair_threads(B) < 8 ? 1024 / pair_threads(B) : 8));
+}
+// launch bounds of the kernel compiled for block edge BC
+constexpr int pair_max_threads(int BC) { return BC ? pair_threads(BC) : 512; }
+constexpr int pair_bound_ctas(int BC) { return BC ? pair_min_ctas(BC) : 2; }
 constexpr int kPairStagesMax = 16;  // staging ring depth limit of the paired cell pass
 
 // Shared-memory loads at 32-bit shared-window addresses.  volatile keeps
@@ -1008,20 +1024,30 @@ __host__ __device__ inline size_t pair_smem_bytes(int B, int nslots) {
 template <int BC, int NT>
 __device__ __forceinline__ void load_tile_pair(float4 *tile, TileShape ts, const GridDims &g, int bx, int by, int bz,
                                                const float *__restrict__ kappa, const float *__restrict__ S) {
-  constexpr int B = BC, B2 = B * B, K = B2 * B / NT;
-  static_assert(B2 * B % NT == 0, "tile cells must divide evenly over the threads");
-  float4 v[K];
+  if constexpr (BC != 0) {
+    constexpr int B = BC, B2 = B * B, K = B2 * B / NT;
+    static_assert(B2 * B % NT == 0, "tile cells must divide evenly over the threads");
+    float4 v[K];
 #pragma unroll
-  for (int k = 0; k < K; ++k) {
-    const int i = (int)threadIdx.x + k * NT, x = i % B, y = (i / B) % B, z = i / B2;
-    const long long gi = ((long long)(bz * B + z) * g.ny + (by * B + y)) * g.nx + (bx * B + x);
-    const long long gm = ((long long)(bz * B + B - 1 - z) * g.ny + (by * B + B - 1 - y)) * g.nx + (bx * B + B - 1 - x);
-    v[k] = make_float4(kappa[gi], kappa[gm], S[gi], S[gm]);
-  }
+    for (int k = 0; k < K; ++k) {
+      const int i = (int)threadIdx.x + k * NT, x = i % B, y = (i / B) % B, z = i / B2;
+      const long long gi = ((long long)(bz * B + z) * g.ny + (by * B + y)) * g.nx + (bx * B + x);
+      const long long gm = ((long long)(bz * B + B - 1 - z) * g.ny + (by * B + B - 1 - y)) * g.nx + (bx * B + B - 1 - x);
+      v[k] = make_float4(kappa[gi], kappa[gm], S[gi], S[gm]);
+    }
 #pragma unroll
-  for (int k = 0; k < K; ++k) {
-    const int i = (int)threadIdx.x + k * NT, x = i % B, y = (i / B) % B, z = i / B2;
-    tile[x + ts.sy * y + ts.sz * z] = v[k];
+    for (int k = 0; k < K; ++k) {
+      const int i = (int)threadIdx.x + k * NT, x = i % B, y = (i / B) % B, z = i / B2;
+      tile[x + ts.sy * y + ts.sz * z] = v[k];
+    }
+  } else {
+    const int B = g.B, B2 = B * B, B3 = B2 * B;
+    for (int i = threadIdx.x; i < B3; i += blockDim.x) {
+      const int x = i % B, y = (i / B) % B, z = i / B2;
+      const long long gi = ((long long)(bz * B + z) * g.ny + (by * B + y)) * g.nx + (bx * B + x);
+      const long long gm = ((long long)(bz * B + B - 1 - z) * g.ny + (by * B + B - 1 - y)) * g.nx + (bx * B + B - 1 - x);
+      tile[x + ts.sy * y + ts.sz * z] = make_float4(kappa[gi], kappa[gm], S[gi], S[gm]);
+    }
   }
 }
 
@@ -1034,6 +1060,53 @@ __device__ __forceinline__ void kahan2(float2 &s, float2 &nc, float2 c, float2 x
   s = t;
 }
 
+// The moments of an antipodal pair's intensities m1 = (I(c, d), I(c', -d)) and
+// m2 = (I(c, -d), I(c', d)): E and P take I(d) + I(-d), F takes I(d) - I(-d),
+// with the primary direction's coefficient pairs.  E and P_ii go into a staged
+// tile's partial sums pk, which the compensated sums take once per tile, the
+// others straight into mom.  Block edges other than 8 and 16 keep P_ij that way
+// too: their unpaired pass took the octants in turn, whose P_ij cancel; the
+// pairs of one octant pair after another do not, and straight sums of them left
+// f 6.9e-8 off, RMS, where it was 5.9e-8 (edge 6, 192 directions; now 5.6e-8).
+template <int BC>
+struct PairSums {
+  static constexpr int kComp = BC ? 4 : 7;  // compensated sums: E, P_ii (, P_ij)
+  static __device__ __forceinline__ constexpr int comp(int i) { return i ? 3 + i : 0; }
+  float2 mom[10], nc[kComp], pk[kComp];
+  __device__ __forceinline__ PairSums() {
+#pragma unroll
+    for (int m = 0; m < 10; ++m) mom[m] = make_float2(0.f, 0.f);
+#pragma unroll
+    for (int m = 0; m < kComp; ++m) nc[m] = pk[m] = make_float2(0.f, 0.f);
+  }
+  template <bool WANT_F>
+  __device__ __forceinline__ void add(float4 c01, float4 c23, float4 c45, float4 c67, float4 c89, float2 m1, float2 m2) {
+    const float2 c[10] = {make_float2(c01.x, c01.y), make_float2(c01.z, c01.w), make_float2(c23.x, c23.y), make_float2(c23.z, c23.w),
+                          make_float2(c45.x, c45.y), make_float2(c45.z, c45.w), make_float2(c67.x, c67.y), make_float2(c67.z, c67.w),
+                          make_float2(c89.x, c89.y), make_float2(c89.z, c89.w)};
+    const float2 sum = __fadd2_rn(m1, m2), dif = __fadd2_rn(m1, neg2(m2));
+    pk[0] = __ffma2_rn(c[0], sum, pk[0]);
+    if (WANT_F) {
+#pragma unroll
+      for (int m = 1; m < 4; ++m) mom[m] = __ffma2_rn(c[m], dif, mom[m]);
+    }
+#pragma unroll
+    for (int m = 4; m < 10; ++m) {
+      if (m < 7 || BC == 0) pk[m - 3] = __ffma2_rn(c[m], sum, pk[m - 3]);
+      else mom[m] = __ffma2_rn(c[m], sum, mom[m]);
+    }
+  }
+  // a staged tile's partial sums into the compensated sums
+  __device__ __forceinline__ void fold() {
+    const float2 one = make_float2(1.f, 1.f);
+#pragma unroll
+    for (int i = 0; i < kComp; ++i) {
+      kahan2(mom[comp(i)], nc[i], one, pk[i]);
+      pk[i] = make_float2(0.f, 0.f);
+    }
+  }
+};
+
 // the head fields the paired cell pass reads at fixed offsets
 static_assert(offsetof(TplHead<float>, sgn) == 16 && offsetof(TplHead<float>, ext) == 28 &&
                   offsetof(TplHead<float>, mirror) == 32 && offsetof(TplHead<float>, cp) % 16 == 0,
@@ -1044,16 +1117,32 @@ static_assert(offsetof(TplHead<float>, sgn) == 16 && offsetof(TplHead<float>, ex
 // block, part 0 takes layer pairs 0 and 3 and part 1 takes 1 and 2 (85e3 and
 // 89e3 warp steps over 192 directions, where z-order parts differ by 15%), so
 // that the CTAs of a wave carry about equal work.
-template <int B>
+template <int BC>
 struct PairCell {
-  int q, x, y, z;  // place among the part's cells; the cell
-  __device__ __forceinline__ PairCell(int part, int parts, uint32_t tid) {
-    q = part * pair_threads(B) + (int)tid;
+  int B, q, x, y, z;  // place among the lower half's cells; the cell
+  bool active;        // false: a thread past the CTA's cells (it redoes the last one and writes nothing)
+  __device__ __forceinline__ PairCell(int edge, int part, int parts, uint32_t tid) {
+    B = BC ? BC : edge;
+    if constexpr (BC != 0) {
+      q = part * pair_threads(BC) + (int)tid;
+      active = true;
+    } else {
+      const int half = (B * B * B + 1) / 2;
+      q = part * pair_threads(B) + (int)tid;
+      active = q < half;
+      q = min(q, half - 1);
+    }
+    if (BC == 0 && B % 4) {
+      x = q % B;
+      y = (q / B) % B;
+      z = q / (B * B);
+      return;
+    }
     const int qb = q >> 5, ln = q & 31;
     x = 4 * (qb % (B / 4)) + (ln & 3);
     y = 4 * ((qb / (B / 4)) % (B / 4)) + ((ln >> 2) & 3);
     int lp = qb / (B * B / 16);
-    if (B == 16 && parts == 2) lp = (0x2130 >> (4 * lp)) & 15;
+    if (BC == 16 && parts == 2) lp = (0x2130 >> (4 * lp)) & 15;
     z = 2 * lp + (ln >> 4);
   }
   __device__ __forceinline__ long long cell(const GridDims &g, int bx, int by, int bz) const {
@@ -1073,7 +1162,7 @@ __device__ __forceinline__ uint32_t fresh_tid() {
 
 // ORDERED (moment modes): every CTA is one share of a work item, see TailPlan.
 template <int MODE, int BC, bool MERGED, bool ORDERED = false>
-__global__ void __launch_bounds__(pair_threads(BC), pair_min_ctas(BC))
+__global__ void __launch_bounds__(pair_max_threads(BC), pair_bound_ctas(BC))
     cell_pair_kernel(GridDims g_arg, int parts, int dt, int nstage, const float *__restrict__ kappa_arg,
                      const float *__restrict__ S_arg, const unsigned char *__restrict__ tpl_arg,
                      const int *__restrict__ order_arg, const float *__restrict__ faces_arg,
@@ -1082,7 +1171,6 @@ __global__ void __launch_bounds__(pair_threads(BC), pair_min_ctas(BC))
                      int *status_arg, const int *__restrict__ block_list, int nfull, int ksplit,
                      float *__restrict__ split_part, int *__restrict__ split_count,
                      const CellGrid *__restrict__ grids, const int2 *__restrict__ items) {
-  constexpr int B = BC, B2 = B * B, NT = pair_threads(BC);
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ __align__(8) uint64_t full[kPairStagesMax], empty[kPairStagesMax];
   constexpr int kOrdMax = 1024;  // direction sets up to nside = 8 keep their order in shared memory
@@ -1103,6 +1191,7 @@ __global__ void __launch_bounds__(pair_threads(BC), pair_min_ctas(BC))
   float *__restrict__ f_out = MERGED ? gd->f_out : f_arg;
   void *emax_bits = MERGED ? gd->emax_bits : emax_arg;
   int *status = MERGED ? gd->status : status_arg;
+  const int B = BC ? BC : g.B, B2 = B * B, NT = BC ? pair_threads(BC) : (int)blockDim.x;
   const bool ord_smem = g.ndir <= kOrdMax;
   const TileShape ts = cell_tile(B);
   const TplLayout TL = tpl_layout<float>(B);
@@ -1126,7 +1215,7 @@ __global__ void __launch_bounds__(pair_threads(BC), pair_min_ctas(BC))
   const int item = cta / parts, part = parts - 1 - (cta - item * parts);
   const int blk = MERGED ? items[item].y : (block_list ? block_list[item] : item);
   const int bx = blk % g.nbx, by = (blk / g.nbx) % g.nby, bz = blk / (g.nbx * g.nby);
-  constexpr int nwarps = NT / 32;
+  const int nwarps = NT / 32;
   const int ntiles_all = (g.ndir + dt - 1) / dt, nshares = slot >= 0 ? ksplit : 1;
   const int tile0 = share * ntiles_all / nshares, ntiles = (share + 1) * ntiles_all / nshares - tile0;
   // producer state, meaningful in thread 0 only; tiles counted from tile0
@@ -1152,31 +1241,24 @@ __global__ void __launch_bounds__(pair_threads(BC), pair_min_ctas(BC))
   }
   if (ord_smem)
     for (int i = threadIdx.x; i < g.ndir; i += NT) s_ord[i] = order[i];
-  load_tile_pair<BC, NT>(tile, ts, g, bx, by, bz, kappa, S);
-  if (threadIdx.x == 0) tile[B] = make_float4(0.f, 0.f, 0.f, 0.f);  // identity entry (padding, x = B)
+  load_tile_pair<BC, BC ? pair_threads(BC) : 0>(tile, ts, g, bx, by, bz, kappa, S);
+  if (threadIdx.x == 0) tile[ts.elems - 1] = make_float4(0.f, 0.f, 0.f, 0.f);  // identity entry
   __syncthreads();
 
-  const PairCell<BC> pc(part, parts, threadIdx.x);
+  const PairCell<BC> pc(B, part, parts, threadIdx.x);
   const uint32_t tile_s = smem_u32(tile);
   const uint32_t t1 = tile_s + 16u * (uint32_t)(pc.x + ts.sy * pc.y + ts.sz * pc.z);
   constexpr bool kWantF = MODE == 0;
   // moments of (c, c') as packed pairs: E, Fx, Fy, Fz, Pxx, Pyy, Pzz, Pxy,
   // Pxz, Pyz; compensated E and Pii (nc: their negated compensations), which
-  // a staged tile's pairs add into plain partial sums pk first, folded into
-  // the compensated sums once per tile (fewer f32x2 operations and fewer
+  // a staged tile's pairs add into plain partial sums first, folded into the
+  // compensated sums once per tile (fewer f32x2 operations and fewer
   // register moves than a compensated addition per pair)
-  float2 mom[10], nc[4];
-#pragma unroll
-  for (int m = 0; m < 10; ++m) mom[m] = make_float2(0.f, 0.f);
-#pragma unroll
-  for (int m = 0; m < 4; ++m) nc[m] = make_float2(0.f, 0.f);
-  float2 pk[4];  // plain partial sums of the compensated moments over one tile
-#pragma unroll
-  for (int m = 0; m < 4; ++m) pk[m] = make_float2(0.f, 0.f);
-  // a tile padding entry (x = B) set to zero: the identity segment
-  const uint32_t id_s = tile_s + 16u * (uint32_t)B;
-  constexpr int W = B + 2;
-  const uint32_t fW = 4u * W;
+  PairSums<BC> ps;
+  float2(&mom)[10] = ps.mom, (&nc)[PairSums<BC>::kComp] = ps.nc;
+  // the tile entry set to zero: the identity segment
+  const uint32_t id_s = tile_s + 16u * (uint32_t)(ts.elems - 1);
+  const uint32_t fW = 4u * (uint32_t)(B + 2);
 
   // Entry value of the ray(s) of one march, by its record: primary slot ps
   // (its weights), faces f1 (primary) and f2 (the pair's second ray).
@@ -1204,7 +1286,7 @@ __global__ void __launch_bounds__(pair_threads(BC), pair_min_ctas(BC))
   // (slot ps), the record of its start cell in that direction
   auto single = [&](uint32_t ps, int k, bool mirror_cell) -> float {
     const int v = ord_smem ? s_ord[k] : __ldg(order + k);
-    const PairCell<BC> c(part, parts, fresh_tid());
+    const PairCell<BC> c(B, part, parts, fresh_tid());
     const int x = mirror_cell ? B - 1 - c.x : c.x, y = mirror_cell ? B - 1 - c.y : c.y, z = mirror_cell ? B - 1 - c.z : c.z;
     const uint32_t tstart = tile_s + 16u * (uint32_t)(x + ts.sy * y + ts.sz * z);
     const uint32_t *r = g.cell_rec + (size_t)order_dir(v) * (B * B2) + cell_rec_index(B, x, y, z);
@@ -1258,47 +1340,25 @@ __global__ void __launch_bounds__(pair_threads(BC), pair_min_ctas(BC))
       if (MODE == 1) {
         const int ea = (int)lds_2x32(sa + 24).y, eb = (int)lds_2x32(sb + 24).y;  // the directions' public indices
         const long long gc1 = pc.cell(g, bx, by, bz), gc2 = pc.mirror(g, bx, by, bz);
-        I_out[(long long)ea * g.ncell + gc1] = m1.x;
-        I_out[(long long)eb * g.ncell + gc2] = m1.y;
-        I_out[(long long)eb * g.ncell + gc1] = m2.x;
-        I_out[(long long)ea * g.ncell + gc2] = m2.y;
+        if (pc.active) {
+          I_out[(long long)ea * g.ncell + gc1] = m1.x;
+          I_out[(long long)eb * g.ncell + gc2] = m1.y;
+          I_out[(long long)eb * g.ncell + gc1] = m2.x;
+          I_out[(long long)ea * g.ncell + gc2] = m2.y;
+        }
       } else if (ORDERED) {
         // this pair's place in the item's list: pairs are consecutive in the order
         const int pair = ((tile0 + t) * dt + j) >> 1;
         float2 *dst = reinterpret_cast<float2 *>(split_part) +
                       ((size_t)slot * (g.ndir >> 1) + pair) * 2 * NT + threadIdx.x;
-        __stcg(dst, __fadd2_rn(m1, m2));
-        if (kWantF) __stcg(dst + NT, __fadd2_rn(m1, neg2(m2)));
+        __stcg(dst, m1);
+        __stcg(dst + NT, m2);
       } else {
-        // E and P take I(d) + I(-d), F takes I(d) - I(-d), with the primary
-        // direction's coefficient pairs
-        const float2 sum = __fadd2_rn(m1, m2), dif = __fadd2_rn(m1, neg2(m2));
         const uint32_t cpa = sa + (uint32_t)offsetof(TplHead<float>, cp);
-        const float4 c01 = lds_f4(cpa), c23 = lds_f4(cpa + 16), c45 = lds_f4(cpa + 32), c67 = lds_f4(cpa + 48),
-                     c89 = lds_f4(cpa + 64);
-        pk[0] = __ffma2_rn(make_float2(c01.x, c01.y), sum, pk[0]);
-        if (kWantF) {
-          mom[1] = __ffma2_rn(make_float2(c01.z, c01.w), dif, mom[1]);
-          mom[2] = __ffma2_rn(make_float2(c23.x, c23.y), dif, mom[2]);
-          mom[3] = __ffma2_rn(make_float2(c23.z, c23.w), dif, mom[3]);
-        }
-        pk[1] = __ffma2_rn(make_float2(c45.x, c45.y), sum, pk[1]);
-        pk[2] = __ffma2_rn(make_float2(c45.z, c45.w), sum, pk[2]);
-        pk[3] = __ffma2_rn(make_float2(c67.x, c67.y), sum, pk[3]);
-        mom[7] = __ffma2_rn(make_float2(c67.z, c67.w), sum, mom[7]);
-        mom[8] = __ffma2_rn(make_float2(c89.x, c89.y), sum, mom[8]);
-        mom[9] = __ffma2_rn(make_float2(c89.z, c89.w), sum, mom[9]);
+        ps.template add<kWantF>(lds_f4(cpa), lds_f4(cpa + 16), lds_f4(cpa + 32), lds_f4(cpa + 48), lds_f4(cpa + 64), m1, m2);
       }
     }
-    if (MODE != 1 && !ORDERED) {  // the tile's plain partial sums into the compensated ones
-      const float2 one = make_float2(1.f, 1.f);
-      kahan2(mom[0], nc[0], one, pk[0]);
-      kahan2(mom[4], nc[1], one, pk[1]);
-      kahan2(mom[5], nc[2], one, pk[2]);
-      kahan2(mom[6], nc[3], one, pk[3]);
-#pragma unroll
-      for (int m = 0; m < 4; ++m) pk[m] = make_float2(0.f, 0.f);
-    }
+    if (MODE != 1 && !ORDERED) ps.fold();
     __syncwarp();
     if ((threadIdx.x & 31) == 0) mbar_arrive(&empty[st]);
     if (threadIdx.x == 0) {
@@ -1329,37 +1389,20 @@ __global__ void __launch_bounds__(pair_threads(BC), pair_min_ctas(BC))
 #pragma unroll 4
       for (int j = 0; j < nd; j += 2) {
         const int pair = (d0 + j) >> 1;
-        const float2 sum = __ldcg(src + (size_t)pair * 2 * NT);
-        const float2 dif = kWantF ? __ldcg(src + (size_t)pair * 2 * NT + NT) : one;
+        const float2 m1 = __ldcg(src + (size_t)pair * 2 * NT), m2 = __ldcg(src + (size_t)pair * 2 * NT + NT);
         const int v = ord_smem ? s_ord[d0 + j] : order[d0 + j];
         const float4 *cp = reinterpret_cast<const float4 *>(tpl_g + (size_t)order_dir(v) * TL.bytes +
                                                             offsetof(TplHead<float>, cp));
-        const float4 c01 = __ldg(cp), c23 = __ldg(cp + 1), c45 = __ldg(cp + 2), c67 = __ldg(cp + 3), c89 = __ldg(cp + 4);
-        pk[0] = __ffma2_rn(make_float2(c01.x, c01.y), sum, pk[0]);
-        if (kWantF) {
-          mom[1] = __ffma2_rn(make_float2(c01.z, c01.w), dif, mom[1]);
-          mom[2] = __ffma2_rn(make_float2(c23.x, c23.y), dif, mom[2]);
-          mom[3] = __ffma2_rn(make_float2(c23.z, c23.w), dif, mom[3]);
-        }
-        pk[1] = __ffma2_rn(make_float2(c45.x, c45.y), sum, pk[1]);
-        pk[2] = __ffma2_rn(make_float2(c45.z, c45.w), sum, pk[2]);
-        pk[3] = __ffma2_rn(make_float2(c67.x, c67.y), sum, pk[3]);
-        mom[7] = __ffma2_rn(make_float2(c67.z, c67.w), sum, mom[7]);
-        mom[8] = __ffma2_rn(make_float2(c89.x, c89.y), sum, mom[8]);
-        mom[9] = __ffma2_rn(make_float2(c89.z, c89.w), sum, mom[9]);
+        ps.template add<kWantF>(__ldg(cp), __ldg(cp + 1), __ldg(cp + 2), __ldg(cp + 3), __ldg(cp + 4), m1, m2);
       }
-      kahan2(mom[0], nc[0], one, pk[0]);
-      kahan2(mom[4], nc[1], one, pk[1]);
-      kahan2(mom[5], nc[2], one, pk[2]);
-      kahan2(mom[6], nc[3], one, pk[3]);
-#pragma unroll
-      for (int m = 0; m < 4; ++m) pk[m] = make_float2(0.f, 0.f);
+      ps.fold();
     }
     if (threadIdx.x == 0) split_count[slot] = 0;  // ready for the next call
   } else if (MODE != 1 && slot >= 0) {
     // one share of a split work item: its partial sums go to the slot's
     // scratch, and the share that finishes last adds the others' (the
-    // compensated sums as compensated sums) and writes the outputs
+    // compensated sums as compensated sums, but for P_ij's last compensation)
+    // and writes the outputs
     constexpr int kVals = 28;
     __shared__ int s_last;
     float *mine = split_part + ((size_t)slot * ksplit + share) * kVals * NT + threadIdx.x;
@@ -1407,8 +1450,10 @@ __global__ void __launch_bounds__(pair_threads(BC), pair_min_ctas(BC))
     // over the CTA's 2L layers, then written row by row, so that every
     // warp writes runs of B consecutive cells of a component (a host-mapped
     // output then crosses the host link in whole runs, not 16-byte pieces)
-    constexpr int L = NT / B2, CELLS = 2 * NT, NV = kWantF ? 16 : 7, NM = kWantF ? 10 : 1;
-    const bool staged = (size_t)nstage * stage_bytes >= sizeof(float) * NV * CELLS;
+    // (block edges 8 and 16, whose CTAs hold whole layers; others write cell by cell).
+    constexpr int NV = kWantF ? 16 : 7, NM = kWantF ? 10 : 1;
+    const int L = NT / B2, CELLS = 2 * NT;
+    const bool staged = BC != 0 && (size_t)nstage * stage_bytes >= sizeof(float) * NV * CELLS;
     float emax = 0.f;
     if (__syncthreads_and(ok)) {  // also: every warp is done with the ring
       float Ms[2][10];
@@ -1418,7 +1463,7 @@ __global__ void __launch_bounds__(pair_threads(BC), pair_min_ctas(BC))
         Ms[1][m] = mom[m].y;
       }
       float *st = reinterpret_cast<float *>(ring);
-      const PairCell<BC> c(part, parts, fresh_tid());
+      const PairCell<BC> c(B, part, parts, fresh_tid());
       const int zs = 2 * ((c.q >> 5) / (B2 / 16) - part * (L / 2)) + ((c.q & 31) >> 4);  // the lower cell's z slot
       const int li[2] = {(zs * B + c.y) * B + c.x, ((L + zs) * B + B - 1 - c.y) * B + B - 1 - c.x};
 #pragma unroll
@@ -1438,7 +1483,7 @@ __global__ void __launch_bounds__(pair_threads(BC), pair_min_ctas(BC))
         if (staged) {
 #pragma unroll
           for (int m = 0; m < NV; ++m) st[m * CELLS + li[r]] = v[m];
-        } else {
+        } else if (c.active) {
 #pragma unroll
           for (int m = 0; m < NV; ++m) {
             float *dst = m < NM ? (kWantF ? M_out + m * g.ncell : E_out) : f_out + (m - NM) * g.ncell;
@@ -1452,7 +1497,7 @@ __global__ void __launch_bounds__(pair_threads(BC), pair_min_ctas(BC))
         for (int i = threadIdx.x; i < CELLS; i += NT) {
           const int zsl = i / B2, y = (i / B) % B, x = i % B, zl = zsl < L ? zsl : zsl - L;
           int lp = part * (L / 2) + (zl >> 1);
-          if (B == 16 && parts == 2) lp = (0x2130 >> (4 * lp)) & 15;
+          if (BC == 16 && parts == 2) lp = (0x2130 >> (4 * lp)) & 15;
           const int z = zsl < L ? 2 * lp + (zl & 1) : B - 1 - (2 * lp + (zl & 1));
           const long long gi = ((long long)(bz * B + z) * g.ny + (by * B + y)) * g.nx + (bx * B + x);
 #pragma unroll
@@ -1469,7 +1514,7 @@ __global__ void __launch_bounds__(pair_threads(BC), pair_min_ctas(BC))
 }
 
 // ------------------------------------------- face pass, mirrored block pairs
-// FP32 face pass for block edges 8 and 16 and direction sets closed under
+// FP32 face pass for block edges up to 16 and direction sets closed under
 // negation with no zero component.  The node ray of block b in direction d
 // from upwind-frame node coordinates L and the node ray of the point-mirrored
 // block b' (nb - 1 - b per axis) in direction -d from the same L are mirror
@@ -1487,7 +1532,18 @@ template <int BC, int NT>
 __device__ __forceinline__ void load_tile_mirrored(float4 *tile, TileShape ts, const GridDims &g, int bx, int by,
                                                    int bz, int mx, int my, int mz, const float *__restrict__ kappa,
                                                    const float *__restrict__ S) {
-  constexpr int B = BC, B2 = B * B, K = B2 * B / NT;
+  if constexpr (BC == 0) {
+    const int B = g.B, B2 = B * B, B3 = B2 * B;
+    for (int i = threadIdx.x; i < B3; i += NT) {
+      const int x = i % B, y = (i / B) % B, z = i / B2;
+      const long long gi = ((long long)(bz * B + z) * g.ny + (by * B + y)) * g.nx + (bx * B + x);
+      const long long gm =
+          ((long long)(mz * B + B - 1 - z) * g.ny + (my * B + B - 1 - y)) * g.nx + (mx * B + B - 1 - x);
+      tile[x + ts.sy * y + ts.sz * z] = make_float4(kappa[gi], kappa[gm], S[gi], S[gm]);
+    }
+    return;
+  }
+  constexpr int B = BC ? BC : 8, B2 = B * B, K = B2 * B / NT;
   static_assert(B2 * B % NT == 0, "tile cells must divide evenly over the threads");
   float4 v[K];
 #pragma unroll
@@ -1518,7 +1574,7 @@ __global__ void __launch_bounds__(kFaceThreads, 2)
                      float *__restrict__ faces, const float *__restrict__ bnd, long long spin_limit, int *status) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ __align__(8) uint64_t full;
-  constexpr int B = BC, W = B + 2, N1 = B + 1, NN = N1 * N1;
+  const int B = BC ? BC : g.B, W = B + 2, N1 = B + 1, NN = N1 * N1;
   const TileShape ts = node_tile(B);
   const TplLayout TL = tpl_layout<float>(B);
   const size_t sb = face_slot_bytes_t<float>(B), fb3 = faces_bytes<float>(B);
@@ -1787,7 +1843,7 @@ int cell_parts(int B) {
 template <typename R, int BC>
 void face_launch(const GridDims &g, const R *kappa, const R *S, const unsigned char *tpl, const FaceItem *items,
                  int nitems, int max_dirs, R *faces, const R *bnd, long long spin, int *status, cudaStream_t st) {
-  if constexpr (sizeof(R) == sizeof(float) && BC != 0) {
+  if constexpr (sizeof(R) == sizeof(float)) {
     if (g.face_paired) {
       cudaLaunchConfig_t cfg = {};
       cudaLaunchAttribute attr[1];
@@ -1795,7 +1851,7 @@ void face_launch(const GridDims &g, const R *kappa, const R *S, const unsigned c
       attr[0].val.programmaticStreamSerializationAllowed = 1;
       cfg.gridDim = dim3(nitems);
       cfg.blockDim = dim3(kFaceThreads);
-      cfg.dynamicSmemBytes = face_pair_smem_bytes(BC, max_dirs);
+      cfg.dynamicSmemBytes = face_pair_smem_bytes(g.B, max_dirs);
       cfg.stream = st;
       cfg.attrs = attr;
       cfg.numAttrs = 1;
@@ -1838,7 +1894,9 @@ inline void pair_staging(int B, int want, int &dt, int &nstage) {
   constexpr long long kSmemPerSM = 233472, kReservedPerCta = 1024;
   constexpr long long kStatic = 1024 * 4 + 2 * kPairStagesMax * 8 + 64;  // order, barriers, margin
   const long long per_cta = std::min<long long>(232448, kSmemPerSM / pair_min_ctas(B) - kReservedPerCta) - kStatic;
-  dt = want > 0 ? want : 8;  // untuned: the tile the autotuner picks on the 128^3 workload
+  // untuned: the tile the autotuner picks on the 128^3 workload; other edges keep
+  // the unpaired pass's 4, and with it its plain sums of at most four directions
+  dt = want > 0 ? want : (B == 8 || B == 16 ? 8 : 4);
   dt = (dt + 1) & ~1;
   if (dt > kMaxTune) dt = kMaxTune;
   for (;;) {
@@ -1853,8 +1911,7 @@ inline void pair_staging(int B, int want, int &dt, int &nstage) {
 
 TailPlan plan_tail_split(int B, int nblk, int nsm, int ndir, int dir_tile) {
   TailPlan p;
-  if (B != 8 && B != 16) return p;
-  const int parts = B * B * B / 2 / pair_threads(B), total = nblk * parts, ntiles = (ndir + dir_tile - 1) / dir_tile;
+  const int parts = pair_parts(B), total = nblk * parts, ntiles = (ndir + dir_tile - 1) / dir_tile;
   p.nfull = total;
   const int wave = nsm * pair_min_ctas(B);
   if (nsm <= 0) return p;
@@ -1898,15 +1955,15 @@ void pair_launch(const GridDims &g, const float *kappa, const float *S, const un
                  const float *faces, const float *bnd, float *I_out, float *M_out, float *E_out, float *f_out,
                  void *emax_bits, long long spin, int *status, const int *block_list, int nlist, cudaStream_t st,
                  const TailSplit *split) {
-  const int parts = BC * BC * BC / 2 / pair_threads(BC);
+  const int B = BC ? BC : g.B, parts = pair_parts(B);
   const int nblk = block_list ? nlist : g.nbx * g.nby * g.nbz;
   int dt, nstage;
-  pair_staging(BC, g.dir_tile, dt, nstage);
+  pair_staging(B, g.dir_tile, dt, nstage);
   // the tail split: whole grids only; the moment passes need its scratch
   TailPlan tp;
   tp.nfull = nblk * parts;
   if (split && !block_list) {
-    const TailPlan q = plan_tail_split(BC, nblk, split->nsm, g.ndir, dt);
+    const TailPlan q = plan_tail_split(B, nblk, split->nsm, g.ndir, dt);
     const bool room = MODE == 1 || (split->part && split->count && q.part_bytes <= split->part_bytes &&
                                     q.slots <= split->slots);
     if (q.k > 1 && room) tp = q;
@@ -1917,8 +1974,8 @@ void pair_launch(const GridDims &g, const float *kappa, const float *S, const un
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // prologue overlaps the face pass's end
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.gridDim = dim3(grid);
-  cfg.blockDim = dim3(pair_threads(BC));
-  cfg.dynamicSmemBytes = pair_smem_bytes(BC, nstage * dt);
+  cfg.blockDim = dim3(pair_threads(B));
+  cfg.dynamicSmemBytes = pair_smem_bytes(B, nstage * dt);
   cfg.stream = st;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
@@ -1936,7 +1993,7 @@ void pair_launch(const GridDims &g, const float *kappa, const float *S, const un
 template <int MODE, int BC>
 void pair_launch_merged(int dir_tile, const CellGrid *grids, const int2 *items, int nitems, long long spin,
                         cudaStream_t st) {
-  const int parts = BC * BC * BC / 2 / pair_threads(BC);
+  const int parts = pair_parts(BC);
   int dt, nstage;
   pair_staging(BC, dir_tile, dt, nstage);
   cudaLaunchConfig_t cfg = {};
@@ -1972,7 +2029,11 @@ cudaError_t set_smem_attrs() {
                         (const void *)cell_pair_kernel<2, 8, true>,   (const void *)cell_pair_kernel<2, 16, true>,
                         (const void *)cell_pair_kernel<0, 8, false, true>, (const void *)cell_pair_kernel<0, 16, false, true>,
                         (const void *)cell_pair_kernel<2, 8, false, true>, (const void *)cell_pair_kernel<2, 16, false, true>,
-                        (const void *)face_pair_kernel<8>,            (const void *)face_pair_kernel<16>};
+                        (const void *)cell_pair_kernel<0, 0, false>,  (const void *)cell_pair_kernel<2, 0, false>,
+                        (const void *)cell_pair_kernel<1, 0, false>,  (const void *)cell_pair_kernel<0, 0, false, true>,
+                        (const void *)cell_pair_kernel<2, 0, false, true>,
+                        (const void *)face_pair_kernel<0>,            (const void *)face_pair_kernel<8>,
+                        (const void *)face_pair_kernel<16>};
   for (const void *f : pfns) {  // less their static shared memory
     cudaFuncAttributes fa;
     cudaError_t e = cudaFuncGetAttributes(&fa, f);
@@ -2018,7 +2079,7 @@ cudaError_t launch_cell_pass(const GridDims &g, int mode, const R *kappa, const 
                              const int *block_list, int nlist, const TailSplit *split) {
   if (block_list && nlist <= 0) return cudaSuccess;
   if constexpr (sizeof(R) == sizeof(float)) {
-    if (g.paired && (g.B == 16 || g.B == 8)) {
+    if (g.paired) {
       const float *k = reinterpret_cast<const float *>(kappa), *s = reinterpret_cast<const float *>(S);
       const float *fc = reinterpret_cast<const float *>(faces), *bd = reinterpret_cast<const float *>(bnd);
       float *Io = reinterpret_cast<float *>(I_out), *Mo = reinterpret_cast<float *>(M_out);
@@ -2031,10 +2092,14 @@ cudaError_t launch_cell_pass(const GridDims &g, int mode, const R *kappa, const 
         if (mode2 == 0) VET_PAIR(0, 16);
         else if (mode2 == 2) VET_PAIR(2, 16);
         else VET_PAIR(1, 16);
-      } else {
+      } else if (g.B == 8) {
         if (mode2 == 0) VET_PAIR(0, 8);
         else if (mode2 == 2) VET_PAIR(2, 8);
         else VET_PAIR(1, 8);
+      } else {
+        if (mode2 == 0) VET_PAIR(0, 0);
+        else if (mode2 == 2) VET_PAIR(2, 0);
+        else VET_PAIR(1, 0);
       }
 #undef VET_PAIR
       return cudaGetLastError();
