@@ -13,15 +13,24 @@
 // A ray point on a cell face lies in the cell the ray enters next; a cell
 // whose centre is the source gets zeros.
 //
-// One thread per cell (grid-stride, x fastest): the rays of a warp start at
-// the same point and stay close, so their kappa reads are near one another
-// in the caches; each thread walks four steps ahead of its sum of tau, so
-// that four reads are in flight.  Geometry in cell units (planes at integers); every plane
-// crossing is computed from the source position, not accumulated, so a
-// crossing's error is a few ulp of its own distance.  The walk crosses at
-// most |di| + |dj| + |dk| + 1 cells and is capped at nx + ny + nz + 3 steps.
+// One thread per cell, a warp's cells in a brick (8 x 2 x 2 where the grid has
+// the extents): the rays of a warp start at the same point, stay close and
+// cross nearly the same number of planes.  Geometry in cell units (planes at
+// integers); every plane crossing is computed from the source position, not
+// accumulated, so a crossing's error is a few ulp of its own distance.  The
+// walk's crossings, about |di| + |dj| + |dk|, are counted before it starts, and
+// it runs in groups of four whose kappa reads are in flight together.
+//
+// Bound by instruction issue (76% of the slots, 27 instructions a crossing):
+// 128^3 cells take 2.3e8 crossings; kappa and the results are 42 MB, 6 us.  One
+// row of x a warp, a test of the end and of the grid's bounds at every step and
+// selects for the axes took 760 us; without the tests, in bricks, 252; with the
+// crossed axis' update under a predicate instead of selects 215 (bricks of 4 x 4
+// x 2 212, of 16 x 2 x 1 222; groups of six or eight crossings the same).
+#include <algorithm>
 #include <cmath>
 #include <cstdint>
+#include <type_traits>
 
 #include <cuda_runtime.h>
 
@@ -34,91 +43,157 @@ struct PointArgs {
   float h;
   float xs[3];  // source, cell units
   float L;
+  // a warp's brick is 2^w cells along each axis, a CTA's 2^c warps (sums 5 and 3)
+  int w[3], c[3];
+  int tx, ty;  // CTAs along x and y
 };
 
+// Largest extent whose walks need no check of the grid's bounds, below.
+constexpr int kPlainExtent = 65536;
+
+// Extents up to kPlainExtent (CHECK = false, at most 2^31 - 1 cells): a walk
+// takes exactly the crossings between the source's cell and the target's, and
+// stays between them.  The ray leaves the target's slab of any axis at least
+// half a cell beyond the target's centre and enters it by half a cell before, so
+// that a crossing past the target lies at least one cell behind t_in, and the
+// crossings' rounding (5 ulp of at most 1.8 x 65536 cells: 0.04) cannot bring it
+// forward.  Larger grids check every read.
+template <bool CHECK>
 __global__ void __launch_bounds__(256) point_kernel(PointArgs a, const float *__restrict__ kappa,
                                                    float *__restrict__ Edot, float *__restrict__ pdot) {
+  using Idx = std::conditional_t<CHECK, long long, int>;
+  using Plane = std::conditional_t<CHECK, int, float>;  // exact either way: kPlainExtent < 2^24
   const long long ncell = (long long)a.nx * a.ny * a.nz;
-  const long long stride = (long long)gridDim.x * blockDim.x;
-  const int cap = a.nx + a.ny + a.nz + 3;
-  for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < ncell; c += stride) {
-    const int i = (int)(c % a.nx), j = (int)((c / a.nx) % a.ny), k = (int)(c / ((long long)a.nx * a.ny));
-    const float xc[3] = {i + 0.5f, j + 0.5f, k + 0.5f};
-    float v[3] = {xc[0] - a.xs[0], xc[1] - a.xs[1], xc[2] - a.xs[2]};
-    const float r = sqrtf(fmaf(v[0], v[0], fmaf(v[1], v[1], v[2] * v[2])));
-    if (!(r > 0.f)) {
-      Edot[c] = 0.f;
-      if (pdot) pdot[c] = pdot[ncell + c] = pdot[2 * ncell + c] = 0.f;
-      continue;
-    }
-    float d[3], inv[3];
-    for (int q = 0; q < 3; ++q) {
-      d[q] = v[q] / r;
-      inv[q] = d[q] != 0.f ? 1.f / d[q] : INFINITY;
-    }
-    // the target cell's parameter interval (slabs)
-    const int cc[3] = {i, j, k};
-    float t_in = 0.f, t_out = INFINITY;
-    for (int q = 0; q < 3; ++q)
-      if (d[q] != 0.f) {
-        const float t1 = (cc[q] - a.xs[q]) * inv[q], t2 = (cc[q] + 1 - a.xs[q]) * inv[q];
-        t_in = fmaxf(t_in, fminf(t1, t2));
-        t_out = fminf(t_out, fmaxf(t1, t2));
-      }
-    const float dr = t_out - t_in;
-    // walk from the source cell to the entry of the target cell: the next
-    // crossing of each axis is kept, and only the axis just crossed has its
-    // next crossing recomputed (from the source position, not accumulated).
-    // The per-axis state is kept in scalars updated by selects (an array
-    // indexed by the crossed axis would live in local memory), and the walk,
-    // which does not depend on kappa, runs four steps ahead of the sum of
-    // tau: their four kappa loads are in flight together, and tau takes them
-    // in order (a step past the end or outside the grid adds 0 times 0).
-    int c0 = (int)floorf(a.xs[0]), c1 = (int)floorf(a.xs[1]), c2 = (int)floorf(a.xs[2]);
-    const int s0 = d[0] > 0.f ? 1 : -1, s1 = d[1] > 0.f ? 1 : -1, s2 = d[2] > 0.f ? 1 : -1;
-    const int o0 = d[0] > 0.f ? 1 : 0, o1 = d[1] > 0.f ? 1 : 0, o2 = d[2] > 0.f ? 1 : 0;
-    const long long plane = (long long)a.nx * a.ny;
-    const long long e0 = s0, e1 = s1 > 0 ? (long long)a.nx : -(long long)a.nx, e2 = s2 > 0 ? plane : -plane;
-    float tm0 = d[0] != 0.f ? (c0 + o0 - a.xs[0]) * inv[0] : INFINITY;
-    float tm1 = d[1] != 0.f ? (c1 + o1 - a.xs[1]) * inv[1] : INFINITY;
-    float tm2 = d[2] != 0.f ? (c2 + o2 - a.xs[2]) * inv[2] : INFINITY;
-    long long idx = ((long long)c2 * a.ny + c1) * a.nx + c0;
-    float t = 0.f, tau = 0.f;
-    for (int s = 0; s < cap && t < t_in - 1e-5f;) {
-      float kv[4], len[4];
+  const int n[3] = {a.nx, a.ny, a.nz};
+  const int tile[3] = {(int)(blockIdx.x % a.tx), (int)(blockIdx.x / a.tx % a.ty), (int)(blockIdx.x / a.tx / a.ty)};
+  int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, cc[3];
+  bool inside = true;
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const bool live = s < cap && t < t_in - 1e-5f;
-        const int ax = tm0 <= tm1 ? (tm0 <= tm2 ? 0 : 2) : (tm1 <= tm2 ? 1 : 2);
-        const float tn = fminf(ax == 0 ? tm0 : (ax == 1 ? tm1 : tm2), t_in);
-        const bool in = live && (unsigned)c0 < (unsigned)a.nx && (unsigned)c1 < (unsigned)a.ny &&
-                        (unsigned)c2 < (unsigned)a.nz;
-        kv[u] = in ? __ldg(kappa + idx) : 0.f;
-        len[u] = in ? tn - t : 0.f;
-        if (live) {
-          t = tn;
-          c0 += ax == 0 ? s0 : 0;
-          c1 += ax == 1 ? s1 : 0;
-          c2 += ax == 2 ? s2 : 0;
-          idx += ax == 0 ? e0 : (ax == 1 ? e1 : e2);
-          if (ax == 0) tm0 = (c0 + o0 - a.xs[0]) * inv[0];
-          if (ax == 1) tm1 = (c1 + o1 - a.xs[1]) * inv[1];
-          if (ax == 2) tm2 = (c2 + o2 - a.xs[2]) * inv[2];
-          ++s;
-        }
-      }
+  for (int q = 0; q < 3; ++q) {
+    cc[q] = (((tile[q] << a.c[q]) + (warp & ((1 << a.c[q]) - 1))) << a.w[q]) + (lane & ((1 << a.w[q]) - 1));
+    lane >>= a.w[q];
+    warp >>= a.c[q];
+    inside = inside && cc[q] < n[q];
+  }
+  if (!inside) return;
+  const long long c = ((long long)cc[2] * a.ny + cc[1]) * a.nx + cc[0];
+  float v[3];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) tau = fmaf(kv[u], len[u], tau);
+  for (int q = 0; q < 3; ++q) v[q] = cc[q] + 0.5f - a.xs[q];
+  const float r = sqrtf(fmaf(v[0], v[0], fmaf(v[1], v[1], v[2] * v[2])));
+  if (!(r > 0.f)) {
+    Edot[c] = 0.f;
+    if (pdot) pdot[c] = pdot[ncell + c] = pdot[2 * ncell + c] = 0.f;
+    return;
+  }
+  float d[3], inv[3], in_q[3];
+  float t_in = 0.f, t_out = INFINITY;  // the target cell's parameter interval (slabs)
+#pragma unroll
+  for (int q = 0; q < 3; ++q) {
+    d[q] = v[q] / r;
+    inv[q] = d[q] != 0.f ? 1.f / d[q] : INFINITY;
+    in_q[q] = 0.f;
+    if (d[q] != 0.f) {
+      const float t1 = (cc[q] - a.xs[q]) * inv[q], t2 = (cc[q] + 1 - a.xs[q]) * inv[q];
+      in_q[q] = fminf(t1, t2);
+      t_in = fmaxf(t_in, in_q[q]);
+      t_out = fminf(t_out, fmaxf(t1, t2));
     }
-    const float taus = tau * a.h, drl = dr * a.h, rl = r * a.h;
-    const float tc = kappa[c] * drl;
-    const float E = a.L * expf(-taus) * (-expm1f(-tc)) / (4.f * 3.14159265358979f * rl * rl * drl);
-    Edot[c] = E;
-    if (pdot) {
-      pdot[c] = E * d[0];
-      pdot[ncell + c] = E * d[1];
-      pdot[2 * ncell + c] = E * d[2];
+  }
+  const float dr = t_out - t_in;
+  // The walk from the source cell to the entry of the target cell: the next
+  // crossing tm of each axis is kept, at plane pl, and only the axis just
+  // crossed has its next crossing recomputed from the source position.  A step
+  // runs from the last crossing to the next, and none starts at t_in - 1e-5 or
+  // later: of an axis' crossings between the two cells only the last, at in_q,
+  // can lie there.
+  const float t_end = t_in - 1e-5f;
+  Plane pl[3], s[3];
+  float tm[3];
+  Idx e[3] = {1, (Idx)a.nx, (Idx)a.nx * a.ny}, idx = 0;
+  int steps = 1;
+#pragma unroll
+  for (int q = 0; q < 3; ++q) {
+    const int cs = min((int)floorf(a.xs[q]), n[q] - 1);  // rounded to 32 bits, a source may lie on the upper boundary
+    const bool up = d[q] > 0.f;
+    steps += abs(cc[q] - cs) - (cc[q] != cs && !(in_q[q] < t_end) ? 1 : 0);
+    idx += cs * e[q];
+    e[q] = up ? e[q] : -e[q];
+    s[q] = (Plane)(up ? 1 : -1);
+    pl[q] = (Plane)(cs + (up ? 1 : 0));
+    tm[q] = d[q] != 0.f ? (pl[q] - a.xs[q]) * inv[q] : INFINITY;
+  }
+  if (!(t_end > 0.f)) steps = 0;
+  float t = 0.f, tau = 0.f;
+  auto step = [&](float &kv, float &len) {
+    if constexpr (!CHECK) {
+      // the clamp below never acts here: the last step ends at the first of the
+      // crossings from t_end on, and the target's own is one of them
+      const float t0 = t;
+      kv = __ldg(kappa + idx);
+      asm("{\n .reg .pred p, q, r;\n .reg .f32 u;\n"
+          " min.f32 u, %4, %5;\n min.f32 %0, u, %6;\n"
+          " setp.eq.f32 p, %4, %0;\n setp.eq.and.f32 q|r, %5, %0, !p;\n"
+          " @p add.f32 %1, %1, %8;\n @p sub.f32 u, %1, %11;\n @p mul.f32 %4, u, %14;\n @p add.s32 %7, %7, %17;\n"
+          " @q add.f32 %2, %2, %9;\n @q sub.f32 u, %2, %12;\n @q mul.f32 %5, u, %15;\n @q add.s32 %7, %7, %18;\n"
+          " @r add.f32 %3, %3, %10;\n @r sub.f32 u, %3, %13;\n @r mul.f32 %6, u, %16;\n @r add.s32 %7, %7, %19;\n}\n"
+          : "=&f"(t), "+f"(pl[0]), "+f"(pl[1]), "+f"(pl[2]), "+f"(tm[0]), "+f"(tm[1]), "+f"(tm[2]), "+r"(idx)
+          : "f"(s[0]), "f"(s[1]), "f"(s[2]), "f"(a.xs[0]), "f"(a.xs[1]), "f"(a.xs[2]), "f"(inv[0]), "f"(inv[1]),
+            "f"(inv[2]), "r"(e[0]), "r"(e[1]), "r"(e[2]));
+      len = t - t0;
+      return;
     }
+    const float tn = fminf(fminf(tm[0], tm[1]), tm[2]);
+    const bool p0 = tm[0] == tn, p1 = !p0 && tm[1] == tn, p2 = !p0 && !p1;
+    const float te = fminf(tn, t_in);
+    len = te - t;
+    t = te;
+    bool in = true;
+    if constexpr (CHECK) {
+#pragma unroll
+      for (int q = 0; q < 3; ++q) in = in && (unsigned)(pl[q] - (s[q] > 0)) < (unsigned)n[q];
+    }
+    kv = in ? __ldg(kappa + idx) : 0.f;
+    len = in ? len : 0.f;
+    if (p0) {
+      pl[0] += s[0];
+      tm[0] = (pl[0] - a.xs[0]) * inv[0];
+      idx += e[0];
+    }
+    if (p1) {
+      pl[1] += s[1];
+      tm[1] = (pl[1] - a.xs[1]) * inv[1];
+      idx += e[1];
+    }
+    if (p2) {
+      pl[2] += s[2];
+      tm[2] = (pl[2] - a.xs[2]) * inv[2];
+      idx += e[2];
+    }
+  };
+  for (; steps >= 4; steps -= 4) {
+    float kv[4], len[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) step(kv[u], len[u]);
+#pragma unroll
+    for (int u = 0; u < 4; ++u) tau = fmaf(kv[u], len[u], tau);
+  }
+  {
+    float kv[3] = {0.f, 0.f, 0.f}, len[3] = {0.f, 0.f, 0.f};
+#pragma unroll
+    for (int u = 0; u < 3; ++u)
+      if (u < steps) step(kv[u], len[u]);
+#pragma unroll
+    for (int u = 0; u < 3; ++u) tau = fmaf(kv[u], len[u], tau);
+  }
+  const float taus = tau * a.h, drl = dr * a.h, rl = r * a.h;
+  const float tc = kappa[c] * drl;
+  const float E = a.L * expf(-taus) * (-expm1f(-tc)) / (4.f * 3.14159265358979f * rl * rl * drl);
+  Edot[c] = E;
+  if (pdot) {
+    pdot[c] = E * d[0];
+    pdot[ncell + c] = E * d[1];
+    pdot[2 * ncell + c] = E * d[2];
   }
 }
 
@@ -152,11 +227,20 @@ extern "C" __attribute__((visibility("default"))) vet_status vet_point_source(co
     a.xs[q] = (float)u;
   }
   if (!on_device(kappa) || !on_device(Edot_out) || (pdot_out && !on_device(pdot_out))) return VET_EINVAL;
-  int dev = 0, sms = 1;
-  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) {
-    cudaGetLastError();
-    return VET_ECUDA;
+  // bricks no wider than the grid's planes: 8 x 2 x 2 cells a warp, 16 x 4 x 4 a CTA
+  for (int q = 1; q < 3; ++q) {
+    a.w[q] = n[q] > 1;
+    a.c[q] = n[q] > 2;
   }
-  point_kernel<<<8 * sms, 256, 0, (cudaStream_t)stream>>>(a, kappa, Edot_out, pdot_out);
+  a.w[0] = 5 - a.w[1] - a.w[2];
+  a.c[0] = 3 - a.c[1] - a.c[2];
+  long long tiles[3];
+  for (int q = 0; q < 3; ++q) tiles[q] = (n[q] + (1LL << (a.w[q] + a.c[q])) - 1) >> (a.w[q] + a.c[q]);
+  a.tx = (int)tiles[0];
+  a.ty = (int)tiles[1];
+  const long long ctas = tiles[0] * tiles[1] * tiles[2];
+  const bool plain = std::max({n[0], n[1], n[2]}) <= kPlainExtent && (long long)n[0] * n[1] * n[2] <= INT32_MAX;
+  auto kernel = plain ? point_kernel<false> : point_kernel<true>;
+  kernel<<<(unsigned)ctas, 256, 0, (cudaStream_t)stream>>>(a, kappa, Edot_out, pdot_out);
   return cudaGetLastError() == cudaSuccess ? VET_OK : VET_ECUDA;
 }
