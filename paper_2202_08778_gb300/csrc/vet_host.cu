@@ -176,22 +176,24 @@ vet_status build_schedule(vet_ctx *c, int group) {
   return VET_OK;
 }
 
-// The paired cell pass's split for the whole grid (the largest plan over the
-// direction tiles the tuning can pick): its scratch (part) and counters lie
-// behind the face intensities, in their allocation.  No scratch where the
-// pass is not paired or no plan splits (the trace's splits need none); off
-// for grids of a batch, whose closures share the GPU: a lone grid's last
-// wave leaves SMs idle, a batch's does not.
+// The split of the paired and of the FP64 cell pass for the whole grid (the
+// largest plan over the direction tiles the tuning can pick): its scratch
+// (part) and counters lie behind the face intensities, in their allocation.
+// No scratch where the pass never splits or no plan does (the trace's splits
+// need none); off for grids of a batch, whose closures share the GPU: a lone
+// grid's last wave leaves SMs idle, a batch's does not.
 vet::TailPlan split_plan(vet_ctx *c) {
   vet::TailPlan best;
   int nsm = 0;
-  if (!c->want_split || !c->dims.paired) return best;
+  if (!c->want_split || !(c->dims.paired || c->fp64)) return best;
   if (cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, c->cfg.device) != cudaSuccess) {
     cudaGetLastError();
     return best;
   }
-  for (int dt = 2; dt <= vet::kMaxTune; dt += 2) {
-    const vet::TailPlan p = vet::plan_tail_split(c->grid.block, c->nblk, nsm, c->N, dt);
+  const int B = c->grid.block;
+  for (int want = 1; want <= vet::kMaxTune; ++want) {
+    const vet::TailPlan p = c->fp64 ? vet::plan_cell_split64(B, c->nblk, nsm, c->N, vet::cell_tile_fit(B, want, true))
+                                    : vet::plan_tail_split(B, c->nblk, nsm, c->N, vet::pair_tile_fit(B, want));
     if (p.part_bytes > best.part_bytes) best = p;
   }
   c->split.nsm = nsm;

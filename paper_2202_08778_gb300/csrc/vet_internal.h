@@ -244,6 +244,9 @@ struct TailPlan {
   bool ordered = false;   // total < wave: per-pair values instead of partial moments
 };
 TailPlan plan_tail_split(int B, int nblk, int nsm, int ndir, int dir_tile);
+// The same for the FP64 cell pass, whose shares always store partial moments
+// ([slot][share][14][threads] doubles), also on grids of less than one wave.
+TailPlan plan_cell_split64(int B, int nblk, int nsm, int ndir, int dir_tile);
 // Largest scratch of an ordered split (beyond: the grid runs unsplit).
 constexpr size_t kOrderedSplitMax = (size_t)128 << 20;
 

@@ -568,7 +568,8 @@ __global__ void __launch_bounds__(kCellThreads, kCellMinCtas<R>)
                      const unsigned char *__restrict__ tpl_g, const int *__restrict__ order,
                      const R *__restrict__ faces, const R *__restrict__ bnd, R *__restrict__ I_out,
                      R *__restrict__ M_out, R *__restrict__ E_out, R *__restrict__ f_out, void *emax_bits,
-                     long long spin_limit, int *status, const int *__restrict__ block_list) {
+                     long long spin_limit, int *status, const int *__restrict__ block_list, int nfull, int ksplit,
+                     double *split_part, int *split_count) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ __align__(8) uint64_t full[2], empty[2];
   const int B = BC ? BC : g.B;
@@ -579,16 +580,26 @@ __global__ void __launch_bounds__(kCellThreads, kCellMinCtas<R>)
   const size_t sb = slot_bytes<R>(B);
   vec2_t<R> *tile = reinterpret_cast<vec2_t<R> *>(smem);
   unsigned char *buf0 = smem + align16(sizeof(vec2_t<R>) * (size_t)ts.elems);
-  const int item = blockIdx.x / parts, part = blockIdx.x - item * parts;
+  // past nfull, ksplit consecutive CTAs share one work item (slot), each a
+  // contiguous run of its direction tiles (FP64 only)
+  constexpr bool kSplit = sizeof(R) == 8;
+  int cta = (int)blockIdx.x, share = 0, slot = -1;
+  if (kSplit && ksplit > 1 && cta >= nfull) {
+    slot = (cta - nfull) / ksplit;
+    share = cta - nfull - slot * ksplit;
+    cta = nfull + slot;
+  }
+  const int item = cta / parts, part = cta - item * parts;
   const int blk = block_list ? block_list[item] : item;
   const int bx = blk % g.nbx, by = (blk / g.nbx) % g.nby, bz = blk / (g.nbx * g.nby);
   const int cpc = B3 / parts;  // cells of this CTA
   const int nwarps = blockDim.x >> 5;
-  const int ntiles = (g.ndir + dt - 1) / dt;
+  const int ntiles_all = (g.ndir + dt - 1) / dt, nshares = slot >= 0 ? ksplit : 1;
+  const int tile0 = share * ntiles_all / nshares, ntiles = (share + 1) * ntiles_all / nshares - tile0;
   int issued = 0, consumed = 0;   // thread 0's count of tiles issued / waited for
   auto issue_tile = [&](int t) {  // thread 0 only
     issued = t + 1;
-    const int b = t & 1, d0 = t * dt, nd = min(dt, g.ndir - d0);
+    const int b = t & 1, d0 = (tile0 + t) * dt, nd = min(dt, g.ndir - d0);
     unsigned char *buf = buf0 + (size_t)b * dt * sb;
     mbar_expect_tx(&full[b], (uint32_t)(sb * nd));
     for (int j = 0; j < nd; ++j)
@@ -626,7 +637,7 @@ __global__ void __launch_bounds__(kCellThreads, kCellMinCtas<R>)
   // this cell's record of the direction after the current one is on its way
   // while the current ray is marched
   const uint32_t *cell_rec = g.cell_rec + cell_rec_index(B, cx, cy, cz);
-  uint32_t next_rec = __ldg(cell_rec + (size_t)order_dir(order[0]) * B3);
+  uint32_t next_rec = __ldg(cell_rec + (size_t)order_dir(order[tile0 * dt]) * B3);
   const long long gc = ((long long)(bz * B + cz) * g.ny + (by * B + cy)) * g.nx + (bx * B + cx);
   // Moments over all directions: a plain partial sum over the directions of
   // one tile, folded into the totals once per tile.  The fold of E, Pxx, Pyy
@@ -645,7 +656,7 @@ __global__ void __launch_bounds__(kCellThreads, kCellMinCtas<R>)
     const uint32_t ph = (uint32_t)((t >> 1) & 1);
     if (!mbar_wait_warp(&full[b], ph, spin_limit, status, 2)) { ok = false; break; }
     consumed = t + 1;
-    const int nd = min(dt, g.ndir - t * dt);
+    const int d0 = (tile0 + t) * dt, nd = min(dt, g.ndir - d0);
     const unsigned char *buf = buf0 + (size_t)b * dt * sb;
     if (active) {
       R part[10];
@@ -654,7 +665,7 @@ __global__ void __launch_bounds__(kCellThreads, kCellMinCtas<R>)
         const Tpl<R> T(buf + sb * j, TL);
         const R *fin = reinterpret_cast<const R *>(buf + sb * j + TL.bytes);
         const CellRec rec{next_rec};
-        next_rec = __ldg(cell_rec + (size_t)order_dir(order[min(t * dt + j + 1, g.ndir - 1)]) * B3);
+        next_rec = __ldg(cell_rec + (size_t)order_dir(order[min(d0 + j + 1, g.ndir - 1)]) * B3);
         const int last = rec.last(), row = rec.row();
         const R Iin = face_value<R>(fin + rec.face(), B + 2, T.cw[row], T.cw[row + B]);
         const R I = march<R>(tile, tc, last, T.cev, g.exp64, Iin);
@@ -700,6 +711,42 @@ __global__ void __launch_bounds__(kCellThreads, kCellMinCtas<R>)
     // after a wait gave up, tiles may still be in flight into this CTA's
     // shared memory: wait (bounded) for every tile issued but not consumed
     for (int t = consumed; t < issued; ++t) mbar_wait(&full[t & 1], (uint32_t)((t >> 1) & 1), kDrainPolls, status, 8);
+  }
+  if constexpr (MODE != 1 && kSplit) {
+    if (slot >= 0) {
+      // one share of a split work item: its sums go to the slot's scratch, and
+      // the share that finishes last adds the others' (the compensated sums as
+      // compensated sums) and writes the outputs
+      __shared__ int s_last;
+      const int NT = blockDim.x;
+      R *mine = split_part + ((size_t)slot * ksplit + share) * 14 * NT + threadIdx.x;
+      for (int m = 0; m < 10; ++m) mine[m * NT] = mom[m];
+      for (int q = 0; q < 4; ++q) mine[(10 + q) * NT] = cmp[q];
+      __threadfence();
+      __syncthreads();
+      if (threadIdx.x == 0) s_last = atomicAdd(split_count + slot, 1) == ksplit - 1;
+      __syncthreads();
+      if (!s_last) return;
+      __threadfence();
+      for (int r = 0; r < ksplit; ++r) {
+        if (r == share) continue;
+        const R *other = split_part + ((size_t)slot * ksplit + r) * 14 * NT + threadIdx.x;
+#pragma unroll
+        for (int m = 0; m < 10; ++m) {
+          const R v = __ldcg(other + m * NT);
+          if (m == 0 || (m >= 4 && m < 7)) {
+            const int q = m == 0 ? 0 : m - 3;
+            const R y = v - (cmp[q] + __ldcg(other + (10 + q) * NT));
+            const R tt = mom[m] + y;
+            cmp[q] = (tt - mom[m]) - y;
+            mom[m] = tt;
+          } else if (kWantF || m >= 7) {
+            mom[m] += v;
+          }
+        }
+      }
+      if (threadIdx.x == 0) split_count[slot] = 0;  // ready for the next call
+    }
   }
   if (MODE != 1) {
     R emax = R(0);
@@ -1840,6 +1887,8 @@ int cell_parts(int B) {
   return parts;
 }
 
+int cell_threads(int B) { return (B * B * B / cell_parts(B) + 31) / 32 * 32; }
+
 template <typename R, int BC>
 void face_launch(const GridDims &g, const R *kappa, const R *S, const unsigned char *tpl, const FaceItem *items,
                  int nitems, int max_dirs, R *faces, const R *bnd, long long spin, int *status, cudaStream_t st) {
@@ -1875,15 +1924,23 @@ void face_launch(const GridDims &g, const R *kappa, const R *S, const unsigned c
 template <typename R, int MODE, int BC>
 void cell_launch(const GridDims &g, const R *kappa, const R *S, const unsigned char *tpl, const int *order,
                  const R *faces, const R *bnd, R *I_out, R *M_out, R *E_out, R *f_out, void *emax_bits,
-                 long long spin, int *status, const int *block_list, int nlist, cudaStream_t st) {
-  const int parts = cell_parts(g.B);
-  const int cpc = g.B * g.B * g.B / parts;
-  const int threads = (cpc + 31) / 32 * 32;
+                 long long spin, int *status, const int *block_list, int nlist, cudaStream_t st,
+                 const TailSplit *split) {
+  const int parts = cell_parts(g.B), threads = cell_threads(g.B);
   const int nblk = block_list ? nlist : g.nbx * g.nby * g.nbz;
   const int dt = cell_dir_tile<R>(g.B, g.dir_tile);
-  cell_pass_kernel<R, MODE, BC><<<nblk * parts, threads, smem_bytes<R>(g.B, 2 * dt), st>>>(
+  TailPlan tp;
+  tp.nfull = nblk * parts;
+  if (sizeof(R) == 8 && split && !block_list) {
+    const TailPlan q = plan_cell_split64(g.B, nblk, split->nsm, g.ndir, dt);
+    const bool room = MODE == 1 || (split->part && split->count && q.part_bytes <= split->part_bytes &&
+                                    q.slots <= split->slots);
+    if (q.k > 1 && room) tp = q;
+  }
+  const int grid = tp.nfull + (nblk * parts - tp.nfull) * tp.k;
+  cell_pass_kernel<R, MODE, BC><<<grid, threads, smem_bytes<R>(g.B, 2 * dt), st>>>(
       g, parts, dt, kappa, S, tpl, order, faces, bnd, I_out, M_out, E_out, f_out, emax_bits, spin, status,
-      block_list);
+      block_list, tp.nfull, tp.k, split ? (double *)split->part : nullptr, split ? split->count : nullptr);
 }
 
 // Staging of the paired cell pass: directions per tile (whole antipodal
@@ -1908,6 +1965,33 @@ inline void pair_staging(int B, int want, int &dt, int &nstage) {
 }
 
 }  // namespace
+
+TailPlan plan_cell_split64(int B, int nblk, int nsm, int ndir, int dt) {
+  TailPlan p;
+  const int parts = cell_parts(B), threads = cell_threads(B), total = nblk * parts, ntiles = (ndir + dt - 1) / dt;
+  p.nfull = total;
+  if (nsm <= 0) return p;
+  // CTAs an SM holds: up to 128 registers a thread, shared memory
+  const int wave = nsm * (int)std::max<size_t>(1, std::min<size_t>(512 / threads, kSmemMax / (smem_bytes<double>(B, 2 * dt) + 1024)));
+  const int r = total % wave;
+  // tail time in CTA times, each share's own start counted as 0.5% of a CTA
+  // (512 cells, 192 directions: about 2 ms); split for a gain above 2% of a CTA.
+  // 64^3 cells in 16^3 blocks, 512 CTAs on 152 places, the last 56 in 8 shares:
+  // closure 11.44 -> 10.20 ms
+  double best = 1.0;
+  for (int k = 2; r && k <= std::min(ntiles, 32); ++k) {
+    const size_t bytes = (size_t)r * k * 14 * threads * sizeof(double);
+    const double cost = (double)(((long long)k * r + wave - 1) / wave) / k + 0.005 * k;
+    if (bytes <= kOrderedSplitMax && cost < best - 0.02) {
+      best = cost;
+      p.k = k;
+      p.nfull = total - r;
+      p.slots = r;
+      p.part_bytes = bytes;
+    }
+  }
+  return p;
+}
 
 TailPlan plan_tail_split(int B, int nblk, int nsm, int ndir, int dir_tile) {
   TailPlan p;
@@ -2107,7 +2191,7 @@ cudaError_t launch_cell_pass(const GridDims &g, int mode, const R *kappa, const 
   }
 #define VET_CELL(MODE, BC)                                                                                  \
   cell_launch<R, MODE, BC>(g, kappa, S, tpl, order, faces, bnd, I_out, M_out, E_out, f_out, emax_bits, spin, \
-                           status, block_list, nlist, st)
+                           status, block_list, nlist, st, split)
   if (mode == 0 && M_out) {
     if (g.B == 16) VET_CELL(0, 16);
     else if (g.B == 8) VET_CELL(0, 8);

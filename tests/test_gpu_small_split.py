@@ -1,10 +1,12 @@
 """Small grids, whose cell pass is split into direction shares to fill the SMs:
-bit for bit what the unsplit pass computes (the same grid in a batch, which
-never splits), with and without the moments, repeatedly and after retuning."""
+bit for bit what the unsplit pass computes in FP32 (the same grid in a batch,
+which never splits), to rounding in FP64; with and without the moments,
+repeatedly and after retuning."""
 import numpy as np
 import pytest
 import torch
 
+from gpu_common import f_error, moment_errors, rel_err
 from paper_2202_08778_gb300 import synth, vet
 
 pytestmark = pytest.mark.gpu
@@ -35,3 +37,32 @@ def test_bits_of_the_unsplit_pass(shape, B, nside):
             for o in out[:2]:
                 assert torch.equal(o[0], out[2][0])
                 assert not with_M or torch.equal(o[1], out[2][1])
+
+
+@pytest.mark.parametrize("shape,B,nside", [((8, 8, 8), 8, 1),      # one CTA, three shares of one direction tile
+                                           ((16, 16, 16), 16, 2),  # 8 CTAs
+                                           ((48, 48, 48), 16, 2),  # 216 CTAs: one wave and a split last one
+                                           ((24, 32, 48), 4, 1),   # 576 CTAs of 64 threads
+                                           ((10, 15, 20), 5, 2), ((21, 14, 28), 7, 2)])
+def test_fp64_shares_match_oracle(ora, shape, B, nside):
+    """FP64 sums differ from the oracle in their order only: 1e-11 on the
+    moments, 1e-12 on f."""
+    p = synth.lognormal_problem(shape=shape, B=B, nside=nside, seed=8)
+    n = int(np.prod(shape))
+    ctx = vet.Context(shape, B, p["h"], nside, p["q"], precision=vet.VET_FP64)
+    Ib = np.random.default_rng(8).uniform(0, 0.5, (6, ctx.N))
+    k, S, ib = (torch.from_numpy(np.ascontiguousarray(x)).cuda() for x in (p["kappa"], p["S"], Ib))
+    f_ref, M_ref, I_ref, _ = ora.vet_closure(p["kappa"], p["S"], ctx.directions(), B, p["h"], Ib)
+    for tile in (0, 1, 8):
+        if tile:
+            ctx.set_tuning(dir_tile=tile)
+        f, M, f_alone, I = (torch.full((r, n), float("nan"), dtype=torch.float64, device="cuda") for r in (6, 10, 6, ctx.N))
+        for _ in range(2):
+            ctx.closure(k, S, ib, f, M)
+        ctx.closure(k, S, ib, f_alone)
+        ctx.trace(k, S, ib, I)
+        ctx.sync()
+        assert rel_err(I.cpu(), I_ref.reshape(ctx.N, -1)) < 1e-11
+        eE, eFP = moment_errors(M.cpu(), M_ref)
+        assert eE < 1e-11 and eFP < 1e-11
+        assert f_error(f.cpu(), f_ref, M_ref) < 1e-12 and f_error(f_alone.cpu(), f_ref, M_ref) < 1e-12
