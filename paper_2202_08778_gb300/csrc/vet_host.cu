@@ -494,7 +494,7 @@ vet_status mark(vet_ctx *c, int i, cudaStream_t st) {
 
 template <typename R>
 vet_status run_face_pass(vet_ctx *c, const R *kappa, const R *S, const R *Ib, cudaStream_t st) {
-  cudaError_t e = vet::launch_fill_boundary<R>(c->dims, (const unsigned char *)c->d_tpl, Ib, (R *)c->d_bnd, st);
+  cudaError_t e = vet::launch_fill_boundary<R>(c->dims, (const unsigned char *)c->d_tpl, Ib, (R *)c->d_bnd, c->d_emax, st);
   if (e) return cuda_err(c, e, "boundary fill launch");
   for (int L = 0; L < c->nlevels; ++L) {
     const int n = c->level_off[L + 1] - c->level_off[L];
@@ -580,18 +580,16 @@ vet_status do_closure(vet_ctx *c, const R *kappa, const R *S, const R *Ib, R *f_
   if (s) return s;
   c->timed = false;
   if ((s = mark(c, 0, st))) return s;
-  cudaError_t e = cudaMemsetAsync(c->d_emax, 0, 8, st);
-  if (e) return cuda_err(c, e, "cudaMemsetAsync");
   if ((s = run_face_pass<R>(c, din[0], din[1], din[2], st))) return s;
   if ((s = mark(c, 1, st))) return s;
   R *Mdev = dout[1];
-  e = vet::launch_cell_pass<R>(c->dims, 0, din[0], din[1], (const unsigned char *)c->d_tpl, c->d_cell_order,
+  cudaError_t e = vet::launch_cell_pass<R>(c->dims, 0, din[0], din[1], (const unsigned char *)c->d_tpl, c->d_cell_order,
                                (const R *)c->d_faces, (const R *)c->d_bnd, nullptr, Mdev, (R *)c->d_E, dout[0],
                                c->d_emax, c->spin, c->d_status, st, nullptr, 0, c->split.nsm ? &c->split : nullptr);
   if (e) return cuda_err(c, e, "cell pass launch");
   if ((s = mark(c, 2, st))) return s;
   const R *E = Mdev ? Mdev : (const R *)c->d_E;
-  e = vet::launch_floor_fix<R>(c->dims.ncell, E, 1, c->d_emax, 1e-30, dout[0], st);
+  e = vet::launch_floor_fix<R>(c->dims.ncell, E, c->d_emax, 1e-30, dout[0], st, true);
   if (e) return cuda_err(c, e, "floor launch");
   if ((s = mark(c, 3, st))) return s;
   c->last_stream = st;
@@ -618,11 +616,9 @@ vet_status vet::exact_on_blocks(vet_ctx *c, const float *kappa, const float *S, 
                                 int nlist, float *f_out, cudaStream_t st) {
   if (!c || c->fp64) return set_err(c, VET_EINVAL, "the learned closure needs an FP32 context");
   if (nlist <= 0) return VET_OK;
-  cudaError_t e = cudaMemsetAsync(c->d_emax, 0, 8, st);
-  if (e) return cuda_err(c, e, "cudaMemsetAsync");
   vet_status s = run_face_pass<float>(c, kappa, S, Ib, st);
   if (s) return s;
-  e = vet::launch_cell_pass<float>(c->dims, 0, kappa, S, (const unsigned char *)c->d_tpl, c->d_cell_order,
+  cudaError_t e = vet::launch_cell_pass<float>(c->dims, 0, kappa, S, (const unsigned char *)c->d_tpl, c->d_cell_order,
                                    (const float *)c->d_faces, (const float *)c->d_bnd, nullptr, nullptr,
                                    (float *)c->d_E, f_out, c->d_emax, c->spin, c->d_status, st, d_list, nlist);
   if (e) return cuda_err(c, e, "cell pass launch");
@@ -1027,7 +1023,6 @@ vet_status capture_merged(vet_batch *b, const float *const *kappa, const float *
   for (int i = 0; i < b->n && !e; ++i) {
     vet_ctx *c = b->ctx[i];
     if ((e = cudaStreamWaitEvent(b->branch[i], b->forked, 0))) break;
-    if ((e = cudaMemsetAsync(c->d_emax, 0, 8, b->branch[i]))) break;
     vet_status st = run_face_pass<float>(c, kappa[i], S[i], Ib ? Ib[i] : nullptr, b->branch[i]);
     if (st != VET_OK) {
       b->err = "grid " + std::to_string(i) + ": " + c->err;
@@ -1053,7 +1048,7 @@ vet_status capture_merged(vet_batch *b, const float *const *kappa, const float *
     const MergedGroup &m = groups[group_of[i]];
     if (i != m.lead && (e = cudaStreamWaitEvent(b->branch[i], b->group_done[group_of[i]], 0))) break;
     const float *E = with_M ? M_out[i] : (const float *)c->d_E;
-    if ((e = vet::launch_floor_fix<float>(c->dims.ncell, E, 1, c->d_emax, 1e-30, f_out[i], b->branch[i]))) break;
+    if ((e = vet::launch_floor_fix<float>(c->dims.ncell, E, c->d_emax, 1e-30, f_out[i], b->branch[i]))) break;
     if ((e = cudaEventRecord(b->joined[i], b->branch[i]))) break;
     e = cudaStreamWaitEvent(b->origin, b->joined[i], 0);
   }

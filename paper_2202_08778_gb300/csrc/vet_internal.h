@@ -306,11 +306,12 @@ cudaError_t launch_ray_records(const GridDims &g, const unsigned char *tpl, cons
 
 // bnd[face][d] <- constant Ib[face][ext(d)] (or 0 when Ib is NULL).
 template <typename R>
-cudaError_t launch_fill_boundary(const GridDims &g, const unsigned char *tpl, const R *Ib, R *bnd, cudaStream_t st);
+cudaError_t launch_fill_boundary(const GridDims &g, const unsigned char *tpl, const R *Ib, R *bnd, void *emax_bits,
+                                 cudaStream_t st);
 
 template <typename R>
-cudaError_t launch_floor_fix(long long ncell, const R *E, long long E_stride, const void *emax_bits,
-                             double floor_rel, R *f_out, cudaStream_t st);
+cudaError_t launch_floor_fix(long long ncell, const R *E, const void *emax_bits, double floor_rel, R *f_out,
+                             cudaStream_t st, bool after_cell_pass = false);
 
 // E64 (optional, device): E of every cell summed in FP64, w64 times the sum
 // of I over the directions (the weights are all equal to w64).

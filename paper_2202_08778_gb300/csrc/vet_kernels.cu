@@ -617,6 +617,7 @@ __global__ void __launch_bounds__(kCellThreads, kCellMinCtas<R>)
   }
   load_tile<R, BC>(tile, ts, g, bx, by, bz, kappa, S);
   __syncthreads();
+  if (MODE != 1) griddep_launch_dependents();  // the floor rule's launch overlaps the pass
 
   const bool active = (int)threadIdx.x < cpc;
   int cx, cy, cz;
@@ -1291,6 +1292,7 @@ __global__ void __launch_bounds__(pair_max_threads(BC), pair_bound_ctas(BC))
   load_tile_pair<BC, BC ? pair_threads(BC) : 0>(tile, ts, g, bx, by, bz, kappa, S);
   if (threadIdx.x == 0) tile[ts.elems - 1] = make_float4(0.f, 0.f, 0.f, 0.f);  // identity entry
   __syncthreads();
+  if (MODE != 1) griddep_launch_dependents();  // the floor rule's launch overlaps the pass
 
   const PairCell<BC> pc(B, part, parts, threadIdx.x);
   const uint32_t tile_s = smem_u32(tile);
@@ -1770,11 +1772,14 @@ __global__ void __launch_bounds__(kFaceThreads, 2)
 }
 
 // Boundary faces of every direction, materialised so that staging is a
-// plain bulk copy: bnd[face][d][i] = Ib[face][ext(d)] (0 for vacuum).
+// plain bulk copy: bnd[face][d][i] = Ib[face][ext(d)] (0 for vacuum).  Clears the
+// word that the cell pass gathers max E in, too (a memset took a launch more).
 template <typename R>
 __global__ void fill_boundary_kernel(const GridDims g, const unsigned char *__restrict__ tpl_g, int tpl_bytes,
-                                     const R *__restrict__ Ib, R *__restrict__ bnd) {
+                                     const R *__restrict__ Ib, R *__restrict__ bnd, void *emax_bits) {
+  griddep_launch_dependents();  // the first level may load its tiles
   const int face = blockIdx.y, d = blockIdx.x;
+  if (emax_bits && face == 0 && d == 0 && threadIdx.x == 0) *static_cast<unsigned long long *>(emax_bits) = 0;
   const int ext = reinterpret_cast<const TplHead<R> *>(tpl_g + (size_t)d * tpl_bytes)->ext;
   const R v = Ib ? Ib[(long long)face * g.ndir + ext] : R(0);
   R *dst = bnd + ((long long)face * g.ndir + d) * g.fstride;
@@ -1793,6 +1798,7 @@ template <> __device__ __forceinline__ double load_max<double>(const void *p) {
 template <typename R>
 __global__ void floor_fix_kernel(long long ncell, const R *__restrict__ E, const void *__restrict__ emax_bits,
                                  double floor_rel, R *__restrict__ f) {
+  griddep_wait();
   const R floor = R(floor_rel) * load_max<R>(emax_bits);
   for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < ncell;
        c += (long long)gridDim.x * blockDim.x) {
@@ -2254,19 +2260,29 @@ cudaError_t launch_ray_records(const GridDims &g, const unsigned char *tpl, cons
 }
 
 template <typename R>
-cudaError_t launch_fill_boundary(const GridDims &g, const unsigned char *tpl, const R *Ib, R *bnd, cudaStream_t st) {
-  fill_boundary_kernel<R><<<dim3(g.ndir, 6), 128, 0, st>>>(g, tpl, tpl_layout<R>(g.B).bytes, Ib, bnd);
+cudaError_t launch_fill_boundary(const GridDims &g, const unsigned char *tpl, const R *Ib, R *bnd, void *emax_bits,
+                                 cudaStream_t st) {
+  fill_boundary_kernel<R><<<dim3(g.ndir, 6), 128, 0, st>>>(g, tpl, tpl_layout<R>(g.B).bytes, Ib, bnd, emax_bits);
   return cudaGetLastError();
 }
 
 template <typename R>
-cudaError_t launch_floor_fix(long long ncell, const R *E, long long, const void *emax_bits, double floor_rel,
-                             R *f_out, cudaStream_t st) {
+cudaError_t launch_floor_fix(long long ncell, const R *E, const void *emax_bits, double floor_rel, R *f_out,
+                             cudaStream_t st, bool after_cell_pass) {
   const int threads = 256;
   long long blocks = (ncell + threads - 1) / threads;
   if (blocks > 152 * 16) blocks = 152 * 16;
   if (blocks < 1) blocks = 1;
-  floor_fix_kernel<R><<<(int)blocks, threads, 0, st>>>(ncell, E, emax_bits, floor_rel, f_out);
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.gridDim = dim3((unsigned)blocks);
+  cfg.blockDim = dim3(threads);
+  cfg.stream = st;
+  cfg.attrs = attr;
+  cfg.numAttrs = after_cell_pass ? 1 : 0;
+  cudaLaunchKernelEx(&cfg, floor_fix_kernel<R>, ncell, E, emax_bits, floor_rel, f_out);
   return cudaGetLastError();
 }
 
@@ -2349,10 +2365,9 @@ cudaError_t prepare_kernels() {
                                                   double, R *, cudaStream_t);                                \
   template cudaError_t launch_ray_records<R>(const GridDims &, const unsigned char *, const uint16_t *, uint32_t *, \
                                              uint2 *, cudaStream_t);                                        \
-  template cudaError_t launch_fill_boundary<R>(const GridDims &, const unsigned char *, const R *, R *,      \
+  template cudaError_t launch_fill_boundary<R>(const GridDims &, const unsigned char *, const R *, R *, void *, \
                                                cudaStream_t);                                                \
-  template cudaError_t launch_floor_fix<R>(long long, const R *, long long, const void *, double, R *,     \
-                                           cudaStream_t);                                                    \
+  template cudaError_t launch_floor_fix<R>(long long, const R *, const void *, double, R *, cudaStream_t, bool); \
   template cudaError_t launch_moments<R>(long long, int, const R *, const R *, R *, cudaStream_t, double *, double);
 
 VET_INSTANTIATE(float)

@@ -195,13 +195,12 @@ VET_API vet_status vet_closure_noalloc(const vet_grid *grid, const vet_config *c
     void *d_emax = base + o_emax;
     auto *d_status = reinterpret_cast<int *>(base + o_status);
     // inputs of this call; the array keeps the previous call's contents, so
-    // the face padding, max-E and status words are cleared explicitly
+    // the face padding and the status word are cleared explicitly
     if ((e = cudaMemcpyAsync(d_tpl, h_tpl, (size_t)N * tbytes, cudaMemcpyHostToDevice, st))) break;
     if ((e = cudaMemcpyAsync(d_items, h_items, sizeof(vet::FaceItem) * (size_t)nitems, cudaMemcpyHostToDevice, st)))
       break;
     if ((e = cudaMemcpyAsync(d_order, h_cell_order, sizeof(int) * N, cudaMemcpyHostToDevice, st))) break;
     if ((e = cudaMemsetAsync(d_faces, 0, faces_bytes, st))) break;
-    if ((e = cudaMemsetAsync(d_emax, 0, 8, st))) break;
     if ((e = cudaMemsetAsync(d_status, 0, sizeof(int), st))) break;
     const long long spin = cfg->spin_limit > 0 ? cfg->spin_limit : (1LL << 22);
     auto *node_rec = static_cast<uint2 *>(g_rec_addr[cfg->device][0]);
@@ -209,7 +208,7 @@ VET_API vet_status vet_closure_noalloc(const vet_grid *grid, const vet_config *c
     if ((e = vet::launch_ray_records<float>(dims, d_tpl, nullptr, cell_rec, node_rec, st))) break;
     dims.node_rec = node_rec;
     dims.cell_rec = cell_rec;
-    if ((e = vet::launch_fill_boundary<float>(dims, d_tpl, Ib, d_bnd, st))) break;
+    if ((e = vet::launch_fill_boundary<float>(dims, d_tpl, Ib, d_bnd, d_emax, st))) break;
     for (int L = 0; L < nlevels && !e; ++L)
       e = vet::launch_face_level<float>(dims, kappa, S, d_tpl, d_items + h_level_off[L],
                                         h_level_off[L + 1] - h_level_off[L], vet::kFaceGroup, d_faces, d_bnd, spin,
@@ -218,7 +217,7 @@ VET_API vet_status vet_closure_noalloc(const vet_grid *grid, const vet_config *c
     if ((e = vet::launch_cell_pass<float>(dims, 0, kappa, S, d_tpl, d_order, d_faces, d_bnd, nullptr, M_out, d_E,
                                           f_out, d_emax, spin, d_status, st)))
       break;
-    if ((e = vet::launch_floor_fix<float>(dims.ncell, M_out ? M_out : d_E, 1, d_emax, 1e-30, f_out, st))) break;
+    if ((e = vet::launch_floor_fix<float>(dims.ncell, M_out ? M_out : d_E, d_emax, 1e-30, f_out, st, true))) break;
     poison_on_failure<<<152, 256, 0, st>>>(d_status, 6 * dims.ncell, f_out);
     e = cudaGetLastError();
   } while (false);
