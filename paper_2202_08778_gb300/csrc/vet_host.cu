@@ -288,7 +288,7 @@ vet_status build_context(vet_ctx *c) {
   if ((e = cudaMemset(c->d_status, 0, sizeof(int)))) return cuda_err(c, e, "cudaMemset(status)");
   if ((e = cudaMemcpy(c->d_tpl, tpl.data(), tpl.size(), cudaMemcpyHostToDevice)))
     return cuda_err(c, e, "upload templates");
-  vet_status st = build_schedule(c, c->face_group);
+  vet_status st = build_schedule(c, c->dims.face_paired ? vet::face_pair_group(B) : vet::kFaceGroup);
   if (st != VET_OK) return st;
   // the cell passes stage by this order: each entry also carries the
   // direction's signs (bits 16-18, flag bit 19)

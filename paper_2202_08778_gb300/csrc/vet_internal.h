@@ -336,6 +336,13 @@ size_t cell_smem_bytes(int B, int nslots, bool fp64);
 // Directions per face-pass item (default; a context may be tuned to 1..8).
 constexpr int kFaceGroup = 4;
 constexpr int kMaxTune = 8;
+// Default of the paired face pass.  An item's rays share its tile and its wait,
+// so small blocks take more directions; from 13 on, eight directions' faces leave
+// room for one CTA an SM instead of two.  Face pass, 192 directions, 4 and 8 a
+// item: edge 4, 64^3 cells, 1.41 and 1.04 ms; 6, 60^3, 0.45 and 0.39; 8, 128^3,
+// 1.86 and 1.56; 12, 108x84x60, 0.343 and 0.330; 14, 98^3, 0.580 and 0.596 (7);
+// 16, 128^3, 0.757 and 0.834.
+constexpr int face_pair_group(int B) { return B <= 12 ? 8 : kFaceGroup; }
 // Largest block edge of the mirrored (paired) FP32 passes: their 16-byte tiles
 // and staged directions fit a CTA's shared memory.
 constexpr int kMaxPairBlock = 16;

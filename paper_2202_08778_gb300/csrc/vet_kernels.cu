@@ -1665,8 +1665,9 @@ __global__ void __launch_bounds__(kFaceThreads, 2)
   // warp 0 stages: the templates (one lane per direction) before the previous
   // level ends, then the incoming faces, its output, one lane per ray and axis
   const int ncopy = 6 * cnt;
-  const float *src[2] = {nullptr, nullptr};
-  unsigned char *dst[2] = {nullptr, nullptr};
+  constexpr int kCopies = (6 * kMaxTune + 31) / 32;  // a lane's
+  const float *src[kCopies] = {};
+  unsigned char *dst[kCopies] = {};
   const uint32_t fb = (uint32_t)(g.fstride * sizeof(float));
   if (threadIdx.x < 32) {
     const int lane = threadIdx.x;
@@ -1679,7 +1680,7 @@ __global__ void __launch_bounds__(kFaceThreads, 2)
     if (lane < cnt)
       bulk_g2s(slots + sb * lane, tpl_g + (size_t)(it.dir_begin + lane) * TL.bytes, (uint32_t)TL.node_bytes, &full);
 #pragma unroll
-    for (int u = 0; u < 2; ++u) {
+    for (int u = 0; u < kCopies; ++u) {
       const int q = lane + 32 * u, r = q / 3, a = q - 3 * r;  // a primary ray (r < cnt) or its mirror
       const bool mir = r >= cnt;
       const int jj = mir ? r - cnt : r, d = (mir ? it.mirror_begin : it.dir_begin) + jj;
@@ -1703,7 +1704,7 @@ __global__ void __launch_bounds__(kFaceThreads, 2)
   if (threadIdx.x < 32) {
     griddep_wait();
 #pragma unroll
-    for (int u = 0; u < 2; ++u)
+    for (int u = 0; u < kCopies; ++u)
       if ((int)threadIdx.x + 32 * u < ncopy) bulk_g2s(dst[u], src[u], fb, &full);
   }
   if (threadIdx.x == 0) tile[B] = make_float4(0.f, 0.f, 0.f, 0.f);  // identity entry (padding, x = B)
