@@ -138,7 +138,6 @@ __device__ __forceinline__ float minus_mean(float l, Pair mean) {
   return isfinite(d.hi) ? __fadd_rn(d.hi, __fsub_rn(d.lo, mean.lo)) : d.hi;
 }
 
-// Grid: x over the cells of a volume, y over the volumes.
 // n / d for any n and d below 2^32: the multiplication's quotient is exact or one short.
 struct Div {
   unsigned d, m;
@@ -149,9 +148,10 @@ struct Div {
   }
 };
 
-// The input rows (bf16), cell by cell.  Its 64-bit divisions for the block of a
-// cell cost more than the logarithms: the learned closure of 128^3 cells 475 us
-// with them, 463 with 32-bit quotients.
+// The input rows (bf16), cell by cell (grid: x over the cells of a volume, y
+// over the volumes).  64-bit divisions for a cell's block cost more than the
+// logarithms: the learned closure of 128^3 cells 475 us with them, 463 with
+// 32-bit quotients.
 template <bool NARROW>
 __global__ void __launch_bounds__(256) feat_pack_kernel(const float *__restrict__ kappa, const float *__restrict__ S,
                                                         const float *__restrict__ E, Vol V, Div dnx, Div dny, Div dB, int B, float h,
