@@ -226,7 +226,7 @@ cudaError_t launch_face_level(const GridDims &g, const R *kappa, const R *S, con
 // tiles (k CTAs each), so that the tail takes about ceil(k r / wave) / k of
 // a CTA's time.  The shares' partial moments meet in `part`
 // ([slot][share][28][threads] floats) and the last share of a slot to
-// finish (counted in `count`, which it resets) adds the others' and writes
+// finish (counted in `count`, which it resets) adds them in order and writes
 // the outputs.
 //
 // A grid of fewer CTAs than one wave (total < wave) is split whole, every CTA

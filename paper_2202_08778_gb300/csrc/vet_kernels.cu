@@ -716,8 +716,9 @@ __global__ void __launch_bounds__(kCellThreads, kCellMinCtas<R>)
   if constexpr (MODE != 1 && kSplit) {
     if (slot >= 0) {
       // one share of a split work item: its sums go to the slot's scratch, and
-      // the share that finishes last adds the others' (the compensated sums as
-      // compensated sums) and writes the outputs
+      // the share that finishes last adds all of them in order (the compensated
+      // sums as compensated sums; the same bits whichever finishes last) and
+      // writes the outputs
       __shared__ int s_last;
       const int NT = blockDim.x;
       R *mine = split_part + ((size_t)slot * ksplit + share) * 14 * NT + threadIdx.x;
@@ -729,8 +730,9 @@ __global__ void __launch_bounds__(kCellThreads, kCellMinCtas<R>)
       __syncthreads();
       if (!s_last) return;
       __threadfence();
+      for (int m = 0; m < 10; ++m) mom[m] = R(0);
+      for (int q = 0; q < 4; ++q) cmp[q] = R(0);
       for (int r = 0; r < ksplit; ++r) {
-        if (r == share) continue;
         const R *other = split_part + ((size_t)slot * ksplit + r) * 14 * NT + threadIdx.x;
 #pragma unroll
         for (int m = 0; m < 10; ++m) {
@@ -1449,9 +1451,9 @@ __global__ void __launch_bounds__(pair_max_threads(BC), pair_bound_ctas(BC))
     if (threadIdx.x == 0) split_count[slot] = 0;  // ready for the next call
   } else if (MODE != 1 && slot >= 0) {
     // one share of a split work item: its partial sums go to the slot's
-    // scratch, and the share that finishes last adds the others' (the
-    // compensated sums as compensated sums, but for P_ij's last compensation)
-    // and writes the outputs
+    // scratch, and the share that finishes last adds all of them in order (the
+    // compensated sums as compensated sums, but for P_ij's last compensation;
+    // the same bits whichever finishes last) and writes the outputs
     constexpr int kVals = 28;
     __shared__ int s_last;
     float *mine = split_part + ((size_t)slot * ksplit + share) * kVals * NT + threadIdx.x;
@@ -1472,8 +1474,11 @@ __global__ void __launch_bounds__(pair_max_threads(BC), pair_bound_ctas(BC))
     if (!s_last) return;
     __threadfence();
     const float2 one = make_float2(1.f, 1.f);
+#pragma unroll
+    for (int m = 0; m < 10; ++m) mom[m] = make_float2(0.f, 0.f);
+#pragma unroll
+    for (int m = 0; m < 4; ++m) nc[m] = make_float2(0.f, 0.f);
     for (int r = 0; r < ksplit; ++r) {
-      if (r == share) continue;
       const float *other = split_part + ((size_t)slot * ksplit + r) * kVals * NT + threadIdx.x;
       float2 pm[10], pn[4];
 #pragma unroll

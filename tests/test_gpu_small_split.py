@@ -66,3 +66,18 @@ def test_fp64_shares_match_oracle(ora, shape, B, nside):
         eE, eFP = moment_errors(M.cpu(), M_ref)
         assert eE < 1e-11 and eFP < 1e-11
         assert f_error(f.cpu(), f_ref, M_ref) < 1e-12 and f_error(f_alone.cpu(), f_ref, M_ref) < 1e-12
+
+
+@pytest.mark.parametrize("shape,B,nside,precision", [((64, 64, 128), 16, 4, vet.VET_FP32),  # 256 CTAs of 152 places
+                                                     ((60, 60, 70), 10, 2, vet.VET_FP32), ((48, 48, 48), 16, 2, vet.VET_FP64),
+                                                     ((16, 32, 16), 16, 4, vet.VET_FP64)])
+def test_repeated_calls_give_the_same_bits(shape, B, nside, precision):
+    p = synth.lognormal_problem(shape=shape, B=B, nside=nside, seed=9)
+    n, dtype = int(np.prod(shape)), torch.float32 if precision == vet.VET_FP32 else torch.float64
+    k, S = (torch.from_numpy(np.ascontiguousarray(p[x])).to("cuda", dtype) for x in ("kappa", "S"))
+    ctx = vet.Context(shape, B, p["h"], nside, p["q"], precision=precision)
+    out = [torch.empty(16, n, dtype=dtype, device="cuda") for _ in range(6)]
+    for o in out:
+        ctx.closure(k, S, None, o[:6], o[6:])
+    ctx.sync()
+    assert all(torch.equal(o, out[0]) for o in out[1:])
