@@ -159,6 +159,8 @@ __global__ void __launch_bounds__(256) feat_pack_kernel(const float *__restrict_
                                                         const float *__restrict__ bstat, __nv_bfloat16 *__restrict__ x0,
                                                         float *__restrict__ feat_out) {
   __shared__ Pair s_mean[2];
+  after_previous();
+  let_next_launch();
   const long long vol = (long long)V.nz * V.ny * V.nx;
   const int v = blockIdx.y;
   if (threadIdx.x < 2) {
@@ -279,6 +281,8 @@ __global__ void __launch_bounds__(256) head_loss_kernel(const float *__restrict_
 __global__ void __launch_bounds__(256) adamw_kernel(NetMeta M, float *__restrict__ p, const float *__restrict__ g,
                                                     float *__restrict__ m, float *__restrict__ v, float lr, float b1,
                                                     float b2, float eps, float wd, float bc1, float bc2, int update) {
+  after_previous();
+  let_next_launch();
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < M.total;
        i += (long long)gridDim.x * blockDim.x) {
     float pi = p[i];
@@ -357,6 +361,8 @@ __global__ void __launch_bounds__(256) indicator_kernel(const float *__restrict_
 
 __global__ void __launch_bounds__(1024) compact_kernel(const unsigned int *__restrict__ flags, int n,
                                                        int *__restrict__ list, int *__restrict__ count) {
+  after_previous();
+  let_next_launch();
   __shared__ int wsum[32];
   const int per = (n + blockDim.x - 1) / blockDim.x;
   const int b = threadIdx.x * per, e = min(n, b + per);
@@ -415,9 +421,8 @@ cudaError_t features(const float *kappa, const float *S, const float *E, const V
   // cell numbers of a volume in 32 bits: quotients by multiplication
   const bool narrow = (long long)V.nz * V.ny * V.nx < (1LL << 31);
   auto *pack = narrow ? feat_pack_kernel<true> : feat_pack_kernel<false>;
-  pack<<<dim3(per_vol, V.n), 256, 0, st>>>(kappa, S, E, V, Div(V.nx), Div(V.ny), Div(B), B, (float)h, sums, bstat, x0,
-                                           feat_out);
-  return cudaGetLastError();
+  return launch_after(pack, dim3(per_vol, V.n), 256, 0, st, kappa, S, E, V, Div(V.nx), Div(V.ny), Div(B), B, (float)h, sums,
+                      bstat, x0, feat_out);
 }
 
 cudaError_t head_loss(const float *o, const float *f_ref, const unsigned char *mask, const Vol &V, float lam,
@@ -434,8 +439,8 @@ cudaError_t head_loss(const float *o, const float *f_ref, const unsigned char *m
 
 cudaError_t adamw(const NetMeta &M, float *p, const float *g, float *m, float *v, float lr, float b1, float b2,
                   float eps, float wd, float bc1, float bc2, int update, cudaStream_t st) {
-  adamw_kernel<<<grid_for(M.total, 256), 256, 0, st>>>(M, p, g, m, v, lr, b1, b2, eps, wd, bc1, bc2, update);
-  return cudaGetLastError();
+  return launch_after(adamw_kernel, dim3(grid_for(M.total, 256)), 256, 0, st, M, p, g, m, v, lr, b1, b2, eps, wd, bc1, bc2,
+                      update);
 }
 
 cudaError_t indicator(const float *o, const Vol &V, int B, float thr, float *f_out, float *r_out, unsigned int *flags,
@@ -449,8 +454,7 @@ cudaError_t indicator(const float *o, const Vol &V, int B, float thr, float *f_o
 }
 
 cudaError_t compact_flags(const unsigned int *flags, int n, int *list, int *count, cudaStream_t st) {
-  compact_kernel<<<1, 1024, 0, st>>>(flags, n, list, count);
-  return cudaGetLastError();
+  return launch_after(compact_kernel, dim3(1), 1024, 0, st, flags, n, list, count);
 }
 
 cudaError_t unpack_outputs(const float *o, const Vol &V, float *o_out, cudaStream_t st) {

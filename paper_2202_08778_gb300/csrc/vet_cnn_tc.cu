@@ -422,6 +422,8 @@ __global__ void __launch_bounds__(kTcThreads, 1)
   __shared__ int n_committed, n_next[2];  // steps whose MMAs were committed; first even and odd step the loaders did not see complete
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  after_previous();
+  let_next_launch();
   for (int h = threadIdx.x; h < 27 * C_OUT * NCI; h += blockDim.x) {
     const int c = h % NCI, co = (h / NCI) % C_OUT, tap = h / (NCI * C_OUT);
     const int4 val = reinterpret_cast<const int4 *>(W + ((size_t)tap * C_OUT + co) * C_IN)[c];
@@ -769,6 +771,7 @@ __global__ void __launch_bounds__(kWgThreads, 1)
   __shared__ float sBias[C_OUT];
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  after_previous();
   if (threadIdx.x < C_OUT) sBias[threadIdx.x] = 0.f;
   if (threadIdx.x == 0) {
     for (int k = 0; k < kWgRing; ++k) {
@@ -1060,8 +1063,8 @@ cudaError_t conv3d_tc(const __nv_bfloat16 *x, const __nv_bfloat16 *W, const floa
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   // one CTA per SM (it takes all of tensor memory), equal shares of the slices
   const long long g = nt < sms ? nt : sms;
-  conv3d_tc_kernel<C_IN, C_OUT, EPI><<<(int)g, kTcThreads, sm, st>>>(x, W, b, V, pre_out, pre_in, out, status);
-  return cudaGetLastError();
+  return launch_after(conv3d_tc_kernel<C_IN, C_OUT, EPI>, dim3((unsigned)g), kTcThreads, sm, st, x, W, b, V, pre_out, pre_in,
+                      out, status);
 }
 
 template <int C_IN, int C_OUT>
@@ -1078,8 +1081,7 @@ cudaError_t wgrad(const __nv_bfloat16 *x, const __nv_bfloat16 *gpre, const Vol &
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const long long g = nt < sms ? nt : sms;
-  wgrad_tc_kernel<C_IN, C_OUT><<<(int)g, kWgThreads, sm, st>>>(x, gpre, V, gW, gb, status);
-  return cudaGetLastError();
+  return launch_after(wgrad_tc_kernel<C_IN, C_OUT>, dim3((unsigned)g), kWgThreads, sm, st, x, gpre, V, gW, gb, status);
 }
 
 #define VET_TC_INST(CI, CO, EPI)                                                                                  \
