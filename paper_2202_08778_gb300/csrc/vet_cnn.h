@@ -55,7 +55,7 @@ __device__ __forceinline__ void let_next_launch() { asm volatile("griddepcontrol
 
 
 // out = epi(conv3d(x, W) + b) on the tcgen05 tensor cores (vet_cnn_tc.cu):
-// tiles of 8 x 16 x 2 cells, accumulators in tensor memory.  Epilogues:
+// columns of 8 x 16 cells marched along z, accumulators in tensor memory.  Epilogues:
 //   EPI_SILU:     pre = acc + b (stored BF16 if pre_out), out = SiLU(pre) BF16
 //   EPI_F32:      out = acc + b, FP32, the first kOutRow channels
 //   EPI_SILU_BWD: out = acc * SiLU'(pre_in) BF16 (data gradient through the

@@ -348,7 +348,7 @@ constexpr int face_pair_group(int B) { return B <= 12 ? 8 : kFaceGroup; }
 constexpr int kMaxPairBlock = 16;
 // Smallest block edge of the paired cell pass: below, a CTA's few cells do not
 // pay for its pairs of staged directions (cell pass, paired against unpaired: edge 4
-// 0.42 and 0.38 ms, 5 0.36 and 0.34, 6 0.42 and 0.56, 12 1.5 and 2.7; the paired
+// 0.42 and 0.38 ms, 5 0.36 and 0.34, 6 0.43 and 0.56, 12 1.6 and 2.7; the paired
 // face pass is ahead from 2 on, 0.59 and 0.67 ms).
 constexpr int kMinPairBlock = 6;
 
