@@ -1008,7 +1008,10 @@ __global__ void __launch_bounds__(kWgThreads, 1)
         const int4 *src = reinterpret_cast<const int4 *>(
                               gpre + ((((long long)cu.run.v * V.nz + cu.run.za) * V.ny + y) * V.nx + xx) * C_OUT) +
                           c;
-#pragma unroll 4
+        // eight reads in flight: these warps' own chain of reads, not the MMAs,
+        // can be the last to end (four in flight: a training step of 4 x 64^3
+        // cells 942 us, eight 924; sixteen spill, 972)
+#pragma unroll 8
         for (int z = 0; z < cu.run.n; ++z) {
           const int4 q = src[z * plane * NCO];
           const __nv_bfloat162 *h = reinterpret_cast<const __nv_bfloat162 *>(&q);
