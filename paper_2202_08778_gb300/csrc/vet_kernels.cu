@@ -1115,15 +1115,19 @@ __device__ __forceinline__ void kahan2(float2 &s, float2 &nc, float2 c, float2 x
 // with the primary direction's coefficient pairs.  E and P_ii go into a staged
 // tile's partial sums pk, which the compensated sums take once per tile, the
 // others straight into mom.  Block edges other than 8 and 16 keep P_ij that way
-// too: their unpaired pass took the octants in turn, whose P_ij cancel; the
-// pairs of one octant pair after another do not, and straight sums of them left
-// f 6.9e-8 off, RMS, where it was 5.9e-8 (edge 6, 192 directions; now 5.6e-8).
+// too and sum F by tile before it is added: their unpaired pass took the octants
+// in turn, whose P_ij and F cancel; the pairs of one octant pair after another do
+// not, and straight sums of them left f 6.9e-8 off, RMS, where it was 5.9e-8 (edge
+// 6, 192 directions; now 5.6e-8), and F 1.4 times as far off as that pass (by tile
+// 0.99; 192 directions, anisotropic intensities).
 template <int BC>
 struct PairSums {
   static constexpr int kComp = BC ? 4 : 7;  // compensated sums: E, P_ii (, P_ij)
   static __device__ __forceinline__ constexpr int comp(int i) { return i ? 3 + i : 0; }
-  float2 mom[10], nc[kComp], pk[kComp];
+  float2 mom[10], nc[kComp], pk[kComp], pf[3];
   __device__ __forceinline__ PairSums() {
+#pragma unroll
+    for (int m = 0; m < 3; ++m) pf[m] = make_float2(0.f, 0.f);
 #pragma unroll
     for (int m = 0; m < 10; ++m) mom[m] = make_float2(0.f, 0.f);
 #pragma unroll
@@ -1138,7 +1142,10 @@ struct PairSums {
     pk[0] = __ffma2_rn(c[0], sum, pk[0]);
     if (WANT_F) {
 #pragma unroll
-      for (int m = 1; m < 4; ++m) mom[m] = __ffma2_rn(c[m], dif, mom[m]);
+      for (int m = 1; m < 4; ++m) {
+        if (BC == 0) pf[m - 1] = __ffma2_rn(c[m], dif, pf[m - 1]);
+        else mom[m] = __ffma2_rn(c[m], dif, mom[m]);
+      }
     }
 #pragma unroll
     for (int m = 4; m < 10; ++m) {
@@ -1146,8 +1153,16 @@ struct PairSums {
       else mom[m] = __ffma2_rn(c[m], sum, mom[m]);
     }
   }
-  // a staged tile's partial sums into the compensated sums
+  // a staged tile's partial sums into the compensated sums and F
+  template <bool WANT_F>
   __device__ __forceinline__ void fold() {
+    if (WANT_F && BC == 0) {
+#pragma unroll
+      for (int m = 0; m < 3; ++m) {
+        mom[1 + m] = __fadd2_rn(mom[1 + m], pf[m]);
+        pf[m] = make_float2(0.f, 0.f);
+      }
+    }
     const float2 one = make_float2(1.f, 1.f);
 #pragma unroll
     for (int i = 0; i < kComp; ++i) {
@@ -1409,7 +1424,7 @@ __global__ void __launch_bounds__(pair_max_threads(BC), pair_bound_ctas(BC))
         ps.template add<kWantF>(lds_f4(cpa), lds_f4(cpa + 16), lds_f4(cpa + 32), lds_f4(cpa + 48), lds_f4(cpa + 64), m1, m2);
       }
     }
-    if (MODE != 1 && !ORDERED) ps.fold();
+    if (MODE != 1 && !ORDERED) ps.template fold<kWantF>();
     __syncwarp();
     if ((threadIdx.x & 31) == 0) mbar_arrive(&empty[st]);
     if (threadIdx.x == 0) {
@@ -1446,7 +1461,7 @@ __global__ void __launch_bounds__(pair_max_threads(BC), pair_bound_ctas(BC))
                                                             offsetof(TplHead<float>, cp));
         ps.template add<kWantF>(__ldg(cp), __ldg(cp + 1), __ldg(cp + 2), __ldg(cp + 3), __ldg(cp + 4), m1, m2);
       }
-      ps.fold();
+      ps.template fold<kWantF>();
     }
     if (threadIdx.x == 0) split_count[slot] = 0;  // ready for the next call
   } else if (MODE != 1 && slot >= 0) {
