@@ -225,7 +225,7 @@ cudaError_t launch_face_level(const GridDims &g, const R *kappa, const R *S, con
 // time; the last r CTAs' work is then cut into k shares of their direction
 // tiles (k CTAs each), so that the tail takes about ceil(k r / wave) / k of
 // a CTA's time.  The shares' partial moments meet in `part`
-// ([slot][share][28][threads] floats) and the last share of a slot to
+// ([slot][share][28, or 34 at edges other than 8 and 16][threads] floats) and the last share of a slot to
 // finish (counted in `count`, which it resets) adds them in order and writes
 // the outputs.
 //

@@ -815,6 +815,9 @@ __host__ __device__ constexpr int pair_min_ctas(int B) {
 // launch bounds of the kernel compiled for block edge BC
 constexpr int pair_max_threads(int BC) { return BC ? pair_threads(BC) : 512; }
 constexpr int pair_bound_ctas(int BC) { return BC ? pair_min_ctas(BC) : 2; }
+// a share's partial sums per thread: ten moments of two cells and the
+// compensations of the compensated ones (PairSums)
+__host__ __device__ constexpr int pair_share_vals(int B) { return B == 8 || B == 16 ? 28 : 34; }
 constexpr int kPairStagesMax = 16;  // staging ring depth limit of the paired cell pass
 
 // Shared-memory loads at 32-bit shared-window addresses.  volatile keeps
@@ -1108,6 +1111,15 @@ __device__ __forceinline__ void kahan2(float2 &s, float2 &nc, float2 c, float2 x
   const float2 t = __fadd2_rn(s, y);
   nc = __fadd2_rn(y, neg2(__fadd2_rn(t, neg2(s))));
   s = t;
+}
+
+// s += v, returns the exact rounding of it (Knuth's TwoSum): a share's sum is of
+// the running sum's size, so that kahan2's rounding of v + nc would count.
+__device__ __forceinline__ float2 two_sum2(float2 &s, float2 v) {
+  const float2 t = __fadd2_rn(s, v), b = __fadd2_rn(t, neg2(s));
+  const float2 e = __fadd2_rn(__fadd2_rn(s, neg2(__fadd2_rn(t, neg2(b)))), __fadd2_rn(v, neg2(b)));
+  s = t;
+  return e;
 }
 
 // The moments of an antipodal pair's intensities m1 = (I(c, d), I(c', -d)) and
@@ -1448,11 +1460,10 @@ __global__ void __launch_bounds__(pair_max_threads(BC), pair_bound_ctas(BC))
     __syncthreads();
     if (!s_last) return;
     __threadfence();
-    const float2 one = make_float2(1.f, 1.f);
     const float2 *src = reinterpret_cast<const float2 *>(split_part) + (size_t)slot * (g.ndir >> 1) * 2 * NT + threadIdx.x;
     for (int d0 = 0; d0 < g.ndir; d0 += dt) {
       const int nd = min(dt, g.ndir - d0);
-#pragma unroll 4
+#pragma unroll(BC ? 4 : 2)  // edges other than 8 and 16 have no registers for more
       for (int j = 0; j < nd; j += 2) {
         const int pair = (d0 + j) >> 1;
         const float2 m1 = __ldcg(src + (size_t)pair * 2 * NT), m2 = __ldcg(src + (size_t)pair * 2 * NT + NT);
@@ -1467,9 +1478,10 @@ __global__ void __launch_bounds__(pair_max_threads(BC), pair_bound_ctas(BC))
   } else if (MODE != 1 && slot >= 0) {
     // one share of a split work item: its partial sums go to the slot's
     // scratch, and the share that finishes last adds all of them in order (the
-    // compensated sums as compensated sums, but for P_ij's last compensation;
-    // the same bits whichever finishes last) and writes the outputs
-    constexpr int kVals = 28;
+    // compensated sums exactly, their compensations and the additions' roundings
+    // beside them; the same bits whichever finishes last) and writes the outputs
+    constexpr int kComp = PairSums<BC>::kComp, kVals = pair_share_vals(BC);
+    static_assert(kVals == 2 * (10 + kComp), "a share's sums and their compensations");
     __shared__ int s_last;
     float *mine = split_part + ((size_t)slot * ksplit + share) * kVals * NT + threadIdx.x;
 #pragma unroll
@@ -1478,7 +1490,7 @@ __global__ void __launch_bounds__(pair_max_threads(BC), pair_bound_ctas(BC))
       mine[(2 * m + 1) * NT] = mom[m].y;
     }
 #pragma unroll
-    for (int m = 0; m < 4; ++m) {
+    for (int m = 0; m < kComp; ++m) {
       mine[(20 + 2 * m) * NT] = nc[m].x;
       mine[(21 + 2 * m) * NT] = nc[m].y;
     }
@@ -1488,29 +1500,28 @@ __global__ void __launch_bounds__(pair_max_threads(BC), pair_bound_ctas(BC))
     __syncthreads();
     if (!s_last) return;
     __threadfence();
-    const float2 one = make_float2(1.f, 1.f);
 #pragma unroll
     for (int m = 0; m < 10; ++m) mom[m] = make_float2(0.f, 0.f);
 #pragma unroll
-    for (int m = 0; m < 4; ++m) nc[m] = make_float2(0.f, 0.f);
+    for (int m = 0; m < kComp; ++m) nc[m] = make_float2(0.f, 0.f);
     for (int r = 0; r < ksplit; ++r) {
       const float *other = split_part + ((size_t)slot * ksplit + r) * kVals * NT + threadIdx.x;
-      float2 pm[10], pn[4];
 #pragma unroll
-      for (int m = 0; m < 10; ++m) pm[m] = make_float2(__ldcg(other + (2 * m) * NT), __ldcg(other + (2 * m + 1) * NT));
-#pragma unroll
-      for (int m = 0; m < 4; ++m) pn[m] = make_float2(__ldcg(other + (20 + 2 * m) * NT), __ldcg(other + (21 + 2 * m) * NT));
-      nc[0] = __fadd2_rn(nc[0], pn[0]);
-      kahan2(mom[0], nc[0], one, pm[0]);
-#pragma unroll
-      for (int m = 0; m < 3; ++m) {
-        nc[1 + m] = __fadd2_rn(nc[1 + m], pn[1 + m]);
-        kahan2(mom[4 + m], nc[1 + m], one, pm[4 + m]);
+      for (int m = 0; m < 10; ++m) {
+        const float2 v = make_float2(__ldcg(other + (2 * m) * NT), __ldcg(other + (2 * m + 1) * NT));
+        if (m == 0 || (m > 3 && m - 3 < kComp)) {
+          const int i = m ? m - 3 : 0;
+          const float2 c = make_float2(__ldcg(other + (20 + 2 * i) * NT), __ldcg(other + (21 + 2 * i) * NT));
+          nc[i] = __fadd2_rn(nc[i], __fadd2_rn(c, two_sum2(mom[m], v)));
+        } else {
+          mom[m] = __fadd2_rn(mom[m], v);
+        }
       }
+    }
 #pragma unroll
-      for (int m = 1; m < 4; ++m) mom[m] = __fadd2_rn(mom[m], pm[m]);
-#pragma unroll
-      for (int m = 7; m < 10; ++m) mom[m] = __fadd2_rn(mom[m], pm[m]);
+    for (int i = 0; i < kComp; ++i) {
+      const int m = PairSums<BC>::comp(i);
+      mom[m] = __fadd2_rn(mom[m], nc[i]);
     }
     if (threadIdx.x == 0) split_count[slot] = 0;  // ready for the next call
   }
@@ -2091,7 +2102,7 @@ TailPlan plan_tail_split(int B, int nblk, int nsm, int ndir, int dir_tile) {
   if (p.k == 1) return p;
   p.nfull = total - r;
   p.slots = r;
-  p.part_bytes = (size_t)r * p.k * 28 * pair_threads(B) * sizeof(float);
+  p.part_bytes = (size_t)r * p.k * pair_share_vals(B) * pair_threads(B) * sizeof(float);
   return p;
 }
 
