@@ -117,11 +117,7 @@ void free_ctx(vet_ctx *c) {
 vet_status build_schedule(vet_ctx *c, int group) {
   const int nb[3] = {c->dims.nbx, c->dims.nby, c->dims.nbz};
   c->nlevels = nb[0] + nb[1] + nb[2] - 2;
-  int sms = 0;
-  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->cfg.device) != cudaSuccess || sms < 1) {
-    cudaGetLastError();
-    sms = 1;
-  }
+  const int sms = std::max(1, c->dims.nsm);
   const bool paired = c->dims.face_paired != 0;
   const long long slots = (paired ? 2LL : 3LL) * sms;
   std::vector<int> lg(c->nlevels, group), off(c->nlevels + 1, 0);
@@ -184,12 +180,8 @@ vet_status build_schedule(vet_ctx *c, int group) {
 // grid's last wave leaves SMs idle, a batch's does not.
 vet::TailPlan split_plan(vet_ctx *c) {
   vet::TailPlan best;
-  int nsm = 0;
-  if (!c->want_split || !(c->dims.paired || c->fp64)) return best;
-  if (cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, c->cfg.device) != cudaSuccess) {
-    cudaGetLastError();
-    return best;
-  }
+  const int nsm = c->dims.nsm;
+  if (!c->want_split || !(c->dims.paired || c->fp64) || nsm < 1) return best;
   const int B = c->grid.block;
   for (int want = 1; want <= vet::kMaxTune; ++want) {
     const vet::TailPlan p = c->fp64 ? vet::plan_cell_split64(B, c->nblk, nsm, c->N, vet::cell_tile_fit(B, want, true))
@@ -203,6 +195,10 @@ vet::TailPlan split_plan(vet_ctx *c) {
 template <typename R>
 vet_status build_context(vet_ctx *c) {
   const int B = c->grid.block, N = c->N;
+  if (cudaDeviceGetAttribute(&c->dims.nsm, cudaDevAttrMultiProcessorCount, c->cfg.device) != cudaSuccess) {
+    cudaGetLastError();
+    c->dims.nsm = 0;
+  }
   std::vector<int> order(N);
   int ob[9];
   vet::geom::internal_order(N, c->dirs_ext.data(), order.data(), ob);
@@ -1078,6 +1074,9 @@ VET_API vet_status vet_batch_create(vet_batch **out, int n, const vet_grid *grid
     }
     b->ctx.push_back(c);
   }
+  for (vet_ctx *c : b->ctx)
+    for (vet_ctx *o : b->ctx)
+      if (o != c) c->dims.beside += o->dims.ncell;
   DeviceGuard dg(b->device);
   cudaError_t e = cudaStreamCreateWithFlags(&b->origin, cudaStreamNonBlocking);
   if (!e) e = cudaEventCreateWithFlags(&b->forked, cudaEventDisableTiming);

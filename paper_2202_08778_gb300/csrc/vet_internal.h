@@ -132,6 +132,8 @@ struct GridDims {
   const uint32_t *cell_rec;  // ray records, see CellRec and NodeRec
   const uint2 *node_rec;
   const double *exp64;  // FP64 passes: tables of the segment weight (vet_exp64.h)
+  int nsm;              // SMs of the device (0: unknown)
+  long long beside;     // cells of the grids whose passes run beside this one's (a batch's other members)
 };
 
 // Ray records.  Where a ray leaves its block, through which entry of the exit
@@ -210,7 +212,7 @@ struct FaceItem {
 // mbarrier); a wait that gives up ORs a code into *status and the kernel
 // returns early with its outputs incomplete.
 //   status bits: 1 face-pass staging, 2 cell-pass staging, 4 cell-pass buffer
-//   release, 8 the final wait for copies still in flight.
+//   release or hand-over between two threads, 8 the final wait for copies still in flight.
 
 // Face pass of one wavefront level: nitems items of at most max_dirs
 // directions each.
@@ -247,7 +249,8 @@ TailPlan plan_tail_split(int B, int nblk, int nsm, int ndir, int dir_tile);
 // The same for the FP64 cell pass, whose shares always store partial moments
 // ([slot][share][14][threads] doubles), also on grids of less than one wave.
 TailPlan plan_cell_split64(int B, int nblk, int nsm, int ndir, int dir_tile);
-// Largest scratch of an ordered split (beyond: the grid runs unsplit).
+// Largest scratch of an ordered split (beyond: the grid runs unsplit, at edges
+// other than 8 and 16 with two threads a pair of cells).
 constexpr size_t kOrderedSplitMax = (size_t)128 << 20;
 
 // One grid of a merged launch of the paired FP32 cell pass (the batched
@@ -349,7 +352,9 @@ constexpr int kMaxPairBlock = 16;
 // Smallest block edge of the paired cell pass: below, a CTA's few cells do not
 // pay for its pairs of staged directions (cell pass, paired against unpaired: edge 4
 // 0.42 and 0.38 ms, 5 0.36 and 0.34, 6 0.43 and 0.56, 12 1.6 and 2.7; the paired
-// face pass is ahead from 2 on, 0.59 and 0.67 ms).
+// face pass is ahead from 2 on, 0.59 and 0.67 ms).  Those grids fill the SMs; what
+// leaves them idle runs in shares (TailPlan) or two threads a pair of cells (HALVES
+// in vet_kernels.cu), and is ahead of one ray a thread from one block on.
 constexpr int kMinPairBlock = 6;
 
 // Per-device kernel attributes; call with the context's device current.

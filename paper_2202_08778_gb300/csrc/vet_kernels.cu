@@ -20,6 +20,7 @@
 #include <algorithm>
 #include <cstddef>
 #include <cstdint>
+#include <type_traits>
 
 #include "vet_exp64.h"
 #include "vet_internal.h"
@@ -1104,17 +1105,31 @@ __device__ __forceinline__ void load_tile_pair(float4 *tile, TileShape ts, const
   }
 }
 
-// Compensated (Kahan) accumulation of t = c * x into s on packed pairs; nc
-// holds the negated compensation.
-__device__ __forceinline__ void kahan2(float2 &s, float2 &nc, float2 c, float2 x) {
-  const float2 y = __ffma2_rn(c, x, nc);
-  const float2 t = __fadd2_rn(s, y);
-  nc = __fadd2_rn(y, neg2(__fadd2_rn(t, neg2(s))));
+// The sums' operations on one cell's values and on those of a pair of cells:
+// the same roundings either way.
+__device__ __forceinline__ float add_rn(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ float2 add_rn(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float sub_rn(float a, float b) { return __fsub_rn(a, b); }
+__device__ __forceinline__ float2 sub_rn(float2 a, float2 b) { return __fadd2_rn(a, neg2(b)); }
+__device__ __forceinline__ float fma_rn(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ float2 fma_rn(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+__device__ __forceinline__ void set_all(float &v, float x) { v = x; }
+__device__ __forceinline__ void set_all(float2 &v, float x) { v = make_float2(x, x); }
+
+// Compensated (Kahan) accumulation of x into s; nc holds the negated
+// compensation.
+template <typename V>
+__device__ __forceinline__ void kahan(V &s, V &nc, V x) {
+  V one;
+  set_all(one, 1.f);
+  const V y = fma_rn(one, x, nc);
+  const V t = add_rn(s, y);
+  nc = sub_rn(y, sub_rn(t, s));
   s = t;
 }
 
 // s += v, returns the exact rounding of it (Knuth's TwoSum): a share's sum is of
-// the running sum's size, so that kahan2's rounding of v + nc would count.
+// the running sum's size, so that kahan's rounding of v + nc would count.
 __device__ __forceinline__ float2 two_sum2(float2 &s, float2 v) {
   const float2 t = __fadd2_rn(s, v), b = __fadd2_rn(t, neg2(s));
   const float2 e = __fadd2_rn(__fadd2_rn(s, neg2(__fadd2_rn(t, neg2(b)))), __fadd2_rn(v, neg2(b)));
@@ -1132,38 +1147,46 @@ __device__ __forceinline__ float2 two_sum2(float2 &s, float2 v) {
 // not, and straight sums of them left f 6.9e-8 off, RMS, where it was 5.9e-8 (edge
 // 6, 192 directions; now 5.6e-8), and F 1.4 times as far off as that pass (by tile
 // 0.99; 192 directions, anisotropic intensities).
-template <int BC>
+// V: float2 (the pair's sums) or float (one of its cells').
+template <int BC, typename V = float2>
 struct PairSums {
   static constexpr int kComp = BC ? 4 : 7;  // compensated sums: E, P_ii (, P_ij)
   static __device__ __forceinline__ constexpr int comp(int i) { return i ? 3 + i : 0; }
-  float2 mom[10], nc[kComp], pk[kComp], pf[3];
+  V mom[10], nc[kComp], pk[kComp], pf[3];
   __device__ __forceinline__ PairSums() {
 #pragma unroll
-    for (int m = 0; m < 3; ++m) pf[m] = make_float2(0.f, 0.f);
+    for (int m = 0; m < 3; ++m) set_all(pf[m], 0.f);
 #pragma unroll
-    for (int m = 0; m < 10; ++m) mom[m] = make_float2(0.f, 0.f);
+    for (int m = 0; m < 10; ++m) set_all(mom[m], 0.f);
 #pragma unroll
-    for (int m = 0; m < kComp; ++m) nc[m] = pk[m] = make_float2(0.f, 0.f);
+    for (int m = 0; m < kComp; ++m) {
+      set_all(nc[m], 0.f);
+      set_all(pk[m], 0.f);
+    }
+  }
+  // sum = I(d) + I(-d), dif = I(d) - I(-d)
+  template <bool WANT_F>
+  __device__ __forceinline__ void add(const V (&c)[10], V sum, V dif) {
+    pk[0] = fma_rn(c[0], sum, pk[0]);
+    if (WANT_F) {
+#pragma unroll
+      for (int m = 1; m < 4; ++m) {
+        if (BC == 0) pf[m - 1] = fma_rn(c[m], dif, pf[m - 1]);
+        else mom[m] = fma_rn(c[m], dif, mom[m]);
+      }
+    }
+#pragma unroll
+    for (int m = 4; m < 10; ++m) {
+      if (m < 7 || BC == 0) pk[m - 3] = fma_rn(c[m], sum, pk[m - 3]);
+      else mom[m] = fma_rn(c[m], sum, mom[m]);
+    }
   }
   template <bool WANT_F>
   __device__ __forceinline__ void add(float4 c01, float4 c23, float4 c45, float4 c67, float4 c89, float2 m1, float2 m2) {
     const float2 c[10] = {make_float2(c01.x, c01.y), make_float2(c01.z, c01.w), make_float2(c23.x, c23.y), make_float2(c23.z, c23.w),
                           make_float2(c45.x, c45.y), make_float2(c45.z, c45.w), make_float2(c67.x, c67.y), make_float2(c67.z, c67.w),
                           make_float2(c89.x, c89.y), make_float2(c89.z, c89.w)};
-    const float2 sum = __fadd2_rn(m1, m2), dif = __fadd2_rn(m1, neg2(m2));
-    pk[0] = __ffma2_rn(c[0], sum, pk[0]);
-    if (WANT_F) {
-#pragma unroll
-      for (int m = 1; m < 4; ++m) {
-        if (BC == 0) pf[m - 1] = __ffma2_rn(c[m], dif, pf[m - 1]);
-        else mom[m] = __ffma2_rn(c[m], dif, mom[m]);
-      }
-    }
-#pragma unroll
-    for (int m = 4; m < 10; ++m) {
-      if (m < 7 || BC == 0) pk[m - 3] = __ffma2_rn(c[m], sum, pk[m - 3]);
-      else mom[m] = __ffma2_rn(c[m], sum, mom[m]);
-    }
+    add<WANT_F>(c, add_rn(m1, m2), sub_rn(m1, m2));
   }
   // a staged tile's partial sums into the compensated sums and F
   template <bool WANT_F>
@@ -1171,22 +1194,22 @@ struct PairSums {
     if (WANT_F && BC == 0) {
 #pragma unroll
       for (int m = 0; m < 3; ++m) {
-        mom[1 + m] = __fadd2_rn(mom[1 + m], pf[m]);
-        pf[m] = make_float2(0.f, 0.f);
+        mom[1 + m] = add_rn(mom[1 + m], pf[m]);
+        set_all(pf[m], 0.f);
       }
     }
-    const float2 one = make_float2(1.f, 1.f);
 #pragma unroll
     for (int i = 0; i < kComp; ++i) {
-      kahan2(mom[comp(i)], nc[i], one, pk[i]);
-      pk[i] = make_float2(0.f, 0.f);
+      kahan(mom[comp(i)], nc[i], pk[i]);
+      set_all(pk[i], 0.f);
     }
   }
 };
 
 // the head fields the paired cell pass reads at fixed offsets
 static_assert(offsetof(TplHead<float>, sgn) == 16 && offsetof(TplHead<float>, ext) == 28 &&
-                  offsetof(TplHead<float>, mirror) == 32 && offsetof(TplHead<float>, cp) % 16 == 0,
+                  offsetof(TplHead<float>, mirror) == 32 && offsetof(TplHead<float>, c) % 16 == 0 &&
+                  offsetof(TplHead<float>, cp) % 16 == 0,
               "TplHead<float> layout");
 
 // A thread's lower-half cell (z < B/2): 4 x 4 x 2 bricks, warp-major.  Layer
@@ -1198,14 +1221,15 @@ template <int BC>
 struct PairCell {
   int B, q, x, y, z;  // place among the lower half's cells; the cell
   bool active;        // false: a thread past the CTA's cells (it redoes the last one and writes nothing)
-  __device__ __forceinline__ PairCell(int edge, int part, int parts, uint32_t tid) {
+  // cells: of a CTA, a multiple of 32 (compiled edges: pair_threads); i: the thread's among them
+  __device__ __forceinline__ PairCell(int edge, int part, int parts, int cells, uint32_t i) {
     B = BC ? BC : edge;
     if constexpr (BC != 0) {
-      q = part * pair_threads(BC) + (int)tid;
+      q = part * pair_threads(BC) + (int)i;
       active = true;
     } else {
       const int half = (B * B * B + 1) / 2;
-      q = part * pair_threads(B) + (int)tid;
+      q = part * cells + (int)i;
       active = q < half;
       q = min(q, half - 1);
     }
@@ -1238,7 +1262,19 @@ __device__ __forceinline__ uint32_t fresh_tid() {
 }
 
 // ORDERED (moment modes): every CTA is one share of a work item, see TailPlan.
-template <int MODE, int BC, bool MERGED, bool ORDERED = false>
+// HALVES (runtime edge, unsplit): two threads a pair of cells (c, c'), half a CTA
+// apart, each of which marches one of the pair's two ray pairs per antipodal pair
+// of directions, the primary's and the antipode's in turn (a cell's two rays are
+// long and short), hands one value to the other through shared memory and sums
+// one of the two cells: the same bits as one thread a pair, from half the
+// marches a thread in twice the threads.  For launches that leave SMs idle, where
+// a thread's chain of marches is the time: a step of a ray pair takes longer than
+// one of a ray, so one thread a pair loses there to one ray a thread.  Closures of
+// 3072 directions, one ray a thread, one thread a pair, two: 64 blocks of edge 6
+// 4.14, 7.36 and 3.65 ms; 27 of edge 12 5.80, 7.65 and 4.16; 8 of edge 14 5.38,
+// 9.71 and 4.34; a batch of one grid of 64 blocks of edge 6, 192 directions, 297,
+// 494 and 258 us.
+template <int MODE, int BC, bool MERGED, bool ORDERED = false, bool HALVES = false>
 __global__ void __launch_bounds__(pair_max_threads(BC), pair_bound_ctas(BC))
     cell_pair_kernel(GridDims g_arg, int parts, int dt, int nstage, const float *__restrict__ kappa_arg,
                      const float *__restrict__ S_arg, const unsigned char *__restrict__ tpl_arg,
@@ -1252,6 +1288,9 @@ __global__ void __launch_bounds__(pair_max_threads(BC), pair_bound_ctas(BC))
   __shared__ __align__(8) uint64_t full[kPairStagesMax], empty[kPairStagesMax];
   constexpr int kOrdMax = 1024;  // direction sets up to nside = 8 keep their order in shared memory
   __shared__ int s_ord[kOrdMax];
+  constexpr int kHandovers = 8;  // warps of one orientation of a HALVES CTA, at most
+  __shared__ __align__(8) uint64_t handed[HALVES ? kHandovers : 1];
+  static_assert(!HALVES || (BC == 0 && !ORDERED && !MERGED), "a launch of a runtime edge");
   // a merged launch (several grids of one block edge) takes its grid from the
   // work item's entry of `grids`; a single grid's launch from the arguments
   const CellGrid *gd = nullptr;
@@ -1273,7 +1312,6 @@ __global__ void __launch_bounds__(pair_max_threads(BC), pair_bound_ctas(BC))
   const TileShape ts = cell_tile(B);
   const TplLayout TL = tpl_layout<float>(B);
   const CellSlot CS = cell_slot(B);
-  const int fstride = g.fstride;
   float4 *tile = reinterpret_cast<float4 *>(smem);
   unsigned char *ring = smem + align16(sizeof(float4) * (size_t)ts.elems);
   const uint32_t ring_s = smem_u32(ring);
@@ -1312,6 +1350,8 @@ __global__ void __launch_bounds__(pair_max_threads(BC), pair_bound_ctas(BC))
       mbar_init(&full[s], 1);
       mbar_init(&empty[s], nwarps);
     }
+    if (HALVES)
+      for (int w = 0; w < nwarps / 2; ++w) mbar_init(&handed[w], 2);
     mbar_fence_init();
     griddep_wait();  // the faces are the face pass's output
     while (issued < ntiles && issued < nstage) issue_tile(issued++);
@@ -1323,7 +1363,12 @@ __global__ void __launch_bounds__(pair_max_threads(BC), pair_bound_ctas(BC))
   __syncthreads();
   if (MODE != 1) griddep_launch_dependents();  // the floor rule's launch overlaps the pass
 
-  const PairCell<BC> pc(B, part, parts, threadIdx.x);
+  const int cells = HALVES ? NT / 2 : NT;  // of the lower half, of this CTA
+  auto pair_cell = [&](uint32_t tid) {
+    return PairCell<BC>(B, part, parts, cells, HALVES && (int)tid >= cells ? tid - cells : tid);
+  };
+  const int other = HALVES && (int)threadIdx.x >= cells;  // HALVES: the thread sums c', not c
+  const PairCell<BC> pc = pair_cell(threadIdx.x);
   const uint32_t tile_s = smem_u32(tile);
   const uint32_t t1 = tile_s + 16u * (uint32_t)(pc.x + ts.sy * pc.y + ts.sz * pc.z);
   constexpr bool kWantF = MODE == 0;
@@ -1332,8 +1377,9 @@ __global__ void __launch_bounds__(pair_max_threads(BC), pair_bound_ctas(BC))
   // a staged tile's pairs add into plain partial sums first, folded into the
   // compensated sums once per tile (fewer f32x2 operations and fewer
   // register moves than a compensated addition per pair)
-  PairSums<BC> ps;
-  float2(&mom)[10] = ps.mom, (&nc)[PairSums<BC>::kComp] = ps.nc;
+  using Sum = std::conditional_t<HALVES, float, float2>;
+  PairSums<BC, Sum> ps;
+  Sum(&mom)[10] = ps.mom, (&nc)[PairSums<BC>::kComp] = ps.nc;
   // the tile entry set to zero: the identity segment
   const uint32_t id_s = tile_s + 16u * (uint32_t)(ts.elems - 1);
   const uint32_t fW = 4u * (uint32_t)(B + 2);
@@ -1364,7 +1410,7 @@ __global__ void __launch_bounds__(pair_max_threads(BC), pair_bound_ctas(BC))
   // (slot ps), the record of its start cell in that direction
   auto single = [&](uint32_t ps, int k, bool mirror_cell) -> float {
     const int v = ord_smem ? s_ord[k] : __ldg(order + k);
-    const PairCell<BC> c(B, part, parts, fresh_tid());
+    const PairCell<BC> c = pair_cell(fresh_tid());
     const int x = mirror_cell ? B - 1 - c.x : c.x, y = mirror_cell ? B - 1 - c.y : c.y, z = mirror_cell ? B - 1 - c.z : c.z;
     const uint32_t tstart = tile_s + 16u * (uint32_t)(x + ts.sy * y + ts.sz * z);
     const uint32_t *r = g.cell_rec + (size_t)order_dir(v) * (B * B2) + cell_rec_index(B, x, y, z);
@@ -1373,6 +1419,11 @@ __global__ void __launch_bounds__(pair_max_threads(BC), pair_bound_ctas(BC))
     return march_one(tstart, ps + CS.cev, rec.last(), Iin.x);
   };
 
+  // HALVES: the direction that this thread marches of the pair (k, k + 1); its
+  // record is read a march ahead, since few warps are there to hide the read
+  // (64 blocks of edge 6, 3072 directions: trace 3.70 -> 3.33 ms)
+  auto turn = [&](int k) { return k + ((k >> 1 & 1) ^ other); };
+  uint32_t next_rec = HALVES ? record(turn(0)) : 0u;
   bool ok = true;
   const uint32_t full_s = smem_u32(full), empty_s = smem_u32(empty);
   for (int t = 0; t < ntiles && ok; ++t) {
@@ -1395,48 +1446,96 @@ __global__ void __launch_bounds__(pair_max_threads(BC), pair_bound_ctas(BC))
     if (threadIdx.x == 0) consumed = t + 1;
     const int nd = min(dt, g.ndir - (tile0 + t) * dt);
     const uint32_t buf = ring_s + (uint32_t)(st * stage_bytes);
-    for (int j = 0; j < nd; j += 2) {  // the antipodal pair (j, j + 1)
-      const uint32_t sa = buf + (uint32_t)(CS.bytes * j), sb = sa + (uint32_t)CS.bytes;
-      const int mirror = (int)lds_2x32(sa + 32).x;
-      const int k = (tile0 + t) * dt + j;
-      const CellRec rb{record(k + 1)};
-      float2 m1, m2;  // m1 = (I(c, d), I(c', -d)), m2 = (I(c, -d), I(c', d))
-      if (mirror) {
-        // the mirror cell's ray in the antipode has the upwind-frame
-        // coordinates of c's in the primary direction: one record for both
-        const CellRec ra{record(k)};
-        const float2 I1 = entry(sa, ra, sa + CS.faces, sb + CS.faces);
-        m1 = march_pair(t1, id_s, sa + CS.cev, ra.last(), I1);
-        const float2 I2 = entry(sb, rb, sb + CS.faces, sa + CS.faces);
-        m2 = march_pair(t1, id_s, sb + CS.cev, rb.last(), I2);
-      } else {
-        // the pair's templates differ (near-tied plane crossings ordered
-        // differently): each ray follows its own direction's template
-        m1 = make_float2(single(sa, k, false), single(sb, k + 1, true));
-        m2 = make_float2(single(sb, k + 1, false), single(sa, k, true));
-      }
-      if (MODE == 1) {
-        const int ea = (int)lds_2x32(sa + 24).y, eb = (int)lds_2x32(sb + 24).y;  // the directions' public indices
-        const long long gc1 = pc.cell(g, bx, by, bz), gc2 = pc.mirror(g, bx, by, bz);
-        if (pc.active) {
-          I_out[(long long)ea * g.ncell + gc1] = m1.x;
-          I_out[(long long)eb * g.ncell + gc2] = m1.y;
-          I_out[(long long)eb * g.ncell + gc1] = m2.x;
-          I_out[(long long)ea * g.ncell + gc2] = m2.y;
+    if constexpr (HALVES) {
+      // both threads' values of the tile's pairs, [pair][thread], in turns of two
+      float2 *hand = reinterpret_cast<float2 *>(ring + (size_t)nstage * stage_bytes) + (t & 1) * (dt / 2) * NT + threadIdx.x;
+      for (int j = 0; j < nd; j += 2) {
+        const int k0 = t * dt + j, k = turn(k0), second = k - k0;  // 0: the primary's march, 1: the antipode's
+        const int ko = second ? k - 1 : k + 1;
+        const CellRec rec{next_rec};
+        next_rec = record(turn(min(k0 + 2, g.ndir - 2)));
+        const uint32_t sa = buf + (uint32_t)(CS.bytes * (j + second)), sb = second ? sa - (uint32_t)CS.bytes : sa + (uint32_t)CS.bytes;
+        float2 m;  // (I(c, its direction), I(c', the other one))
+        if ((int)lds_2x32(sa + 32).x) {
+          const float2 Iin = entry(sa, rec, sa + CS.faces, sb + CS.faces);
+          m = march_pair(t1, id_s, sa + CS.cev, rec.last(), Iin);
+        } else {
+          m = make_float2(single(sa, k, false), single(sb, ko, true));
         }
-      } else if (ORDERED) {
-        // this pair's place in the item's list: pairs are consecutive in the order
-        const int pair = ((tile0 + t) * dt + j) >> 1;
-        float2 *dst = reinterpret_cast<float2 *>(split_part) +
-                      ((size_t)slot * (g.ndir >> 1) + pair) * 2 * NT + threadIdx.x;
-        __stcg(dst, m1);
-        __stcg(dst + NT, m2);
-      } else {
-        const uint32_t cpa = sa + (uint32_t)offsetof(TplHead<float>, cp);
-        ps.template add<kWantF>(lds_f4(cpa), lds_f4(cpa + 16), lds_f4(cpa + 32), lds_f4(cpa + 48), lds_f4(cpa + 64), m1, m2);
+        if (MODE == 1) {
+          const int ea = (int)lds_2x32(sa + 24).y, eb = (int)lds_2x32(sb + 24).y;
+          if (pc.active) {
+            I_out[(long long)ea * g.ncell + pc.cell(g, bx, by, bz)] = m.x;
+            I_out[(long long)eb * g.ncell + pc.mirror(g, bx, by, bz)] = m.y;
+          }
+        } else {
+          hand[(j >> 1) * NT] = m;
+        }
       }
+      if (MODE != 1) {
+        // a hand-over is complete when both warps have stored theirs; a buffer
+        // is stored to again only after the next one is
+        __syncwarp();
+        uint64_t *bar = &handed[(threadIdx.x >> 5) % (nwarps / 2)];
+        if ((threadIdx.x & 31) == 0) mbar_arrive(bar);
+        if (!mbar_wait_sleep_warp(smem_u32(bar), (uint32_t)(t & 1), spin_limit, status, 4)) { ok = false; break; }
+        const float2 *from = hand + (other ? -cells : cells);
+        for (int j = 0; j < nd; j += 2) {
+          const float2 a = hand[(j >> 1) * NT], b = from[(j >> 1) * NT];
+          const float mine = other ? a.y : a.x, got = other ? b.y : b.x;
+          const uint32_t ca = buf + (uint32_t)(CS.bytes * j) + (uint32_t)offsetof(TplHead<float>, c);
+          const float4 c03 = lds_f4(ca), c47 = lds_f4(ca + 16);
+          const float2 c89 = lds_f2(ca + 32);
+          const float c[10] = {c03.x, c03.y, c03.z, c03.w, c47.x, c47.y, c47.z, c47.w, c89.x, c89.y};
+          const float dif = __fsub_rn(mine, got);
+          ps.template add<kWantF>(c, __fadd_rn(mine, got), (t * dt + j) >> 1 & 1 ? -dif : dif);
+        }
+        ps.template fold<kWantF>();
+      }
+    } else {
+      for (int j = 0; j < nd; j += 2) {  // the antipodal pair (j, j + 1)
+        const uint32_t sa = buf + (uint32_t)(CS.bytes * j), sb = sa + (uint32_t)CS.bytes;
+        const int mirror = (int)lds_2x32(sa + 32).x;
+        const int k = (tile0 + t) * dt + j;
+        const CellRec rb{record(k + 1)};
+        float2 m1, m2;  // m1 = (I(c, d), I(c', -d)), m2 = (I(c, -d), I(c', d))
+        if (mirror) {
+          // the mirror cell's ray in the antipode has the upwind-frame
+          // coordinates of c's in the primary direction: one record for both
+          const CellRec ra{record(k)};
+          const float2 I1 = entry(sa, ra, sa + CS.faces, sb + CS.faces);
+          m1 = march_pair(t1, id_s, sa + CS.cev, ra.last(), I1);
+          const float2 I2 = entry(sb, rb, sb + CS.faces, sa + CS.faces);
+          m2 = march_pair(t1, id_s, sb + CS.cev, rb.last(), I2);
+        } else {
+          // the pair's templates differ (near-tied plane crossings ordered
+          // differently): each ray follows its own direction's template
+          m1 = make_float2(single(sa, k, false), single(sb, k + 1, true));
+          m2 = make_float2(single(sb, k + 1, false), single(sa, k, true));
+        }
+        if (MODE == 1) {
+          const int ea = (int)lds_2x32(sa + 24).y, eb = (int)lds_2x32(sb + 24).y;  // the directions' public indices
+          const long long gc1 = pc.cell(g, bx, by, bz), gc2 = pc.mirror(g, bx, by, bz);
+          if (pc.active) {
+            I_out[(long long)ea * g.ncell + gc1] = m1.x;
+            I_out[(long long)eb * g.ncell + gc2] = m1.y;
+            I_out[(long long)eb * g.ncell + gc1] = m2.x;
+            I_out[(long long)ea * g.ncell + gc2] = m2.y;
+          }
+        } else if (ORDERED) {
+          // this pair's place in the item's list: pairs are consecutive in the order
+          const int pair = ((tile0 + t) * dt + j) >> 1;
+          float2 *dst = reinterpret_cast<float2 *>(split_part) +
+                        ((size_t)slot * (g.ndir >> 1) + pair) * 2 * NT + threadIdx.x;
+          __stcg(dst, m1);
+          __stcg(dst + NT, m2);
+        } else {
+          const uint32_t cpa = sa + (uint32_t)offsetof(TplHead<float>, cp);
+          ps.template add<kWantF>(lds_f4(cpa), lds_f4(cpa + 16), lds_f4(cpa + 32), lds_f4(cpa + 48), lds_f4(cpa + 64), m1, m2);
+        }
+      }
+      if (MODE != 1 && !ORDERED) ps.template fold<kWantF>();
     }
-    if (MODE != 1 && !ORDERED) ps.template fold<kWantF>();
     __syncwarp();
     if ((threadIdx.x & 31) == 0) mbar_arrive(&empty[st]);
     if (threadIdx.x == 0) {
@@ -1450,7 +1549,9 @@ __global__ void __launch_bounds__(pair_max_threads(BC), pair_bound_ctas(BC))
     for (int t = consumed; t < issued; ++t)
       if (!mbar_wait_sleep(full_s + 8 * (t % nstage), (uint32_t)((t / nstage) & 1), kDrainPolls)) atomicOr(status, 8);
   }
-  if (MODE != 1 && ORDERED) {
+  if constexpr (HALVES) {
+    // never split
+  } else if (MODE != 1 && ORDERED) {
     // the share that finishes last adds every pair's values, tile by tile as
     // the unsplit pass does, and writes the outputs
     __shared__ int s_last;
@@ -1536,19 +1637,26 @@ __global__ void __launch_bounds__(pair_max_threads(BC), pair_bound_ctas(BC))
     const bool staged = BC != 0 && (size_t)nstage * stage_bytes >= sizeof(float) * NV * CELLS;
     float emax = 0.f;
     if (__syncthreads_and(ok)) {  // also: every warp is done with the ring
-      float Ms[2][10];
+      constexpr int kMine = HALVES ? 1 : 2;  // cells of a thread
+      float Ms[kMine][10];
 #pragma unroll
       for (int m = 0; m < 10; ++m) {
-        Ms[0][m] = mom[m].x;
-        Ms[1][m] = mom[m].y;
+        if constexpr (HALVES) {
+          Ms[0][m] = mom[m];
+        } else {
+          Ms[0][m] = mom[m].x;
+          Ms[1][m] = mom[m].y;
+        }
       }
       float *st = reinterpret_cast<float *>(ring);
-      const PairCell<BC> c(B, part, parts, fresh_tid());
+      const uint32_t tid = fresh_tid();
+      const PairCell<BC> c = pair_cell(tid);
       const int zs = 2 * ((c.q >> 5) / (B2 / 16) - part * (L / 2)) + ((c.q & 31) >> 4);  // the lower cell's z slot
       const int li[2] = {(zs * B + c.y) * B + c.x, ((L + zs) * B + B - 1 - c.y) * B + B - 1 - c.x};
 #pragma unroll
-      for (int r = 0; r < 2; ++r) {
-        const long long gc = r ? c.mirror(g, bx, by, bz) : c.cell(g, bx, by, bz);
+      for (int r = 0; r < kMine; ++r) {
+        const bool mirror = HALVES ? (int)tid >= cells : r != 0;
+        const long long gc = mirror ? c.mirror(g, bx, by, bz) : c.cell(g, bx, by, bz);
         const float E = Ms[r][0];
         float v[NV];
         if (kWantF) {
@@ -2017,14 +2125,19 @@ void cell_launch(const GridDims &g, const R *kappa, const R *S, const unsigned c
       block_list, tp.nfull, tp.k, split ? (double *)split->part : nullptr, split ? split->count : nullptr);
 }
 
+// Dynamic shared memory of a paired cell-pass CTA where an SM holds `ctas` of them.
+inline long long pair_smem_limit(int ctas) {
+  constexpr long long kSmemPerSM = 233472, kReservedPerCta = 1024;
+  constexpr long long kStatic = 1024 * 4 + 2 * kPairStagesMax * 8 + 64;  // order, barriers, margin
+  return std::min<long long>(232448, kSmemPerSM / ctas - kReservedPerCta) - kStatic;
+}
+
 // Staging of the paired cell pass: directions per tile (whole antipodal
 // pairs: the tuned tile rounded up to even) and ring depth, the most stages
 // (at most kPairStagesMax) that fit the shared memory of one of the
 // pair_min_ctas(B) CTAs an SM holds beside the paired tile.
 inline void pair_staging(int B, int want, int &dt, int &nstage) {
-  constexpr long long kSmemPerSM = 233472, kReservedPerCta = 1024;
-  constexpr long long kStatic = 1024 * 4 + 2 * kPairStagesMax * 8 + 64;  // order, barriers, margin
-  const long long per_cta = std::min<long long>(232448, kSmemPerSM / pair_min_ctas(B) - kReservedPerCta) - kStatic;
+  const long long per_cta = pair_smem_limit(pair_min_ctas(B));
   // untuned: the tile the autotuner picks on the 128^3 workload; other edges keep
   // the unpaired pass's 4, and with it its plain sums of at most four directions
   dt = want > 0 ? want : (B == 8 || B == 16 ? 8 : 4);
@@ -2108,6 +2221,42 @@ TailPlan plan_tail_split(int B, int nblk, int nsm, int ndir, int dir_tile) {
 
 namespace {
 
+// A launch of the paired cell pass with two threads a pair of cells (HALVES):
+// the unsplit launch's direction tile, and with it its bits.  Taken where the CTAs
+// of the whole launch and of the grids beside it fit the SMs at once: past that
+// one thread a pair has as many warps as the SMs run, without the hand-overs.
+struct HalvesPlan {
+  int parts = 0, threads = 0, nstage = 0;  // parts = 0: one thread a pair
+  size_t smem = 0;
+};
+HalvesPlan plan_halves(const GridDims &g, int nblk, int dt) {
+  const int half = (g.B * g.B * g.B + 1) / 2;
+  const double grids = 1.0 + (double)g.beside / (double)g.ncell;
+  // CTAs of `warps` warps of either orientation, `ctas` of them an SM
+  auto fit = [&](int warps, int ctas) {
+    HalvesPlan p;
+    p.threads = 64 * warps;
+    p.parts = (half + 32 * warps - 1) / (32 * warps);
+    const long long hand = (long long)dt * p.threads * (long long)sizeof(float2);
+    const long long n = (pair_smem_limit(ctas) - (long long)pair_smem_bytes(g.B, 0) - hand) / ((long long)dt * cell_slot(g.B).bytes);
+    if (n < 2 || (double)nblk * p.parts * grids > (double)g.nsm * ctas) return HalvesPlan{};
+    p.nstage = (int)std::min<long long>(kPairStagesMax, n);
+    // one CTA an SM: room for no second one, so that they spread over the SMs also
+    // where another grid's CTAs are (two grids of 27 blocks of edge 10 in a batch,
+    // 192 directions: 439 us without, now 331)
+    p.smem = std::max(pair_smem_bytes(g.B, p.nstage * dt) + (size_t)hand, ctas > 1 ? 0 : (size_t)pair_smem_limit(2) + 16);
+    return p;
+  };
+  // the smallest CTAs (a warp for every scheduler) of which an SM takes one; else
+  // the largest, as many an SM as its registers hold
+  for (int warps = 2; warps <= 8; ++warps)
+    if (const HalvesPlan p = fit(warps, 1); p.parts) return p;
+  const int parts = (2 * half + 511) / 512, warps = ((half + parts - 1) / parts + 31) / 32;
+  for (int ctas = 1024 / (64 * warps); ctas > 1; --ctas)
+    if (const HalvesPlan p = fit(warps, ctas); p.parts) return p;
+  return {};
+}
+
 template <int MODE, int BC>
 void pair_launch(const GridDims &g, const float *kappa, const float *S, const unsigned char *tpl, const int *order,
                  const float *faces, const float *bnd, float *I_out, float *M_out, float *E_out, float *f_out,
@@ -2125,6 +2274,18 @@ void pair_launch(const GridDims &g, const float *kappa, const float *S, const un
     const bool room = MODE == 1 || (split->part && split->count && q.part_bytes <= split->part_bytes &&
                                     q.slots <= split->slots);
     if (q.k > 1 && room) tp = q;
+  }
+  if constexpr (BC == 0) {
+    const HalvesPlan hp = tp.k > 1 ? HalvesPlan{} : plan_halves(g, nblk, dt);
+    if (hp.parts) {
+      // not a dependent launch: CTAs that start while the face pass still holds
+      // SMs crowd on the others (27 blocks of edge 12, 3072 directions, one thread a
+      // pair: the cell pass alone 6.1 ms, launched as a dependent 7.3)
+      cell_pair_kernel<MODE, BC, false, false, true><<<nblk * hp.parts, hp.threads, hp.smem, st>>>(
+          g, hp.parts, dt, hp.nstage, kappa, S, tpl, order, faces, bnd, I_out, M_out, E_out, f_out, emax_bits, spin, status,
+          block_list, nblk * hp.parts, 1, nullptr, nullptr, nullptr, nullptr);
+      return;
+    }
   }
   const int grid = tp.nfull + (nblk * parts - tp.nfull) * tp.k;
   cudaLaunchConfig_t cfg = {};
@@ -2190,6 +2351,9 @@ cudaError_t set_smem_attrs() {
                         (const void *)cell_pair_kernel<0, 0, false>,  (const void *)cell_pair_kernel<2, 0, false>,
                         (const void *)cell_pair_kernel<1, 0, false>,  (const void *)cell_pair_kernel<0, 0, false, true>,
                         (const void *)cell_pair_kernel<2, 0, false, true>,
+                        (const void *)cell_pair_kernel<0, 0, false, false, true>,
+                        (const void *)cell_pair_kernel<1, 0, false, false, true>,
+                        (const void *)cell_pair_kernel<2, 0, false, false, true>,
                         (const void *)face_pair_kernel<0>,            (const void *)face_pair_kernel<8>,
                         (const void *)face_pair_kernel<16>};
   for (const void *f : pfns) {  // less their static shared memory
