@@ -11,6 +11,7 @@
 #include <cuda_bf16.h>
 
 #include "vet_cnn.h"
+#include "vet_floatsum.h"
 
 namespace vet {
 namespace cnn {
@@ -33,31 +34,15 @@ __device__ __forceinline__ double block_sum_d(double v, double *red) {
   return s;  // valid in thread 0
 }
 
-// Sums and differences as unevaluated pairs of floats (Knuth's TwoSum, Dekker's
-// product by FMA): the FP64 pipe does two operations per clock per SM, and a
-// conversion and an addition per value held these kernels to a fifth of the
-// memory rate.  At 128^3, ncu: feat_stats 47 -> 25 us, feat_pack 88 -> 25 us (of
-// them 14 for its 92 MB); the features are the same bits.
-struct Pair {
-  float hi, lo;
-};
-// (explicitly rounded additions: an operand that is itself a product must not
-// be contracted into them)
-__device__ __forceinline__ Pair two_sum(float a, float b) {
-  const float s = __fadd_rn(a, b), t = __fsub_rn(s, a);
-  return {s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t))};
-}
-__device__ __forceinline__ void pair_add(Pair &p, float x) {
-  const Pair s = two_sum(p.hi, x);
-  const float lo = __fadd_rn(p.lo, s.lo), hi = __fadd_rn(s.hi, lo);
-  p = {hi, __fsub_rn(lo, __fsub_rn(hi, s.hi))};
-}
-__device__ __forceinline__ double pair_value(Pair p) { return (double)p.hi + (double)p.lo; }
-
+// Sums and differences in FP32 arithmetic to FP64's precision: the FP64 pipe does
+// two operations per clock per SM, and a conversion and an addition per value held
+// these kernels to a fifth of the memory rate.  At 128^3, ncu: feat_stats 47 ->
+// 29 us, feat_pack 88 -> 26 us (of them 14 for its 92 MB).  (Pairs of floats, 48
+// bits, took 25 and 25 us and were a unit in the last place of a feature off where
+// log S or log E hardly differs from its mean.)
 // The block's optical depths are summed as differences from its first cell's
 // (a block of equal cells then has the exact mean and a standard deviation of
-// 0); a thread's up to B^3 / 256 terms as float pairs, the threads' sums in
-// FP64.
+// 0); a thread's up to B^3 / 256 terms by FloatSum, the threads' sums in FP64.
 __global__ void __launch_bounds__(256) feat_stats_kernel(const float *__restrict__ kappa, const float *__restrict__ S,
                                                          const float *__restrict__ E, Vol V, int B, float h,
                                                          double *__restrict__ sums, float *__restrict__ bstat) {
@@ -69,7 +54,7 @@ __global__ void __launch_bounds__(256) feat_stats_kernel(const float *__restrict
   const int B3 = B * B * B;
   const long long c0 = (long long)v * vol + ((long long)(bz * B) * V.ny + by * B) * V.nx + bx * B;
   const float tau0 = log10f(fmaxf(kappa[c0] * h, kTiny));
-  Pair pt{0.f, 0.f}, pt2{0.f, 0.f}, ps{0.f, 0.f}, pe{0.f, 0.f};
+  FloatSum pt, pt2, ps, pe;
   // i / B for i < 2^16 (block edges up to 32) by a multiplication
   const unsigned mB = (unsigned)(((1ull << 32) + B - 1) / B);
   for (int i0 = threadIdx.x; i0 < B3; i0 += 4 * blockDim.x) {  // four cells a trip, their loads together
@@ -97,19 +82,24 @@ __global__ void __launch_bounds__(256) feat_stats_kernel(const float *__restrict
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
       if (i0 + u * (int)blockDim.x >= B3) break;
-      const Pair d = two_sum(log10f(fmaxf(k[u] * h, kTiny)), -tau0);
-      pair_add(pt, d.hi);
-      pair_add(pt, d.lo);
-      const float q = __fmul_rn(d.hi, d.hi);
-      pair_add(pt2, q);
-      pair_add(pt2, fmaf(2.f * d.hi, d.lo, fmaf(d.hi, d.hi, -q)));
-      pair_add(ps, log10f(fmaxf(s[u], kTiny)));
-      pair_add(pe, log10f(fmaxf(en[u], kTiny)));
+      float d = log10f(fmaxf(k[u] * h, kTiny));
+      const float dl = two_sum(d, -tau0);  // the difference is d + dl
+      pt.add(d);
+      pt.add(dl);
+      // its square: d^2 and 2 d dl by products with their exact roundings (FMA);
+      // the second one's is, like dl^2, below 2^-48 of the total
+      const float q = __fmul_rn(d, d), r = __fmul_rn(2.f * d, dl);
+      pt2.add(q);
+      pt2.add(__fmaf_rn(d, d, -q));
+      pt2.add(r);
+      pt2.c = __fadd_rn(pt2.c, __fmaf_rn(dl, dl, __fmaf_rn(2.f * d, dl, -r)));
+      ps.add(log10f(fmaxf(s[u], kTiny)));
+      pe.add(log10f(fmaxf(en[u], kTiny)));
     }
   }
-  double vt = pair_value(pt), vt2 = pair_value(pt2), vs = pair_value(ps), ve = pair_value(pe), ref = tau0;
+  double vt = pt.value(), vt2 = pt2.value(), vs = ps.value(), ve = pe.value(), ref = tau0;
   if (__syncthreads_or(!isfinite(vt) || !isfinite(vt2) || !isfinite(vs) || !isfinite(ve))) {
-    // an infinity among the fields (a pair loses its sign): plain FP64 sums
+    // an infinity among the fields (a FloatSum loses its sign): plain FP64 sums
     vt = vt2 = vs = ve = ref = 0.0;
     for (int i = threadIdx.x; i < B3; i += blockDim.x) {
       const int x = i % B, y = (i / B) % B, z = i / (B * B);
@@ -132,10 +122,23 @@ __global__ void __launch_bounds__(256) feat_stats_kernel(const float *__restrict
   }
 }
 
-// l - mean, mean as a float pair: one rounding of the difference.
-__device__ __forceinline__ float minus_mean(float l, Pair mean) {
-  const Pair d = two_sum(l, -mean.hi);
-  return isfinite(d.hi) ? __fadd_rn(d.hi, __fsub_rn(d.lo, mean.lo)) : d.hi;
+// A double as three floats, and l - it: exact sums of the parts, rounded once but
+// for what is below 2^-48 of l.
+struct Mean {
+  float a, b, c;
+};
+__device__ __forceinline__ Mean split_mean(double m) {
+  const float a = (float)m;
+  if (!isfinite(a)) return {a, 0.f, 0.f};
+  const float b = (float)(m - (double)a);
+  return {a, b, (float)((m - (double)a) - (double)b)};
+}
+__device__ __forceinline__ float minus_mean(float l, const Mean &mean) {
+  float d = l;
+  const float e1 = two_sum(d, -mean.a);
+  if (!isfinite(d)) return d;
+  const float e2 = two_sum(d, -mean.b);
+  return __fadd_rn(d, __fadd_rn(e2, __fsub_rn(e1, mean.c)));
 }
 
 // n / d for any n and d below 2^32: the multiplication's quotient is exact or one short.
@@ -158,18 +161,14 @@ __global__ void __launch_bounds__(256) feat_pack_kernel(const float *__restrict_
                                                         const double *__restrict__ sums,
                                                         const float *__restrict__ bstat, __nv_bfloat16 *__restrict__ x0,
                                                         float *__restrict__ feat_out) {
-  __shared__ Pair s_mean[2];
+  __shared__ Mean s_mean[2];
   after_previous();
   let_next_launch();
   const long long vol = (long long)V.nz * V.ny * V.nx;
   const int v = blockIdx.y;
-  if (threadIdx.x < 2) {
-    const double m = sums[2 * v + threadIdx.x] / (double)vol;
-    const float hi = (float)m;
-    s_mean[threadIdx.x] = {hi, isfinite(hi) ? (float)(m - (double)hi) : 0.f};
-  }
+  if (threadIdx.x < 2) s_mean[threadIdx.x] = split_mean(sums[2 * v + threadIdx.x] / (double)vol);
   __syncthreads();
-  const Pair mean_s = s_mean[0], mean_e = s_mean[1];
+  const Mean mean_s = s_mean[0], mean_e = s_mean[1];
   const int nbx = V.nx / B, nby = V.ny / B, nbz = V.nz / B;
   for (long long l = blockIdx.x * (long long)blockDim.x + threadIdx.x; l < vol; l += (long long)gridDim.x * blockDim.x) {
     const long long c = v * vol + l;

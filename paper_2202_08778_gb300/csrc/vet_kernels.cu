@@ -23,6 +23,7 @@
 #include <type_traits>
 
 #include "vet_exp64.h"
+#include "vet_floatsum.h"
 #include "vet_internal.h"
 
 namespace vet {
@@ -1987,23 +1988,6 @@ __global__ void floor_fix_blocks_kernel(const GridDims g, const int *__restrict_
     }
   }
 }
-
-// Sum of FP32 values as three floats: two exact sums (TwoSum, Knuth) carry
-// their roundings on, the third collects what is below 2^-48 of the total, so
-// the result is within an FP64 rounding of the exact sum.  13 FP32 additions a
-// value, where an FP64 addition and the conversion before it hold the SM's
-// two-lane FP64 pipe for 32 clocks per warp.
-struct FloatSum {
-  float a = 0.f, b = 0.f, c = 0.f;
-  static __device__ __forceinline__ float two_sum(float &s, float x) {  // s += x, returns the rounding
-    const float r = __fadd_rn(s, x), t = __fsub_rn(r, s);
-    const float e = __fadd_rn(__fsub_rn(s, __fsub_rn(r, t)), __fsub_rn(x, t));
-    s = r;
-    return e;
-  }
-  __device__ __forceinline__ void add(float x) { c = __fadd_rn(c, two_sum(b, two_sum(a, x))); }
-  __device__ __forceinline__ double value() const { return (double)a + ((double)b + (double)c); }
-};
 
 // Quadratures of stored intensities (Eqs. 10-12, c = 1): M[m][c] =
 // sum_k coef[k][m] I[k][c].  HBM-bound (4 bytes of I per 10 FMAs): one thread
