@@ -38,7 +38,7 @@ __device__ __forceinline__ double block_sum_d(double v, double *red) {
 // two operations per clock per SM, and a conversion and an addition per value held
 // these kernels to a fifth of the memory rate.  At 128^3, ncu: feat_stats 47 ->
 // 29 us, feat_pack 88 -> 26 us (of them 14 for its 92 MB).  (Pairs of floats, 48
-// bits, took 25 and 25 us and were a unit in the last place of a feature off where
+// bits, took 25 and 25 us and left features up to half a unit further off where
 // log S or log E hardly differs from its mean.)
 // The block's optical depths are summed as differences from its first cell's
 // (a block of equal cells then has the exact mean and a standard deviation of
