@@ -91,8 +91,15 @@ typedef struct {
 typedef struct vet_ctx vet_ctx;
 
 /* Create a context: validates grid and config, builds the direction set and
- * the per-direction ray templates, allocates the face-intensity workspace
- * (N x blocks x 3 x about (block+2)^2 values).  *out is NULL on failure. */
+ * the per-direction ray templates and allocates the workspace on the device:
+ *   - face intensities, N x blocks x 3 x about (block+2)^2 values;
+ *   - ray records, N x (4 block^3 + 48 (block+1)^2) bytes;
+ *   - scratch of at most 128 MB where the cell pass is cut into shares of the
+ *     directions to fill the SMs: on FP32 grids that leave SMs idle 4 bytes a
+ *     cell and direction (32^3 cells in 8^3 blocks, 192 directions: 25 MB beside
+ *     15 MB of faces), else partial moments of the last blocks.  It only buys
+ *     time: without room for it the context works unsplit.
+ * *out is NULL on failure. */
 vet_status vet_create(vet_ctx **out, const vet_grid *grid, const vet_config *cfg);
 
 /* Release the context and all its device memory.  NULL is accepted. */

@@ -262,11 +262,19 @@ vet_status build_context(vet_ctx *c) {
   c->dims.fstride = vet::face_stride_elems<R>(B);
   const size_t face_elems = (size_t)N * c->nblk * 3 * c->dims.fstride;
   if ((e = cudaMalloc(&c->d_tpl, tpl.size()))) return cuda_err(c, e, "cudaMalloc(templates)");
-  // faces, then the split's counters and scratch
-  const vet::TailPlan plan = split_plan(c);
-  const size_t face_bytes = round256(sizeof(R) * face_elems), count_bytes = round256(sizeof(int) * plan.slots);
-  if ((e = cudaMalloc(&c->d_faces, face_bytes + count_bytes + plan.part_bytes)))
-    return cuda_err(c, e, "cudaMalloc(face intensities)");
+  // faces, then the split's counters and scratch; where there is room for the faces
+  // alone, the cell pass runs unsplit
+  vet::TailPlan plan = split_plan(c);
+  const size_t face_bytes = round256(sizeof(R) * face_elems);
+  size_t count_bytes = round256(sizeof(int) * plan.slots);
+  e = cudaMalloc(&c->d_faces, face_bytes + count_bytes + plan.part_bytes);
+  if (e == cudaErrorMemoryAllocation && plan.k > 1) {
+    cudaGetLastError();
+    plan = {};
+    count_bytes = 0;
+    e = cudaMalloc(&c->d_faces, face_bytes);
+  }
+  if (e) return cuda_err(c, e, "cudaMalloc(face intensities)");
   // the padding row and column of every stored face stay zero for good
   if ((e = cudaMemset(c->d_faces, 0, face_bytes + count_bytes))) return cuda_err(c, e, "cudaMemset(face intensities)");
   if (plan.k > 1) {
