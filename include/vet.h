@@ -454,9 +454,10 @@ vet_status vet_hlle_wavespeed(const vet_grid *grid, const float *f, const float 
  * outputs; what they cannot provide is the library's workspace.
  *
  * vet_closure_noalloc computes exactly what vet_create + vet_closure (FP32)
- * compute, without a context: every piece of workspace lives in one static
- * device array of VET_NOALLOC_SCRATCH_BYTES compiled into libvet, which every
- * GPU that loads the library holds until the process exits, and the host-side
+ * compute, without a context: the workspace lives in a static device array of
+ * VET_NOALLOC_SCRATCH_BYTES and 5.8 MB of static tables beside it (where each
+ * ray starts, made anew on every call) compiled into libvet, which every GPU
+ * that loads the library holds until the process exits, and the host-side
  * geometry uses fixed static host arrays.  It calls no cudaMalloc, cudaFree or
  * other allocating routine.
  *   - Limits: FP32 only; nside 1, 2 or 4; block edge 2..16; and the problem's

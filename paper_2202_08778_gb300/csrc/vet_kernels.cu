@@ -578,7 +578,6 @@ __global__ void __launch_bounds__(kCellThreads, kCellMinCtas<R>)
   const int B2 = B * B, B3 = B2 * B;
   const TileShape ts = cell_tile(B);
   const TplLayout TL = tpl_layout<R>(B);
-  const int fstride = g.fstride;
   const size_t sb = slot_bytes<R>(B);
   vec2_t<R> *tile = reinterpret_cast<vec2_t<R> *>(smem);
   unsigned char *buf0 = smem + align16(sizeof(vec2_t<R>) * (size_t)ts.elems);
@@ -839,13 +838,6 @@ __device__ __forceinline__ float lds_f32(uint32_t a) {
   asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(a));
   return v;
 }
-__device__ __forceinline__ int lds_s16(uint32_t a) {
-  int v;
-  asm volatile("ld.shared.s16 %0, [%1];" : "=r"(v) : "r"(a));
-  return v;
-}
-
-
 __device__ __forceinline__ float4 lds_f4(uint32_t a) {
   float4 v;
   asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(a));
@@ -975,15 +967,13 @@ __device__ __forceinline__ float march_one(uint32_t t, uint32_t ev, int last, fl
 // Paired-cell-pass slot: the template head, the template's cell-ray parts,
 // then the three incoming faces (offsets in bytes from the slot's start).
 struct CellSlot {
-  int cev, cpos, ck, cw, faces, bytes;
+  int cev, cw, faces, bytes;
 };
 __host__ __device__ inline CellSlot cell_slot(int B) {
   const TplLayout L = tpl_layout<float>(B);
   const int shift = L.cev - L.nev;  // the node-ray parts are not staged
   CellSlot s;
   s.cev = L.cev - shift;
-  s.cpos = L.cpos - shift;
-  s.ck = L.ck - shift;
   s.cw = L.cw - shift;
   s.faces = L.bytes - shift;
   s.bytes = s.faces + (int)faces_bytes<float>(B);

@@ -8,12 +8,13 @@
 // pool.  Such callers own their input and output buffers but cannot give the
 // library a workspace.
 //
-// How: every piece of workspace (direction templates, face-pass schedule,
-// boundary and face intensities, E, the max-E word, the status word) lives in
-// one file-scope device array of VET_NOALLOC_SCRATCH_BYTES that every GPU
-// loading the library holds until the process exits; the host-side geometry
-// is built in fixed static host arrays.  The array's device address is looked
-// up once per device, on the first call made with that device selected.
+// How: the workspace (direction templates, face-pass schedule, boundary and
+// face intensities, E, the max-E word, the status word) lives in one file-scope
+// device array of VET_NOALLOC_SCRATCH_BYTES, the ray records in two more (5.8
+// MB) that are filled anew on every call; every GPU loading the library holds
+// them until the process exits; the host-side geometry is built in fixed static
+// host arrays.  The arrays' device addresses are looked up once per device, on
+// the first call made with that device selected.
 #include <cstring>
 #include <mutex>
 #include <string>
