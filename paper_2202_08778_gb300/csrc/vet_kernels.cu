@@ -718,8 +718,8 @@ __global__ void __launch_bounds__(kCellThreads, kCellMinCtas<R>)
     if (slot >= 0) {
       // one share of a split work item: its sums go to the slot's scratch, and
       // the share that finishes last adds all of them in order (the compensated
-      // sums as compensated sums; the same bits whichever finishes last) and
-      // writes the outputs
+      // sums exactly, their compensations and the additions' roundings beside
+      // them; the same bits whichever finishes last) and writes the outputs
       __shared__ int s_last;
       const int NT = blockDim.x;
       R *mine = split_part + ((size_t)slot * ksplit + share) * 14 * NT + threadIdx.x;
@@ -740,15 +740,19 @@ __global__ void __launch_bounds__(kCellThreads, kCellMinCtas<R>)
           const R v = __ldcg(other + m * NT);
           if (m == 0 || (m >= 4 && m < 7)) {
             const int q = m == 0 ? 0 : m - 3;
-            const R y = v - (cmp[q] + __ldcg(other + (10 + q) * NT));
-            const R tt = mom[m] + y;
-            cmp[q] = (tt - mom[m]) - y;
+            // the larger one first (by exponent and leading bits, integers): the
+            // addition's rounding is then exact in two operations (Dekker)
+            const bool less = (__double2hiint(mom[m]) & 0x7fffffff) < (__double2hiint(v) & 0x7fffffff);
+            const R a = less ? v : mom[m], b = less ? mom[m] : v, tt = a + b;
+            cmp[q] += __ldcg(other + (10 + q) * NT) - (b - (tt - a));
             mom[m] = tt;
           } else if (kWantF || m >= 7) {
             mom[m] += v;
           }
         }
       }
+      mom[0] -= cmp[0];
+      for (int q = 1; q < 4; ++q) mom[3 + q] -= cmp[q];
       if (threadIdx.x == 0) split_count[slot] = 0;  // ready for the next call
     }
   }
