@@ -77,3 +77,21 @@ def test_no_slower_than_a_ray_a_thread(B, blocks):
     paired = _time(lambda: batch.closure([k], [S], None, [f]))
     single = _time(lambda: vet.closure_noalloc(shape, B, p["h"], 4, k, S, None, f, rot_q=p["q"]))
     assert paired < single, (paired, single)
+
+
+def test_hand_over_that_gives_up_is_reported():
+    """One poll a wait: the launch ends, the call reports the timeout, and a patient batch still gives its bits."""
+    B, nside = 12, 4
+    shape = (3 * B, 3 * B, 3 * B)
+    p, k, S = _fields(shape, B, nside, 8)
+    f, f2, lost = (torch.empty(6, k.numel(), device="cuda") for _ in range(3))
+    patient, impatient = (vet.Batch([(shape, B, p["h"], nside, p["q"])], spin_limit=s) for s in (0, 1))
+    patient.closure([k], [S], None, [f])
+    patient.sync()
+    impatient.closure([k], [S], None, [lost])
+    with pytest.raises(vet.VetError) as err:
+        impatient.sync()
+    assert err.value.status == vet.VET_ETIMEOUT
+    patient.closure([k], [S], None, [f2])
+    patient.sync()
+    assert torch.equal(f, f2)
