@@ -125,8 +125,8 @@ vet_status vet_trace(vet_ctx *ctx, const float *kappa, const float *S, const flo
  * VET_EINVAL if E64_out is not device memory. */
 vet_status vet_moments(vet_ctx *ctx, const float *I, float *M_out, double *E64_out, void *stream);
 
-/* Whole closure, fused: trace + quadratures + f = P/E (Eq. 13) without
- * storing I.  f_out[6][cells] required; M_out[10][cells] optional (NULL).
+/* Whole closure, fused: trace + quadratures + f = P/E (Eq. 13) without an
+ * output of I.  f_out[6][cells] required; M_out[10][cells] optional (NULL).
  * FP32 context only. */
 vet_status vet_closure(vet_ctx *ctx, const float *kappa, const float *S, const float *Ib, float *f_out,
                        float *M_out, void *stream);
