@@ -37,16 +37,16 @@ __device__ __forceinline__ double block_sum_d(double v, double *red) {
 // Sums and differences in FP32 arithmetic to FP64's precision: the FP64 pipe does
 // two operations per clock per SM, and a conversion and an addition per value held
 // these kernels to a fifth of the memory rate.  At 128^3, ncu: feat_stats 47 ->
-// 29 us, feat_pack 88 -> 26 us (of them 14 for its 92 MB).  (Pairs of floats, 48
-// bits, took 25 and 25 us and left features up to half a unit further off where
-// log S or log E hardly differs from its mean.)
+// 24 us, feat_pack 88 -> 20 us (of them 14 for its 92 MB).  (Pairs of floats, 48
+// bits, left features up to half a unit further off where log S or log E hardly
+// differs from its mean.)
 // The block's optical depths are summed as differences from its first cell's
 // (a block of equal cells then has the exact mean and a standard deviation of
 // 0); a thread's up to B^3 / 256 terms by FloatSum, the threads' sums in FP64.
 __global__ void __launch_bounds__(256) feat_stats_kernel(const float *__restrict__ kappa, const float *__restrict__ S,
                                                          const float *__restrict__ E, Vol V, int B, float h,
                                                          double *__restrict__ sums, float *__restrict__ bstat) {
-  __shared__ double red[8];
+  __shared__ double red[8][4];
   const int nbx = V.nx / B, nby = V.ny / B, nbz = V.nz / B;
   const int blk = blockIdx.x, v = blockIdx.y;
   const int bx = blk % nbx, by = (blk / nbx) % nby, bz = blk / (nbx * nby);
@@ -84,15 +84,12 @@ __global__ void __launch_bounds__(256) feat_stats_kernel(const float *__restrict
       if (i0 + u * (int)blockDim.x >= B3) break;
       float d = log10f(fmaxf(k[u] * h, kTiny));
       const float dl = two_sum(d, -tau0);  // the difference is d + dl
-      pt.add(d);
-      pt.add(dl);
+      pt.add(d, dl);
       // its square: d^2 and 2 d dl by products with their exact roundings (FMA);
       // the second one's is, like dl^2, below 2^-48 of the total
       const float q = __fmul_rn(d, d), r = __fmul_rn(2.f * d, dl);
-      pt2.add(q);
-      pt2.add(__fmaf_rn(d, d, -q));
-      pt2.add(r);
-      pt2.c = __fadd_rn(pt2.c, __fmaf_rn(dl, dl, __fmaf_rn(2.f * d, dl, -r)));
+      pt2.add(q, __fmaf_rn(d, d, -q));
+      pt2.c = __fadd_rn(pt2.c, __fadd_rn(two_sum(pt2.b, r), __fmaf_rn(dl, dl, __fmaf_rn(2.f * d, dl, -r))));
       ps.add(log10f(fmaxf(s[u], kTiny)));
       pe.add(log10f(fmaxf(en[u], kTiny)));
     }
@@ -111,15 +108,28 @@ __global__ void __launch_bounds__(256) feat_stats_kernel(const float *__restrict
       ve += log10f(fmaxf(E[c], kTiny));
     }
   }
-  const double st = block_sum_d(vt, red), st2 = block_sum_d(vt2, red);
-  const double ss = block_sum_d(vs, red), se = block_sum_d(ve, red);
+  // the warp's four sums in six FP64 additions a lane, each exchange halving what a
+  // lane carries; then the warps' by four threads
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const bool up = lane & 16, mid = lane & 8;
+  double v0 = up ? vs : vt, v1 = up ? ve : vt2;
+  v0 += __shfl_xor_sync(0xffffffffu, up ? vt : vs, 16);
+  v1 += __shfl_xor_sync(0xffffffffu, up ? vt2 : ve, 16);
+  double w = (mid ? v1 : v0) + __shfl_xor_sync(0xffffffffu, mid ? v0 : v1, 8);
+  for (int o = 4; o > 0; o >>= 1) w += __shfl_xor_sync(0xffffffffu, w, o);
+  if ((lane & 7) == 0) red[warp][lane >> 3] = w;
+  __syncthreads();
+  if (threadIdx.x >= 32) return;
+  double sum = 0.0;
+  if (threadIdx.x < 4)
+    for (int q = 0; q < 8; ++q) sum += red[q][threadIdx.x];
+  const double st2 = __shfl_sync(0xffffffffu, sum, 1);
   if (threadIdx.x == 0) {
-    const double mean = st / B3, var = fmax(st2 / B3 - mean * mean, 0.0);
+    const double mean = sum / B3, var = fmax(st2 / B3 - mean * mean, 0.0);
     bstat[((long long)v * nbx * nby * nbz + blk) * 2] = (float)(ref + mean);
     bstat[((long long)v * nbx * nby * nbz + blk) * 2 + 1] = (float)sqrt(var);
-    atomicAdd(sums + 2 * v, ss);
-    atomicAdd(sums + 2 * v + 1, se);
   }
+  if (threadIdx.x == 2 || threadIdx.x == 3) atomicAdd(sums + 2 * v + threadIdx.x - 2, sum);
 }
 
 // A double as three floats, and l - it: exact sums of the parts, rounded once but
@@ -136,9 +146,9 @@ __device__ __forceinline__ Mean split_mean(double m) {
 __device__ __forceinline__ float minus_mean(float l, const Mean &mean) {
   float d = l;
   const float e1 = two_sum(d, -mean.a);
-  if (!isfinite(d)) return d;
-  const float e2 = two_sum(d, -mean.b);
-  return __fadd_rn(d, __fadd_rn(e2, __fsub_rn(e1, mean.c)));
+  const float first = d;
+  const float e2 = two_sum(d, -mean.b), r = __fadd_rn(d, __fadd_rn(e2, __fsub_rn(e1, mean.c)));
+  return isfinite(first) ? r : first;  // a select: a return in between took 6 us of 47
 }
 
 // n / d for any n and d below 2^32: the multiplication's quotient is exact or one short.

@@ -24,6 +24,11 @@ __device__ __forceinline__ float two_sum(float &s, float x) {
 struct FloatSum {
   float a = 0.f, b = 0.f, c = 0.f;
   __device__ __forceinline__ void add(float x) { c = __fadd_rn(c, two_sum(b, two_sum(a, x))); }
+  // x + y, |y| below 2^-23 |x|
+  __device__ __forceinline__ void add(float x, float y) {
+    const float e = two_sum(b, two_sum(a, x));
+    c = __fadd_rn(c, __fadd_rn(e, two_sum(b, y)));
+  }
   __device__ __forceinline__ double value() const { return (double)a + ((double)b + (double)c); }
 };
 
