@@ -559,7 +559,7 @@ vet_status do_moments(vet_ctx *c, const R *I, R *M_out, void *stream, bool fp64,
   bool had_host = false;
   s = stage_args<R>(c, st, {{I, (size_t)c->N * nc}}, {{M_out, 10 * nc}}, din, dout, back, bytes, had_host);
   if (s) return s;
-  cudaError_t e = vet::launch_moments<R>(c->dims.ncell, c->N, din[0], (const R *)c->d_coef, dout[0], st, E64_out,
+  cudaError_t e = vet::launch_moments<R>(c->dims.ncell, c->N, din[0], (const R *)c->d_coef, dout[0], c->dims.nsm, st, E64_out,
                                          c->dirs_ext[3]);
   if (e) return cuda_err(c, e, "moments launch");
   c->last_stream = st;

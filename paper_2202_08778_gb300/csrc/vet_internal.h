@@ -319,7 +319,7 @@ cudaError_t launch_floor_fix(long long ncell, const R *E, const void *emax_bits,
 // E64 (optional, device): E of every cell summed in FP64, w64 times the sum
 // of I over the directions (the weights are all equal to w64).
 template <typename R>
-cudaError_t launch_moments(long long ncell, int ndir, const R *I, const R *coef, R *M_out,
+cudaError_t launch_moments(long long ncell, int ndir, const R *I, const R *coef, R *M_out, int nsm,
                            cudaStream_t st, double *E64 = nullptr, double w64 = 0.0);
 
 // Dynamic shared memory of an unpaired face-pass CTA staging `dirs` directions.

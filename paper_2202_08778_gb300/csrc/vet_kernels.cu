@@ -1987,7 +1987,7 @@ __global__ void floor_fix_blocks_kernel(const GridDims g, const int *__restrict_
 // sum_k coef[k][m] I[k][c].  HBM-bound (4 bytes of I per 10 FMAs): one thread
 // per V consecutive cells with V-wide loads, directions unrolled by 4 so that
 // several loads are in flight, coefficients of a chunk of 64 directions in
-// shared memory.  With E64 the sum of I goes through FloatSum and V is 2 (96 x
+// shared memory.  With E64 the sum of I goes through FloatSum and V is at most 2 (96 x
 // 64 x 48 cells, 192 directions, L2 flushed: 234 -> 72 us against FP64 additions of
 // every value; without E64 79 -> 58 us by two cells a thread).
 template <typename R, int V, bool WITH_E64>
@@ -2493,18 +2493,31 @@ cudaError_t launch_floor_fix_blocks(const GridDims &g, const int *block_list, in
 }
 
 template <typename R>
-cudaError_t launch_moments(long long ncell, int ndir, const R *I, const R *coef, R *M_out, cudaStream_t st,
+cudaError_t launch_moments(long long ncell, int ndir, const R *I, const R *coef, R *M_out, int nsm, cudaStream_t st,
                            double *E64, double w64) {
   const int threads = 256;
   // vector loads need every direction's row to start aligned to them
   auto fits = [&](int v) {
     return ncell % v == 0 && ((reinterpret_cast<uintptr_t>(I) | reinterpret_cast<uintptr_t>(M_out)) & (v * sizeof(R) - 1)) == 0;
   };
-  // four FP32 cells a thread where that still gives the SMs enough loads in
-  // flight (threads of 152 SMs x 1024), else two; two with E64 (registers)
+  // FP32 cells a thread (four not with E64: registers) by the rounds of four CTAs
+  // an SM that they take, a round of two and of four cells at 1.25 and 2.2 times
+  // one of one cell.  192 directions, us with 1, 2 and 4 cells: 32768 cells 16, 18, 29;
+  // 196608 68, 43, 66; 294912 75, 49, 68; 460800 112, 87, 78; 884736 213, 133, 148;
+  // 1179648 283, 178, 165.  The sums' order, and so their bits, is the same.
   int v = 1;
-  if (sizeof(R) == 4 && !E64 && fits(4) && ncell >= 4LL * 152 * 1024) v = 4;
-  else if (fits(2)) v = 2;
+  if (sizeof(R) == 4) {
+    double best = 0.0;
+    for (int w : {1, 2, 4}) {
+      const long long round = 4LL * std::max(1, nsm) * threads * w;
+      const double cost = (double)((ncell + round - 1) / round) * (w == 1 ? 1.0 : w == 2 ? 1.25 : 2.2);
+      if (w > 1 && (!fits(w) || (E64 && w == 4) || cost >= best)) continue;
+      v = w;
+      best = cost;
+    }
+  } else if (fits(2)) {
+    v = 2;
+  }
   const long long blocks = ((ncell + v - 1) / v + threads - 1) / threads;
   if (blocks < 1) return cudaSuccess;
 #define VET_MOM(V, WE) moments_kernel<R, V, WE><<<(unsigned)blocks, threads, 0, st>>>(ncell, ndir, I, coef, M_out, E64, w64)
@@ -2566,7 +2579,7 @@ cudaError_t prepare_kernels() {
   template cudaError_t launch_fill_boundary<R>(const GridDims &, const unsigned char *, const R *, R *, void *, \
                                                cudaStream_t);                                                \
   template cudaError_t launch_floor_fix<R>(long long, const R *, const void *, double, R *, cudaStream_t, bool); \
-  template cudaError_t launch_moments<R>(long long, int, const R *, const R *, R *, cudaStream_t, double *, double);
+  template cudaError_t launch_moments<R>(long long, int, const R *, const R *, R *, int, cudaStream_t, double *, double);
 
 VET_INSTANTIATE(float)
 VET_INSTANTIATE(double)
