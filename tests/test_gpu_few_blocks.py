@@ -95,3 +95,32 @@ def test_hand_over_that_gives_up_is_reported():
     patient.closure([k], [S], None, [f2])
     patient.sync()
     assert torch.equal(f, f2)
+
+
+@pytest.mark.parametrize("B", [6, 10, 12])
+def test_listed_blocks_give_the_bits_of_the_whole_grid(B):
+    """The learned closure's fallback on a few blocks (two threads a pair) against the plain closure of a
+    grid that fills the SMs once (one)."""
+    side = {6: 8, 10: 6, 12: 5}[B]
+    shape = (side * B,) * 3
+    p, k, S = _fields(shape, B, 2, 70 + B)
+    n = k.numel()
+    ctx = vet.Context(shape, B, p["h"], 2, p["q"])
+    rng = np.random.default_rng(B)
+    model = vet.Model()
+    model.set_params([(rng.uniform(-0.05, 0.05, (27, co, ci)), np.zeros(co)) for ci, co in vet.layer_shapes()])
+    E = torch.rand(n, device="cuda") + 0.5
+    f, plain, r = torch.empty(6, n, device="cuda"), torch.empty(6, n, device="cuda"), torch.empty(n, device="cuda")
+    flags = torch.empty(side ** 3, dtype=torch.int32, device="cuda")
+    model.closure(ctx, k, S, E, f, threshold=float("inf"))
+    model.last_indicator(r, n)
+    at = torch.arange(n, device="cuda")
+    x, y, z = at % shape[2], at // shape[2] % shape[1], at // (shape[1] * shape[2])
+    block = (z // B * side + y // B) * side + x // B
+    worst = torch.zeros(side ** 3, device="cuda").scatter_reduce(0, block, r, "amax").sort(descending=True).values
+    kept = model.closure(ctx, k, S, E, f, threshold=float(worst[5]), block_flags=flags)
+    ctx.closure(k, S, None, plain)
+    ctx.sync()
+    listed = flags.bool()[block]
+    assert 0 < kept <= 5 and int(flags.bool().sum()) == kept
+    assert torch.equal(f[:, listed], plain[:, listed]) and not torch.equal(f[:, ~listed], plain[:, ~listed])
